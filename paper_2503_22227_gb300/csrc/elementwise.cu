@@ -85,72 +85,20 @@ int launch_tensor(const Context &c, const TensorArgs &a, uint32_t count, cudaStr
 // ------------------------------------------------------------------ key-switch inner product
 
 // y_p[i] = sum_j c_j[i] * key_j[p][i] (+ P * add_p[i] on ciphertext primes).
-// The batch item is the fastest-varying block index, so the CTAs of all
-// ciphertexts that read one block of the evaluation key are dispatched back
-// to back: the key crosses HBM once per batch and is served from L2 after.
-//
-// Every load of a thread is issued before its first multiply (BETA is the
-// exact digit count for the common small cases), so a warp keeps 2 + 3 BETA
-// 16-byte loads in flight instead of stalling on each digit in turn.
-template <int BETA>
-__device__ __forceinline__ void ip_body(const IpArgs &A, const DevMod &m, uint32_t item,
-                                        uint32_t i, size_t n, size_t x, uint32_t beta) {
-    const uint32_t KL = A.L + A.K;
-    const bool own_here = A.own != nullptr && i < A.level;
-    const uint32_t own_digit = own_here ? i / A.alpha : 0xffffffffu;
-    const uint64_t *ext = A.ext + item * A.ext_item;
-    const bool fold = i < A.level && A.pfac[i] != 0;
-    ulonglong2 d0 = make_ulonglong2(0, 0), d1 = make_ulonglong2(0, 0);
-    if (fold && A.add0) d0 = ld2(A.add0 + item * A.add_item + size_t(i) * n + x);
-    if (fold && A.add1) d1 = ld2(A.add1 + item * A.add_item + size_t(i) * n + x);
-    ulonglong2 c[BETA], kb[BETA], ka[BETA];
-#pragma unroll
-    for (int j = 0; j < BETA; j++) {
-        if (uint32_t(j) < beta) {
-            c[j] = (uint32_t(j) == own_digit) ? ld2(A.own + item * A.own_item + size_t(i) * n + x)
-                                              : ld2(ext + (size_t(j) * A.M + i) * n + x);
-            kb[j] = ld2(A.key + ((size_t(j) * 2 + 0) * KL + A.key_limb[i]) * n + x);
-            ka[j] = ld2(A.key + ((size_t(j) * 2 + 1) * KL + A.key_limb[i]) * n + x);
-        }
-    }
-    // keys (and P) are in Montgomery form: one reduction per sum
-    U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
-    if (fold) {
-        const uint64_t pf = A.pfac[i];
-        mac(a0, d0.x, pf);
-        mac(a1, d0.y, pf);
-        mac(b0, d1.x, pf);
-        mac(b1, d1.y, pf);
-    }
-#pragma unroll
-    for (int j = 0; j < BETA; j++) {
-        if (uint32_t(j) < beta) {
-            mac(a0, c[j].x, kb[j].x);
-            mac(a1, c[j].y, kb[j].y);
-            mac(b0, c[j].x, ka[j].x);
-            mac(b1, c[j].y, ka[j].y);
-        }
-    }
-    uint64_t *y = A.y + item * A.y_item;
-    st2(y + size_t(i) * n + x, csub(redc(a0, m.q, m.qinv), m.q), csub(redc(a1, m.q, m.qinv), m.q));
-    st2(y + (size_t(A.M) + i) * n + x, csub(redc(b0, m.q, m.qinv), m.q),
-        csub(redc(b1, m.q, m.qinv), m.q));
-}
 
-template <int BETA>
-__global__ void __launch_bounds__(256)
-k_ip(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
-    grid_dep_wait();
-    const size_t n = size_t(1) << log_n;
-    const uint32_t item = blockIdx.x, i = blockIdx.z;
-    const size_t x = 2 * (size_t(blockIdx.y) * blockDim.x + threadIdx.x);
-    if (x >= n) return;
-    const DevMod m = mods[A.prime[i]];
-    ip_body<BETA>(A, m, item, i, n, x, A.beta);
+// The first limb of an item's own digits and of its addends.
+__device__ __forceinline__ const uint64_t *ip_own(const IpArgs &A, uint32_t item, size_t n) {
+    return A.gathered ? A.ga[item] + size_t(A.level) * n : A.own + item * A.own_item;
+}
+__device__ __forceinline__ const uint64_t *ip_add0(const IpArgs &A, uint32_t item) {
+    return A.gathered ? A.ga[item] : A.add0 + item * A.add_item;
 }
 
 // Many digits (beta > 8): digit by digit, loads interleaved with products,
-// so registers stay bounded.
+// so registers stay bounded.  The batch item is the fastest-varying block
+// index, so the CTAs of all ciphertexts that read one block of the
+// evaluation key are dispatched back to back: the key crosses HBM once per
+// batch and is served from L2 after.
 __global__ void __launch_bounds__(256)
 k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     grid_dep_wait();
@@ -166,7 +114,7 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
     if (i < A.level && A.pfac[i] != 0) {
         if (A.add0) {
-            const ulonglong2 d = ld2(A.add0 + item * A.add_item + size_t(i) * n + x);
+            const ulonglong2 d = ld2(ip_add0(A, item) + size_t(i) * n + x);
             mac(a0, d.x, A.pfac[i]);
             mac(a1, d.y, A.pfac[i]);
         }
@@ -177,7 +125,7 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
         }
     }
     for (uint32_t j = 0; j < A.beta; j++) {
-        const ulonglong2 c = (j == own_digit) ? ld2(A.own + item * A.own_item + size_t(i) * n + x)
+        const ulonglong2 c = (j == own_digit) ? ld2(ip_own(A, item, n) + size_t(i) * n + x)
                                               : ld2(ext + (size_t(j) * A.M + i) * n + x);
         const ulonglong2 kb = ld2(A.key + ((size_t(j) * 2 + 0) * KL + A.key_limb[i]) * n + x);
         const ulonglong2 ka = ld2(A.key + ((size_t(j) * 2 + 1) * KL + A.key_limb[i]) * n + x);
@@ -198,8 +146,8 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
 // memory) and streams each ciphertext's digit (and fold) tiles through two
 // shared buffers, the next ciphertext's copies in flight while the threads
 // compute on the current one; all threads then read shared memory only.
-// Used when every address is 16-byte aligned (bulk-copy rule) and
-// BETA <= 8; same arithmetic as k_ip, bit for bit.  Tiles of 512
+// Used for BETA <= 8; every address is 16-byte aligned (the bulk-copy rule),
+// which the host checks.  Tiles of 512
 // coefficients (256 threads) up to 4 digits; 256 coefficients (128 threads)
 // for 5 to 8 digits, so that the 2 BETA key tiles and the two buffers
 // (72 KB at BETA = 8) leave room for 3 CTAs per SM.
@@ -241,11 +189,11 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
         mbar_expect_tx(&bars[b], item_bytes);
         const uint64_t *ext = A.ext + item * A.ext_item;
         for (uint32_t j = 0; j < beta; j++) {
-            const uint64_t *src = (j == own_digit) ? A.own + item * A.own_item + size_t(i) * n
+            const uint64_t *src = (j == own_digit) ? ip_own(A, item, n) + size_t(i) * n
                                                    : ext + (size_t(j) * A.M + i) * n;
             bulk_load(dst + j * kIpTile, src + x0, TB, &bars[b]);
         }
-        if (f0) bulk_load(dst + BETA * kIpTile, A.add0 + item * A.add_item + size_t(i) * n + x0, TB, &bars[b]);
+        if (f0) bulk_load(dst + BETA * kIpTile, ip_add0(A, item) + size_t(i) * n + x0, TB, &bars[b]);
         if (f1) bulk_load(dst + (BETA + 1) * kIpTile, A.add1 + item * A.add_item + size_t(i) * n + x0, TB, &bars[b]);
     };
 
@@ -337,8 +285,6 @@ int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s) {
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-static int launch_ip_regs(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s);
-
 // Ciphertext groups of a bulk inner-product launch: 1 to 4, whichever fills
 // the waves of CTAs best (resident CTAs per SM from the occupancy API), with
 // the groups' uneven sizes counted, and only if that beats one group by 10%
@@ -368,13 +314,14 @@ static unsigned ip_groups(K kernel, unsigned threads, size_t smem, size_t ctas, 
 
 int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
     const size_t n = c.n;
-    bool bulk = a.beta <= 8 && a.status != nullptr && n % 512 == 0 && aligned16(a.ext) &&
-                aligned16(a.key) && aligned16(a.y) && (!a.own || aligned16(a.own)) &&
-                (!a.add0 || aligned16(a.add0)) && (!a.add1 || aligned16(a.add1)) &&
-                (a.ext_item * 8) % 16 == 0 && (a.own_item * 8) % 16 == 0 &&
-                (a.add_item * 8) % 16 == 0 && (a.y_item * 8) % 16 == 0;
-    if (bulk) {
-        switch (a.beta) {
+    // bulk copies: every buffer is a workspace, a key or a ciphertext, refused
+    // at the entry points unless 16-byte aligned
+    bool aligned = a.status != nullptr && aligned16(a.ext) && aligned16(a.key) && aligned16(a.y) &&
+                   aligned16(a.own) && aligned16(a.add0) && aligned16(a.add1) &&
+                   ((a.ext_item | a.own_item | a.add_item | a.y_item) & 1) == 0;
+    for (uint32_t k = 0; a.gathered && k < count; k++) aligned = aligned && aligned16(a.ga[k]);
+    if (!aligned) return CATFHE_EINVAL;
+    switch (a.beta) {
 #define IPB(B)                                                                                   \
     case B: {                                                                                    \
         constexpr uint32_t tile = IpTile<B>::value;                                              \
@@ -387,34 +334,20 @@ int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s)
                    a, c.d_mods, c.log_n, count);                                                 \
         break;                                                                                   \
     }
-            IPB(1) IPB(2) IPB(3) IPB(4) IPB(5) IPB(6) IPB(7) IPB(8)
+        IPB(1) IPB(2) IPB(3) IPB(4) IPB(5) IPB(6) IPB(7) IPB(8)
 #undef IPB
-            default: bulk = false;
-        }
-        if (bulk) return ok();
-    }
-    return launch_ip_regs(c, a, count, s);
-}
-
-static int launch_ip_regs(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
-    const dim3 g(count, unsigned((c.n / 2 + 255) / 256), a.M);
-    switch (a.beta) {
-        case 1: launch_pdl(k_ip<1>, g, dim3(256), 0, s, a, c.d_mods, c.log_n); break;
-        case 2: launch_pdl(k_ip<2>, g, dim3(256), 0, s, a, c.d_mods, c.log_n); break;
-        case 3: launch_pdl(k_ip<3>, g, dim3(256), 0, s, a, c.d_mods, c.log_n); break;
-        case 4: launch_pdl(k_ip<4>, g, dim3(256), 0, s, a, c.d_mods, c.log_n); break;
         default:
-            if (a.beta <= 8)
-                launch_pdl(k_ip<8>, g, dim3(256), 0, s, a, c.d_mods, c.log_n);
-            else
-                launch_pdl(k_ip_stream, g, dim3(256), 0, s, a, c.d_mods, c.log_n);
+            launch_pdl(k_ip_stream, dim3(count, unsigned((n / 2 + 255) / 256), a.M), dim3(256), 0, s,
+                       a, c.d_mods, c.log_n);
     }
     return ok();
 }
 
 // ------------------------------------------------------------------ ModDown combine
 
-// out_p[i] = (y_p[i] - lift_p[i]) * D^-1 (+ add_p[i]).
+// out_p[i] = (y_p[i] - lift_p[i]) * D^-1 (+ add_p[i]), coefficient form; with
+// a Galois element g the coefficient at x goes to x g mod 2N, negated past N
+// (one scattered store per word instead of permuted copies of the inputs).
 __global__ void __launch_bounds__(256)
 k_combine(const CombineArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     const size_t n = size_t(1) << log_n;
@@ -425,8 +358,15 @@ k_combine(const CombineArgs A, const DevMod *__restrict__ mods, uint32_t log_n) 
     const uint64_t y = A.y[item * A.y_item + p * A.y_poly + size_t(i) * n + x];
     const uint64_t l = A.lift[item * A.lift_item + p * A.lift_poly + size_t(i) * n + x];
     uint64_t r = shoup(y + q - l, A.dinv[i], A.dinv_s[i], q);
-    if (A.add) r = add_mod(r, A.add[item * A.add_item + p * A.add_poly + size_t(i) * n + x], q);
-    A.out[item * A.out_item + p * A.out_poly + size_t(i) * n + x] = r;
+    if (A.add && p < A.add_polys)
+        r = add_mod(r, A.add[item * A.add_item + p * A.add_poly + size_t(i) * n + x], q);
+    size_t to = x;
+    if (A.galois) {
+        const uint32_t k = (uint32_t(x) * A.galois) & uint32_t(2 * n - 1);
+        to = k & (n - 1);
+        if (k >= n && r) r = q - r;
+    }
+    A.out[item * A.out_item + p * A.out_poly + size_t(i) * n + to] = r;
 }
 
 int launch_combine(const Context &c, const CombineArgs &a, uint32_t count, cudaStream_t s) {
@@ -460,30 +400,6 @@ int launch_automorph_ntt(const Context &c, const uint64_t *in, uint64_t *out, ui
     return ok();
 }
 
-__global__ void __launch_bounds__(256)
-k_automorph_ntt_map(const uint64_t *__restrict__ in, uint64_t *__restrict__ out, const LimbMap map,
-                    uint64_t g, uint32_t log_n) {
-    grid_dep_wait();
-    const size_t n = size_t(1) << log_n;
-    const size_t k = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const uint32_t limb = blockIdx.y, grp = limb / map.period, r = limb % map.period;
-    const uint64_t *src = in + (size_t(grp) * map.src_stride + map.src_off[r]) * n;
-    uint64_t *dst = out + (size_t(grp) * map.dst_stride + map.dst_off[r]) * n;
-    const uint64_t mask2n = 2 * n - 1;
-    const uint32_t i = __brev(uint32_t(k)) >> (32 - log_n);
-    const uint64_t e = ((2 * uint64_t(i) + 1) * g) & mask2n;
-    dst[k] = src[__brev(uint32_t((e - 1) >> 1)) >> (32 - log_n)];
-}
-
-int launch_automorph_ntt_map(const Context &c, const uint64_t *in, uint64_t *out,
-                             const LimbMap &map, uint32_t limbs_total, uint64_t g, cudaStream_t s) {
-    if (limbs_total == 0) return CATFHE_OK;
-    launch_pdl(k_automorph_ntt_map, coeff_grid(c.n, limbs_total), dim3(256), 0, s, in, out, map,
-               uint64_t(g % (2 * c.n)), uint32_t(c.log_n));
-    return ok();
-}
-
 // ------------------------------------------------------------------ plaintext product
 
 __global__ void __launch_bounds__(256)
@@ -502,41 +418,6 @@ int launch_mul_plain(const Context &c, const uint64_t *a, const uint64_t *pt, ui
                      uint32_t level, uint32_t n_limbs, cudaStream_t s) {
     if (n_limbs == 0) return CATFHE_OK;
     k_mul_plain<<<coeff_grid(c.n / 2, n_limbs), 256, 0, s>>>(a, pt, out, level, c.d_mods, c.log_n);
-    return ok();
-}
-
-// Coefficient form: out[k] = +in[i] if i g = k (mod 2N), -in[i] if i g = k + N.
-__global__ void __launch_bounds__(256)
-k_automorph_coeff(const uint64_t *__restrict__ in, uint64_t *__restrict__ out, const LimbMap map,
-                  const DevMod *__restrict__ mods, uint64_t ginv, uint32_t log_n) {
-    const size_t n = size_t(1) << log_n;
-    const size_t k = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const uint32_t limb = blockIdx.y, g = limb / map.period, r = limb % map.period;
-    const uint64_t *src = in + (size_t(g) * map.src_stride + map.src_off[r]) * n;
-    uint64_t *dst = out + (size_t(g) * map.dst_stride + map.dst_off[r]) * n;
-    const uint64_t q = mods[map.prime[r]].q;
-    const uint64_t i1 = (uint64_t(k) * ginv) & (2 * n - 1);
-    if (i1 < n) {
-        dst[k] = src[i1];
-    } else {
-        const uint64_t v = src[i1 - n];
-        dst[k] = v ? q - v : 0;
-    }
-}
-
-static uint64_t inv_mod_pow2(uint64_t g, uint64_t two_n) {
-    // g odd: Newton iteration for the inverse modulo a power of two
-    uint64_t x = g;
-    for (int i = 0; i < 6; i++) x *= 2 - g * x;
-    return x & (two_n - 1);
-}
-
-int launch_automorph_coeff(const Context &c, const uint64_t *in, uint64_t *out,
-                           const LimbMap &map, uint32_t n_limbs, uint64_t g, cudaStream_t s) {
-    const uint64_t ginv = inv_mod_pow2(g % (2 * c.n), 2 * c.n);
-    k_automorph_coeff<<<coeff_grid(c.n, n_limbs), 256, 0, s>>>(in, out, map, c.d_mods, ginv,
-                                                               c.log_n);
     return ok();
 }
 

@@ -43,6 +43,10 @@ struct LimbMap {
     uint16_t src_off[kMapMax];
     uint16_t dst_off[kMapMax];
     uint8_t prime[kMapMax];
+    // inverse transform only: nonzero when group g's sources lie at gsrc[g]
+    // (gathered ciphertexts) instead of src + g * src_stride limbs
+    uint32_t gathered;
+    const uint64_t *gsrc[kGatherMax];
 };
 
 // Constants of one exact, centred base conversion from k source moduli to T
@@ -161,7 +165,10 @@ struct Keys {
     uint64_t *s_ntt = nullptr;                 // [L+K][N] NTT form
     uint64_t *pk = nullptr;                    // [2][L][N] NTT form
     // id -> [beta][2][L+K][N], NTT form and Montgomery form (times 2^64 mod
-    // the limb's prime), so the inner product needs one reduction per sum
+    // the limb's prime), so the inner product needs one reduction per sum.
+    // The key of a Galois element g is stored with its slots permuted by
+    // sigma_g^-1: key switching then runs on the unrotated ciphertext, and
+    // sigma_g is applied once, to the result, by the kernel that writes it
     std::map<uint64_t, uint64_t *> ksk;
 };
 
@@ -180,17 +187,20 @@ int launch_ntt_inv(const Context &c, const uint64_t *src, uint64_t *dst, const L
                    uint32_t n_limbs, cudaStream_t s);
 
 // Forward NTT whose last pass also finishes the ModDown: for map entry r of
-// group g it writes out = (y - NTT(lift)) * dinv[r] (+ add) instead of the
+// group g it writes out = (y - NTT(lift)) * dinv[r] instead of the
 // transform (the lift itself is left in its column-pass state).
 struct NttEpilogue {
-    const uint64_t *y, *add;
+    const uint64_t *y;
     uint64_t *out;
-    uint32_t y_stride, add_stride, out_stride;  // per group, in limbs
-    uint16_t y_off[kMapMax], add_off[kMapMax], out_off[kMapMax];
+    uint32_t y_stride, out_stride;              // per group, in limbs
+    uint16_t y_off[kMapMax], out_off[kMapMax];
     uint64_t dinv[kMapMax], dinv_s[kMapMax];
     uint32_t gathered;                          // nonzero: group g writes gout[g]
     uint64_t *gout[kGatherMax];
     int *status;                                // the context's status word (bulk-copy wait)
+    // sigma_g applied to the result as it is written: g and its inverse mod
+    // 2N (both 0: no permutation)
+    uint32_t galois, galois_inv;
 };
 // Bit-packed transfer form (pack.cu): words per polynomial at `level`, and
 // the device unpack / pack of `polys` polynomials.
@@ -269,6 +279,11 @@ struct IpArgs {
     uint16_t key_limb[kMapMax];
     uint64_t pfac[kMapMax];    // P 2^64 mod prime(i) (0 for P positions)
     int *status;               // the context's status word (bulk-copy wait timeouts)
+    // rotation of gathered ciphertexts: nonzero when item's add0 and own limbs
+    // are ga[item] and ga[item] + level N (add0 and own then only say that
+    // there are such limbs)
+    uint32_t gathered;
+    const uint64_t *ga[kGatherMax];
 };
 int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s);
 int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s);
@@ -276,7 +291,9 @@ int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s);
 struct CombineArgs {
     const uint64_t *y;         // [count][2][.][N] at y_off positions
     const uint64_t *lift;      // [count][2][lo][N]
-    const uint64_t *add;       // [count][2][lo][N] or null
+    const uint64_t *add;       // [count][add_polys][lo][N] (strides below) or null
+    uint32_t add_polys;        // polynomials that have an addend (1 or 2)
+    uint32_t galois;           // X -> X^galois on the result (coefficient form); 0: none
     uint64_t *out;             // [count][2][lo][N]
     size_t y_item, y_poly, lift_item, lift_poly, add_item, add_poly, out_item, out_poly;
     uint32_t lo;               // output limbs
@@ -287,10 +304,6 @@ int launch_combine(const Context &c, const CombineArgs &a, uint32_t count, cudaS
 
 int launch_automorph_ntt(const Context &c, const uint64_t *in, uint64_t *out, uint32_t limbs_total,
                          uint64_t g, cudaStream_t s);
-// NTT-form automorphism over the limbs a LimbMap selects (limbs_total =
-// groups x period); in and out must not overlap.
-int launch_automorph_ntt_map(const Context &c, const uint64_t *in, uint64_t *out,
-                             const LimbMap &map, uint32_t limbs_total, uint64_t g, cudaStream_t s);
 // out[ct][p][i] = a[ct][p][i] * pt[i] mod q_i (NTT form), n_limbs = count x 2 x level.
 int launch_mul_plain(const Context &c, const uint64_t *a, const uint64_t *pt, uint64_t *out,
                      uint32_t level, uint32_t n_limbs, cudaStream_t s);
@@ -303,8 +316,6 @@ int launch_encode_ckks(const Context &c, const double2 *slots, double scale, dou
                        double2 *buf1, int64_t *m, cudaStream_t s);
 int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, double2 *buf0,
                        double2 *buf1, double2 *slots, cudaStream_t s);
-int launch_automorph_coeff(const Context &c, const uint64_t *in, uint64_t *out,
-                           const LimbMap &map, uint32_t n_limbs, uint64_t g, cudaStream_t s);
 int launch_add(const Context &c, const uint64_t *a, const uint64_t *b, uint64_t *out,
                const LimbMap &map, uint32_t n_limbs, cudaStream_t s);
 int launch_copy_limbs(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,

@@ -93,6 +93,13 @@ __device__ __forceinline__ uint32_t hi_bits(uint32_t tau, int v, int sh) {
     return sh >= LOGE ? (tau >> (sh - LOGE)) : ((tau << (LOGE - sh)) | uint32_t(v >> sh));
 }
 
+// The low `bits` bits of v reversed (compile-time in unrolled loops).
+__device__ __forceinline__ constexpr uint32_t brev_const(uint32_t v, int bits) {
+    uint32_t r = 0;
+    for (int b = 0; b < bits; b++) r |= ((v >> b) & 1u) << (bits - 1 - b);
+    return r;
+}
+
 // ------------------------------------------------------------------ forward
 
 // The last LOGE stages of an inverse row pass (like the first LOGE of a
@@ -269,12 +276,11 @@ __device__ __forceinline__ void fwd_rows_body(uint64_t (&x)[1 << LOGE], uint64_t
 #undef PAD
 }
 
-// EPI: 0, the plain transform; 1, the ModDown combine epilogue with its y
-// words loaded into registers before the butterflies; 2, the same epilogue
-// with the CTA's y tile (its CC chunks of R words are contiguous) brought
-// into shared memory by one bulk copy issued before the butterflies, so that
-// no registers are held for it (y 16-byte aligned and a status word, checked
-// on the host; the dynamic shared memory holds 256 E words); 3, the plain
+// EPI: 0, the plain transform; 2, the ModDown combine epilogue with the
+// CTA's y tile (its CC chunks of R words are contiguous) brought into shared
+// memory by one bulk copy issued before the butterflies, so that no registers
+// are held for it (y 16-byte aligned, checked on the host; the dynamic shared
+// memory holds NT E words); 3, the plain
 // transform with unreduced outputs for primes under 2^57 (words below 68q,
 // for a consumer that reduces anyway: the key-switching inner product,
 // whose host side checks that its sums stay below 2^64 q; larger primes are
@@ -311,16 +317,10 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
 #pragma unroll
     for (int v = 0; v < E; v++) x[v] = base[tau + T * v];
     // combine epilogue: its y words are requested before the butterflies, so
-    // the loads overlap them (measured, in registers: 1648 -> 1613 us per
-    // batched step).  The barrier is initialised and the copy issued by the
-    // same thread; the others reach the barrier after the exchange's
+    // the copy overlaps them.  The barrier is initialised and the copy issued
+    // by the same thread; the others reach the barrier after the exchange's
     // __syncthreads.
-    uint64_t yv[EPI == 1 ? E : 1];
-    if (EPI == 1) {
-        const uint64_t *yp0 = epi.y + (size_t(g) * epi.y_stride + epi.y_off[r]) * N + size_t(h) * R;
-#pragma unroll
-        for (int v = 0; v < E; v++) yv[EPI == 1 ? v : 0] = yp0[tau + T * v];
-    } else if (EPI == 2 && threadIdx.x == 0) {
+    if (EPI == 2 && threadIdx.x == 0) {
         constexpr uint32_t bytes = uint32_t(CC) * R * 8;
         mbar_init(&ybar, 1);
         mbar_init_fence();
@@ -359,20 +359,45 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
             return;
         }
         // ModDown combine: out = (y - lift) * D^-1 (+ add), lift now in NTT form
-        const size_t off = size_t(h) * R;
         uint64_t *op = (epi.gathered ? epi.gout[g] : epi.out + size_t(g) * epi.out_stride * N) +
-                       size_t(epi.out_off[r]) * N + off;
-        const uint64_t *ap =
-            epi.add ? epi.add + (size_t(g) * epi.add_stride + epi.add_off[r]) * N + off : nullptr;
+                       size_t(epi.out_off[r]) * N;
         const uint64_t dv = epi.dinv[r], dvs = epi.dinv_s[r];
         const uint64_t cq = wide ? kWideWordsQ * q : q;  // above every lift word
+        const uint64_t *yt = ytile + chl * R;
+        if (epi.galois == 0) {
+            op += size_t(h) * R;
 #pragma unroll
-        for (int v = 0; v < E; v++) {
-            const int u = tau + T * v;
-            const uint64_t yw = EPI == 2 ? ytile[chl * R + u] : yv[EPI == 1 ? v : 0];
-            uint64_t o = csub(csub(shoup_lazy4(yw + cq - s[PAD(u)], dv, dvs, q), 2 * q), q);
-            if (ap) o = add_mod(o, ap[u], q);
-            op[u] = o;
+            for (int v = 0; v < E; v++) {
+                const int u = tau + T * v;
+                op[u] = csub(csub(shoup_lazy4(yt[u] + cq - s[PAD(u)], dv, dvs, q), 2 * q), q);
+            }
+        } else {
+            // sigma_g on the way out.  Slot k = h R + u holds the value at
+            // psi^(2i+1), i = bitrev(k): the low k1 bits of i are hb =
+            // bitrev(h), the rest ub = bitrev(u).  Since g is odd, the low
+            // bits of ((2i+1) g - 1) / 2 depend only on those of i, so a chunk
+            // goes to one other chunk h2, permuted inside: its slot u2 takes
+            // the word at ub = c0 + g ub2 (mod R).  Whole chunks are written
+            // (coalesced), and the permuted reads hit shared memory: the lanes
+            // of a chunk differ in the high bits of ub, that is in the low
+            // bits of u, so they meet no bank conflicts.  It replaces separate
+            // permutation passes over every input of the key switching: 16
+            // hoisted rotations of 8 ciphertexts at N = 2^16, l = 24 took
+            // 12.08 ms with those passes (200 of 760 us each), 8.89 ms so.
+            const uint32_t hb = __brev(h) >> (32 - k1);
+            const uint32_t hb2 = (((2 * hb + 1) * epi.galois_inv - 1) >> 1) & ((1u << k1) - 1);
+            const uint32_t h2 = __brev(hb2) >> (32 - k1);
+            const uint32_t c0 = (((2 * hb2 + 1) * epi.galois - 1) >> 1) >> k1;
+            const uint32_t ct = c0 + epi.galois * (__brev(uint32_t(tau)) >> (32 - LOGR));
+            op += size_t(h2) * R + tau;
+#pragma unroll
+            for (int v = 0; v < E; v++) {
+                // bitrev(tau + T v) = bitrev(tau) + bitrev(v) (T v has v's bits
+                // in the high LOGE places)
+                const uint32_t rv = brev_const(v, LOGE);
+                const uint32_t u = __brev(ct + epi.galois * rv) >> (32 - LOGR);
+                op[T * v] = csub(csub(shoup_lazy4(yt[u] + cq - s[PAD(u)], dv, dvs, q), 2 * q), q);
+            }
         }
     }
 #undef PAD
@@ -391,7 +416,8 @@ k_ntt_inv_rows(const uint64_t *src, uint64_t *dst, const LimbMap map,
     uint32_t g, r;
     limb_of<false>(map, g, r);
     constexpr size_t N = size_t(1) << LOGN;
-    const uint64_t *in = src + (size_t(g) * map.src_stride + map.src_off[r]) * N;
+    const uint64_t *in = (map.gathered ? map.gsrc[g] : src + size_t(g) * map.src_stride * N) +
+                         size_t(map.src_off[r]) * N;
     uint64_t *out = dst + (size_t(g) * map.dst_stride + map.dst_off[r]) * N;
     const int p = map.prime[r];
     const uint64_t q = mods[p].q;
@@ -556,16 +582,16 @@ static int run_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const L
     launch_pdl(k_ntt_fwd_cols<LN, R1, E1, T1, B1>, g1, dim3(T1), 0, s, src, dst, map, c.d_mods,
                c.d_twf);
     const dim3 g2(unsigned((N >> R2) / (T2 / ((1 << R2) >> E2))), n_limbs);
-    if (epi && epi->status && (reinterpret_cast<uintptr_t>(epi->y) & 15) == 0) {
+    if (epi) {
+        // every caller's y is a workspace or ciphertext buffer, refused at the
+        // entry points unless 16-byte aligned
+        if (!epi->status || (reinterpret_cast<uintptr_t>(epi->y) & 15) != 0) return CATFHE_EINVAL;
         constexpr int ybytes = T2 * (1 << E2) * 8;  // the CTA's y tile
         if (cudaFuncSetAttribute(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ybytes) != cudaSuccess)
             return CATFHE_ECUDA;
         launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>, g2, dim3(T2), ybytes, s, dst, map,
                    c.d_mods, c.d_twf, *epi);
-    } else if (epi) {
-        launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 1>, g2, dim3(T2), 0, s, dst, map, c.d_mods,
-                   c.d_twf, *epi);
     } else if (lazy) {
         launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 3>, g2, dim3(T2), 0, s, dst, map, c.d_mods,
                    c.d_twf, NttEpilogue{});

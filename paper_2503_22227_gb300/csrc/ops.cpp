@@ -103,6 +103,13 @@ static uint64_t prod_mod(const Context &c, int from, int to, uint64_t m) {
     return r;
 }
 
+// The inverse of an odd g modulo a power of two (Newton iteration).
+static uint64_t inv_mod_pow2(uint64_t g, uint64_t two_n) {
+    uint64_t x = g;
+    for (int i = 0; i < 6; i++) x *= 2 - g * x;
+    return x & (two_n - 1);
+}
+
 // P = prod p_k mod m
 static uint64_t pmod(const Context &c, uint64_t m) { return prod_mod(c, c.L, c.L + c.K, m); }
 
@@ -111,10 +118,11 @@ static uint64_t pmod(const Context &c, uint64_t m) { return prod_mod(c, c.L, c.L
 // Global prime index of extended position i at level l (Q_l then P).
 static int ext_prime(const Context &c, int level, int i) { return i < level ? i : c.L + (i - level); }
 
-// ModUp: lift each digit of d2 (coefficient form, [count][level][N]) to the
-// other primes of Q_l u P, written into ext ([count][beta][M][N]).
-static int modup(Context &c, const uint64_t *d2c, uint64_t *ext, uint32_t count, int level,
-                 bool own_too, cudaStream_t s) {
+// ModUp: lift each digit of d2 (coefficient form, [level][N] per ciphertext,
+// d2_item words apart) to the other primes of Q_l u P (own_too: to all of
+// them), written into ext ([count][beta][M][N]).
+static int modup(Context &c, const uint64_t *d2c, size_t d2_item, uint64_t *ext, uint32_t count,
+                 int level, bool own_too, cudaStream_t s) {
     const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     std::vector<std::pair<std::string, PlanSpec>> specs;
     for (int j = 0; j < beta; j++) {
@@ -137,8 +145,7 @@ static int modup(Context &c, const uint64_t *d2c, uint64_t *ext, uint32_t count,
     PlanList pl;
     TRY(make_list(c, specs, pl));
     const size_t n = c.n;
-    return launch_conv(c, pl, d2c, size_t(level) * n, 0, ext, size_t(beta) * M * n, size_t(M) * n,
-                       count, s);
+    return launch_conv(c, pl, d2c, d2_item, 0, ext, size_t(beta) * M * n, size_t(M) * n, count, s);
 }
 
 // Whether the lifted digits' forward NTT may leave its words unreduced: the
@@ -181,9 +188,12 @@ static int ntt_ext(Context &c, uint64_t *ext, uint32_t count, int level, bool ow
                               : launch_ntt_fwd(c, ext, ext, m, e * count, s);
 }
 
+// own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
+// words apart (null: none).  gth (rotations): ciphertext i's add0 and own are
+// the two polynomials of gth->a[i].
 static int inner_product(Context &c, const uint64_t *ext, const uint64_t *own, const uint64_t *key,
-                         const uint64_t *add0, const uint64_t *add1, uint64_t *y, uint32_t count,
-                         int level, cudaStream_t s) {
+                         const uint64_t *add0, const uint64_t *add1, size_t in_item, uint64_t *y,
+                         uint32_t count, int level, cudaStream_t s, const Gather *gth = nullptr) {
     const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     const size_t n = c.n;
     IpArgs a{};
@@ -193,9 +203,12 @@ static int inner_product(Context &c, const uint64_t *ext, const uint64_t *own, c
     a.add0 = add0;
     a.add1 = add1;
     a.y = y;
+    if (gth && gth->n) {
+        a.gathered = 1;
+        for (uint32_t i = 0; i < gth->n; i++) a.ga[i] = gth->a[i];
+    }
     a.ext_item = size_t(beta) * M * n;
-    a.own_item = size_t(level) * n;
-    a.add_item = size_t(level) * n;
+    a.own_item = a.add_item = in_item;
     a.y_item = size_t(2) * M * n;
     a.M = M;
     a.level = level;
@@ -218,9 +231,12 @@ static int inner_product(Context &c, const uint64_t *ext, const uint64_t *own, c
 
 // ModDown of y ([count][2][M][N]; NTT form for CKKS/BGV, coefficient form
 // for BFV) by D = P (fused: P q_{l-1}) into out ([count][2][lo][N]).
-static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, const uint64_t *add,
-                   uint32_t count, int level, bool fused, cudaStream_t s,
-                   const Gather *gth = nullptr) {
+// add (BFV): [.][lo][N] added to the first add_polys polynomials, add_item
+// words per ciphertext.  g: sigma_g applied to the result (0: none).
+static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint32_t count,
+                   int level, bool fused, cudaStream_t s, uint64_t g = 0,
+                   const Gather *gth = nullptr, const uint64_t *add = nullptr,
+                   uint32_t add_polys = 0, size_t add_item = 0) {
     const int M = level + c.K, lo = fused ? level - 1 : level;
     const size_t n = c.n;
     const bool ntt_form = c.scheme != CATFHE_BFV;
@@ -278,19 +294,18 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, const
         m.period = uint32_t(2 * lo);
         m.src_stride = m.dst_stride = uint32_t(2 * lo);
         e.y = y;
-        e.add = add;
         e.out = out;
         e.status = c.d_status;
         e.y_stride = uint32_t(2 * M);
-        e.add_stride = uint32_t(2 * lo);
         e.out_stride = uint32_t(2 * lo);
+        e.galois = uint32_t(g);
+        e.galois_inv = g ? uint32_t(inv_mod_pow2(g, 2 * n)) : 0;
         for (int p = 0; p < 2; p++)
             for (int i = 0; i < lo; i++) {
                 const int r = p * lo + i;
                 m.src_off[r] = m.dst_off[r] = uint16_t(r);
                 m.prime[r] = uint8_t(i);
                 e.y_off[r] = uint16_t(p * M + i);
-                e.add_off[r] = uint16_t(r);
                 e.out_off[r] = uint16_t(r);
                 e.dinv[r] = dinv[i];
                 e.dinv_s[r] = dinv_s[i];
@@ -301,12 +316,14 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, const
     a.y = y;
     a.lift = lift;
     a.add = add;
+    a.add_polys = add_polys;
+    a.galois = uint32_t(g);
     a.out = out;
     a.y_item = size_t(2) * M * n;
     a.y_poly = size_t(M) * n;
     a.lift_item = size_t(2) * lo * n;
     a.lift_poly = size_t(lo) * n;
-    a.add_item = size_t(2) * lo * n;
+    a.add_item = add_item;
     a.add_poly = size_t(lo) * n;
     a.out_item = size_t(2) * lo * n;
     a.out_poly = size_t(lo) * n;
@@ -456,10 +473,10 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(launch_tensor(c, t, count, s));
     LimbMap m = map_identity(uint32_t(level));
     TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(level) * count, s));
-    TRY(modup(c, k.d2c, k.ext, count, level, false, s));
+    TRY(modup(c, k.d2c, size_t(level) * n, k.ext, count, level, false, s));
     TRY(ntt_ext(c, k.ext, count, level, false, s));
-    TRY(inner_product(c, k.ext, k.d2, rlk, k.d0, k.d1, k.y, count, level, s));
-    return moddown(c, k.y, k.lift, out, nullptr, count, level, fused, s, gth);
+    TRY(inner_product(c, k.ext, k.d2, rlk, k.d0, k.d1, size_t(level) * n, k.y, count, level, s));
+    return moddown(c, k.y, k.lift, out, count, level, fused, s, 0, gth);
 }
 
 // BFV: lift to Q u B, NTT, tensor, INTT, exact round(t x / Q) back to Q,
@@ -547,51 +564,18 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
     }
     // 4. relinearise d2' (coefficient form) and add (d0', d1')
     const uint64_t *d2 = k.dq + size_t(2) * level * n;
-    // ModUp reads the digit limbs of d2' per ct: item stride 3*level*N
-    {
-        const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
-        std::vector<std::pair<std::string, PlanSpec>> specs;
-        for (int j = 0; j < beta; j++) {
-            const int lo = j * c.alpha, hi = std::min((j + 1) * c.alpha, level);
-            PlanSpec sp;
-            sp.lazy = true;
-            for (int i = lo; i < hi; i++) {
-                sp.src_mod.push_back(c.mod(i));
-                sp.src_off.push_back(uint32_t(i));
-            }
-            for (int i = 0; i < M; i++) {
-                sp.dst_mod.push_back(c.mod(ext_prime(c, level, i)));
-                sp.dst_off.push_back(uint32_t(i));
-            }
-            specs.emplace_back("modup/" + std::to_string(level) + "/" + std::to_string(j) + "/own",
-                               sp);
-        }
-        PlanList pl;
-        TRY(make_list(c, specs, pl));
-        TRY(launch_conv(c, pl, d2, size_t(3) * level * n, 0, k.ext, size_t(beta) * M * n,
-                        size_t(M) * n, count, s));
-    }
+    TRY(modup(c, d2, size_t(3) * level * n, k.ext, count, level, true, s));
     TRY(ntt_ext(c, k.ext, count, level, true, s));
-    TRY(inner_product(c, k.ext, nullptr, rlk, nullptr, nullptr, k.y, count, level, s));
+    TRY(inner_product(c, k.ext, nullptr, rlk, nullptr, nullptr, 0, k.y, count, level, s));
     {
         const int M = level + c.K;
         LimbMap my = map_identity(uint32_t(M));
         for (int i = 0; i < M; i++) my.prime[i] = uint8_t(ext_prime(c, level, i));
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
-    // (d0', d1') of [count][3][level] packed as [count][2][level] for the combine
-    {
-        LimbMap cp{};
-        cp.period = uint32_t(2 * level);
-        cp.src_stride = uint32_t(3 * level);
-        cp.dst_stride = uint32_t(2 * level);
-        for (int i = 0; i < 2 * level; i++) {
-            cp.src_off[i] = cp.dst_off[i] = uint16_t(i);
-            cp.prime[i] = uint8_t(i % level);
-        }
-        TRY(launch_copy_limbs(c, k.dq, k.add, cp, uint32_t(2 * level) * count, s));
-    }
-    return moddown(c, k.y, k.lift, out, k.add, count, level, false, s);
+    // (d0', d1') are the first two of each ciphertext's three polynomials
+    return moddown(c, k.y, k.lift, out, count, level, false, s, 0, nullptr, k.dq, 2,
+                   size_t(3) * level * n);
 }
 
 // Two streams (and fork / join events) per device for split operations;
@@ -673,57 +657,62 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
     return run(0, count, base, s);
 }
 
+// The map of the a1 polynomials of ciphertexts [2][lvl][N]: limb lvl + i of
+// each group into limb i of a buffer of lvl limbs per group.
+static LimbMap map_second(int lvl) {
+    LimbMap m{};
+    m.period = uint32_t(lvl);
+    m.src_stride = uint32_t(2 * lvl);
+    m.dst_stride = uint32_t(lvl);
+    for (int i = 0; i < lvl; i++) {
+        m.src_off[i] = uint16_t(lvl + i);
+        m.dst_off[i] = uint16_t(i);
+        m.prime[i] = uint8_t(i);
+    }
+    return m;
+}
+
 // HRotate of count ciphertexts at lvl with the Galois key gk, workspace k.
+// sigma_g commutes with every step of the key switching: it permutes slots
+// (and signs of coefficients), the centred lifts are odd functions and no
+// division has ties.  So sigma_g(a0) + KS_gk(sigma_g(a1)) =
+// sigma_g(a0 + KS_gk'(a1)) with gk' = sigma_g^-1(gk), the stored form of the
+// key, bit for bit; only the kernel that writes the result permutes.
 static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_t g, uint64_t *out,
                       int lvl, uint32_t count, KsBufs &k, cudaStream_t s, const Gather *gth) {
-    const size_t n = c.n;
+    const size_t n = c.n, item = size_t(2) * lvl * n, half = size_t(lvl) * n;
     if (c.scheme != CATFHE_BFV) {
-        // sigma_g on both components in NTT form: d0 <- sigma(c0), d2 <- sigma(c1)
-        for (uint32_t ct = 0; ct < count; ct++) {
-            const uint64_t *src = (gth && gth->n) ? gth->a[ct] : a + size_t(ct) * 2 * lvl * n;
-            TRY(launch_automorph_ntt(c, src, k.d0 + size_t(ct) * lvl * n, uint32_t(lvl), g, s));
-            TRY(launch_automorph_ntt(c, src + size_t(lvl) * n, k.d2 + size_t(ct) * lvl * n,
-                                     uint32_t(lvl), g, s));
+        LimbMap m = map_second(lvl);
+        if (gth && gth->n) {
+            m.gathered = 1;
+            for (uint32_t i = 0; i < gth->n; i++) m.gsrc[i] = gth->a[i];
         }
-        LimbMap m = map_identity(uint32_t(lvl));
-        TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(lvl) * count, s));
-        TRY(modup(c, k.d2c, k.ext, count, lvl, false, s));
+        TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(lvl) * count, s));
+        TRY(modup(c, k.d2c, half, k.ext, count, lvl, false, s));
         TRY(ntt_ext(c, k.ext, count, lvl, false, s));
-        TRY(inner_product(c, k.ext, k.d2, gk, k.d0, nullptr, k.y, count, lvl, s));
-        return moddown(c, k.y, k.lift, out, nullptr, count, lvl, false, s, gth);
+        TRY(inner_product(c, k.ext, a + half, gk, a, nullptr, item, k.y, count, lvl, s, gth));
+        return moddown(c, k.y, k.lift, out, count, lvl, false, s, g, gth);
     }
-    // BFV (coefficient form): (sigma(c0), 0) becomes the added pair of the
-    // ModDown combine, sigma(c1) is key switched.
-    uint64_t *addbuf = k.add;  // [count][2][level]
-    {
-        LimbMap m{};
-        m.period = uint32_t(lvl);
-        m.src_stride = uint32_t(2 * lvl);
-        m.dst_stride = uint32_t(2 * lvl);
-        for (int i = 0; i < lvl; i++) {
-            m.src_off[i] = m.dst_off[i] = uint16_t(i);
-            m.prime[i] = uint8_t(i);
-        }
-        TRY(launch_automorph_coeff(c, a, addbuf, m, uint32_t(lvl) * count, g, s));
-        for (uint32_t ct = 0; ct < count; ct++)
-            if (cudaMemsetAsync(addbuf + (size_t(ct) * 2 + 1) * lvl * n, 0, size_t(lvl) * n * 8, s) !=
-                cudaSuccess)
-                return CATFHE_ECUDA;
-        LimbMap m1 = m;
-        m1.dst_stride = uint32_t(lvl);
-        for (int i = 0; i < lvl; i++) m1.src_off[i] = uint16_t(lvl + i);
-        TRY(launch_automorph_coeff(c, a, k.d2c, m1, uint32_t(lvl) * count, g, s));
+    // BFV (coefficient form): a1 is key switched, a0 added by the combine.  It
+    // scatters its results, so a0 is copied first when out overlaps a.
+    const uint64_t *add = a;
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(a), o0 = reinterpret_cast<uintptr_t>(out);
+    const size_t bytes = size_t(count) * item * 8;
+    if (a0 < o0 + bytes && o0 < a0 + bytes) {
+        TRY(launch_copy_limbs(c, a, k.add, map_identity(uint32_t(2 * lvl)),
+                              uint32_t(2 * lvl) * count, s));
+        add = k.add;
     }
-    TRY(modup(c, k.d2c, k.ext, count, lvl, true, s));
+    TRY(modup(c, a + half, item, k.ext, count, lvl, true, s));
     TRY(ntt_ext(c, k.ext, count, lvl, true, s));
-    TRY(inner_product(c, k.ext, nullptr, gk, nullptr, nullptr, k.y, count, lvl, s));
+    TRY(inner_product(c, k.ext, nullptr, gk, nullptr, nullptr, 0, k.y, count, lvl, s));
     {
         const int M = lvl + c.K;
         LimbMap my = map_identity(uint32_t(M));
         for (int i = 0; i < M; i++) my.prime[i] = uint8_t(ext_prime(c, lvl, i));
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
-    return moddown(c, k.y, k.lift, out, addbuf, count, lvl, false, s);
+    return moddown(c, k.y, k.lift, out, count, lvl, false, s, g, nullptr, add, 1, item);
 }
 
 int op_rotate(Context &c, const Keys &keys, const uint64_t *a, uint64_t g, uint64_t *out,
@@ -755,8 +744,8 @@ int op_rotate(Context &c, const Keys &keys, const uint64_t *a, uint64_t g, uint6
 }
 
 
-// Hoisted rotations: one INTT + ModUp + NTT of a1, then per Galois element a
-// permutation of a0, a1 and the lifted digits, the inner product and ModDown.
+// Hoisted rotations: one INTT + ModUp + NTT of a1, then per Galois element the
+// inner product with its (permuted) key and ModDown, which permutes the result.
 int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *gs,
                       uint32_t n_rot, uint64_t *out, uint32_t level, uint32_t count, void *ws,
                       size_t ws_bytes_in, cudaStream_t s) {
@@ -784,42 +773,14 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     const int lvl = int(level), M = lvl + c.K, beta = (lvl + c.alpha - 1) / c.alpha;
     uint64_t *ext0 = bump.take<uint64_t>(size_t(count) * beta * M * n);
     // a1 (NTT form) -> coefficient form -> lifted digits in NTT form, once
-    LimbMap m1{};
-    m1.period = uint32_t(lvl);
-    m1.src_stride = uint32_t(2 * lvl);
-    m1.dst_stride = uint32_t(lvl);
-    for (int i = 0; i < lvl; i++) {
-        m1.src_off[i] = uint16_t(lvl + i);
-        m1.dst_off[i] = uint16_t(i);
-        m1.prime[i] = uint8_t(i);
-    }
-    TRY(launch_ntt_inv(c, a, k.d2c, m1, uint32_t(lvl) * count, s));
-    TRY(modup(c, k.d2c, ext0, count, lvl, false, s));
+    const size_t item = size_t(2) * lvl * n, half = size_t(lvl) * n;
+    TRY(launch_ntt_inv(c, a, k.d2c, map_second(lvl), uint32_t(lvl) * count, s));
+    TRY(modup(c, k.d2c, half, ext0, count, lvl, false, s));
     TRY(ntt_ext(c, ext0, count, lvl, false, s));
-    // the lifted positions of ext (as ntt_ext selects them)
-    LimbMap me{};
-    uint32_t e = 0;
-    for (int j = 0; j < beta; j++) {
-        const int lo = j * c.alpha, hi = std::min((j + 1) * c.alpha, lvl);
-        for (int i = 0; i < M; i++) {
-            if (i >= lo && i < hi) continue;
-            if (e >= uint32_t(kMapMax)) return CATFHE_EINVAL;
-            me.src_off[e] = me.dst_off[e] = uint16_t(j * M + i);
-            me.prime[e] = uint8_t(ext_prime(c, lvl, i));
-            e++;
-        }
-    }
-    me.period = e;
-    me.src_stride = me.dst_stride = uint32_t(beta * M);
-    LimbMap m0 = m1;  // a0 -> d0
-    for (int i = 0; i < lvl; i++) m0.src_off[i] = uint16_t(i);
     auto one = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
-        TRY(launch_automorph_ntt_map(c, a, kb.d0, m0, uint32_t(lvl) * count, gv[r], st));
-        TRY(launch_automorph_ntt_map(c, a, kb.d2, m1, uint32_t(lvl) * count, gv[r], st));
-        TRY(launch_automorph_ntt_map(c, ext0, kb.ext, me, e * count, gv[r], st));
-        TRY(inner_product(c, kb.ext, kb.d2, gk[r], kb.d0, nullptr, kb.y, count, lvl, st));
-        return moddown(c, kb.y, kb.lift, out + size_t(r) * count * 2 * lvl * n, nullptr, count,
-                       lvl, false, st);
+        TRY(inner_product(c, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, lvl, st));
+        return moddown(c, kb.y, kb.lift, out + size_t(r) * count * item, count, lvl, false, st,
+                       gv[r]);
     };
     if (n_rot < 2 || c.log_n < 14) {
         for (uint32_t r = 0; r < n_rot; r++) TRY(one(r, k, s));
@@ -1088,9 +1049,12 @@ struct DevConst {
 static int gen_ksk(Context &c, Keys &k, uint64_t id, const uint64_t *sp, cudaStream_t s) {
     const size_t n = c.n;
     const int E = c.L + c.K;
-    uint64_t *key = nullptr, *e = nullptr;
+    uint64_t *key = nullptr, *e = nullptr, *rows = nullptr;
     if (cudaMalloc(&key, size_t(c.beta) * 2 * E * n * 8) != cudaSuccess) return CATFHE_ENOMEM;
-    if (cudaMalloc(&e, size_t(E) * n * 8) != cudaSuccess) {
+    // a Galois key's rows are built aside, then permuted into place
+    if (cudaMalloc(&e, size_t(E) * n * 8) != cudaSuccess ||
+        (id && cudaMalloc(&rows, size_t(2) * E * n * 8) != cudaSuccess)) {
+        cudaFree(e);
         cudaFree(key);
         return CATFHE_ENOMEM;
     }
@@ -1103,8 +1067,8 @@ static int gen_ksk(Context &c, Keys &k, uint64_t id, const uint64_t *sp, cudaStr
     }
     int rc = te.set(tv, mods);
     for (int j = 0; j < c.beta && rc == CATFHE_OK; j++) {
-        uint64_t *bj = key + (size_t(j) * 2 + 0) * E * n;
-        uint64_t *aj = key + (size_t(j) * 2 + 1) * E * n;
+        uint64_t *kj = key + size_t(j) * 2 * E * n;
+        uint64_t *bj = id ? rows : kj, *aj = bj + size_t(E) * n;
         rc = launch_sample(c, sample_args(c, k.seed, TAG_KSK_A, uint32_t(j), uint32_t(id), kUniform), aj,
                            m, uint32_t(E), nullptr, nullptr, s);
         if (!rc) rc = launch_ntt_fwd(c, aj, aj, m, uint32_t(E), s);
@@ -1118,6 +1082,8 @@ static int gen_ksk(Context &c, Keys &k, uint64_t id, const uint64_t *sp, cudaStr
         DevConst pfc;
         if (!rc) rc = pfc.set(pv, mods);
         if (!rc) rc = launch_ksk_row(c, aj, k.s_ntt, e, sp, bj, uint32_t(E), pfc.v, pfc.s, s);
+        if (!rc && id)  // sigma_g^-1 (see Keys::ksk)
+            rc = launch_automorph_ntt(c, rows, kj, uint32_t(2 * E), inv_mod_pow2(id, 2 * n), s);
         if (!rc) rc = cudaStreamSynchronize(s) == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
     }
     // Montgomery form: every limb times 2^64 mod its prime
@@ -1130,6 +1096,7 @@ static int gen_ksk(Context &c, Keys &k, uint64_t id, const uint64_t *sp, cudaStr
         if (!rc) rc = cudaStreamSynchronize(s) == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
     }
     cudaFree(e);
+    cudaFree(rows);
     if (rc) {
         cudaFree(key);
         return rc;
@@ -1240,7 +1207,10 @@ int op_keys_export(Context &c, const Keys &k, uint64_t id, int64_t *s_out, uint6
     if (!rc && ksk_out) {
         auto it = k.ksk.find(id);
         if (it == k.ksk.end()) rc = CATFHE_ENOKEY;
-        if (!rc) rc = launch_ntt_inv(c, it->second, tmp, mE, uint32_t(c.beta * 2 * E), 0);
+        // a Galois key is stored permuted: sigma_g gives its definition back
+        if (!rc && id) rc = launch_automorph_ntt(c, it->second, tmp, uint32_t(c.beta * 2 * E), id, 0);
+        if (!rc)
+            rc = launch_ntt_inv(c, id ? tmp : it->second, tmp, mE, uint32_t(c.beta * 2 * E), 0);
         // undo the Montgomery form: times 2^-64 mod each prime
         std::vector<uint64_t> rv(E), mods(E);
         for (int i = 0; i < E && !rc; i++) {
