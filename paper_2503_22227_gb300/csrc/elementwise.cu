@@ -87,11 +87,13 @@ int launch_tensor(const Context &c, const TensorArgs &a, uint32_t count, cudaStr
 // y_p[i] = sum_j c_j[i] * key_j[p][i] (+ P * add_p[i] on ciphertext primes).
 
 // The first limb of an item's own digits and of its addends.
+template <bool GATHER>
 __device__ __forceinline__ const uint64_t *ip_own(const IpArgs &A, uint32_t item, size_t n) {
-    return A.gathered ? A.ga[item] + size_t(A.level) * n : A.own + item * A.own_item;
+    return GATHER ? A.ga[item] + size_t(A.level) * n : A.own + item * A.own_item;
 }
+template <bool GATHER>
 __device__ __forceinline__ const uint64_t *ip_add0(const IpArgs &A, uint32_t item) {
-    return A.gathered ? A.ga[item] : A.add0 + item * A.add_item;
+    return GATHER ? A.ga[item] : A.add0 + item * A.add_item;
 }
 
 // Many digits (beta > 8): digit by digit, loads interleaved with products,
@@ -99,6 +101,7 @@ __device__ __forceinline__ const uint64_t *ip_add0(const IpArgs &A, uint32_t ite
 // index, so the CTAs of all ciphertexts that read one block of the
 // evaluation key are dispatched back to back: the key crosses HBM once per
 // batch and is served from L2 after.
+template <bool GATHER>
 __global__ void __launch_bounds__(256)
 k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     grid_dep_wait();
@@ -114,7 +117,7 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
     if (i < A.level && A.pfac[i] != 0) {
         if (A.add0) {
-            const ulonglong2 d = ld2(ip_add0(A, item) + size_t(i) * n + x);
+            const ulonglong2 d = ld2(ip_add0<GATHER>(A, item) + size_t(i) * n + x);
             mac(a0, d.x, A.pfac[i]);
             mac(a1, d.y, A.pfac[i]);
         }
@@ -125,7 +128,7 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
         }
     }
     for (uint32_t j = 0; j < A.beta; j++) {
-        const ulonglong2 c = (j == own_digit) ? ld2(ip_own(A, item, n) + size_t(i) * n + x)
+        const ulonglong2 c = (j == own_digit) ? ld2(ip_own<GATHER>(A, item, n) + size_t(i) * n + x)
                                               : ld2(ext + (size_t(j) * A.M + i) * n + x);
         const ulonglong2 kb = ld2(A.key + ((size_t(j) * 2 + 0) * KL + A.key_limb[i]) * n + x);
         const ulonglong2 ka = ld2(A.key + ((size_t(j) * 2 + 1) * KL + A.key_limb[i]) * n + x);
@@ -159,7 +162,7 @@ struct IpTile {
 // blockIdx.z: a group of consecutive ciphertexts of the launch (the host
 // splits them when one group per tile would leave the last wave of CTAs
 // mostly empty); each group's CTA loads its key tiles once.
-template <int BETA>
+template <int BETA, bool GATHER>
 __global__ void __launch_bounds__(IpTile<BETA>::value / 2)
 k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint32_t count) {
     grid_dep_wait();
@@ -189,11 +192,11 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
         mbar_expect_tx(&bars[b], item_bytes);
         const uint64_t *ext = A.ext + item * A.ext_item;
         for (uint32_t j = 0; j < beta; j++) {
-            const uint64_t *src = (j == own_digit) ? ip_own(A, item, n) + size_t(i) * n
+            const uint64_t *src = (j == own_digit) ? ip_own<GATHER>(A, item, n) + size_t(i) * n
                                                    : ext + (size_t(j) * A.M + i) * n;
             bulk_load(dst + j * kIpTile, src + x0, TB, &bars[b]);
         }
-        if (f0) bulk_load(dst + BETA * kIpTile, ip_add0(A, item) + size_t(i) * n + x0, TB, &bars[b]);
+        if (f0) bulk_load(dst + BETA * kIpTile, ip_add0<GATHER>(A, item) + size_t(i) * n + x0, TB, &bars[b]);
         if (f1) bulk_load(dst + (BETA + 1) * kIpTile, A.add1 + item * A.add_item + size_t(i) * n + x0, TB, &bars[b]);
     };
 
@@ -312,8 +315,39 @@ static unsigned ip_groups(K kernel, unsigned threads, size_t smem, size_t ctas, 
     return top >= 1.1 * one ? best : 1;
 }
 
+template <int BETA, bool GATHER>
+static int ip_run_bulk(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
+    constexpr uint32_t tile = IpTile<BETA>::value;
+    constexpr size_t smem = size_t(4 * BETA + 4) * tile * 8;
+    const auto kernel = k_ip_bulk<BETA, GATHER>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
+        cudaSuccess)
+        return CATFHE_ECUDA;
+    const unsigned groups = ip_groups(kernel, tile / 2, smem, c.n / tile * a.M, count);
+    launch_pdl(kernel, dim3(unsigned(c.n / tile), a.M, groups), dim3(tile / 2), smem, s, a, c.d_mods,
+               uint32_t(c.log_n), count);
+    return ok();
+}
+
+template <bool GATHER>
+static int ip_run(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
+    switch (a.beta) {
+        case 1: return ip_run_bulk<1, GATHER>(c, a, count, s);
+        case 2: return ip_run_bulk<2, GATHER>(c, a, count, s);
+        case 3: return ip_run_bulk<3, GATHER>(c, a, count, s);
+        case 4: return ip_run_bulk<4, GATHER>(c, a, count, s);
+        case 5: return ip_run_bulk<5, GATHER>(c, a, count, s);
+        case 6: return ip_run_bulk<6, GATHER>(c, a, count, s);
+        case 7: return ip_run_bulk<7, GATHER>(c, a, count, s);
+        case 8: return ip_run_bulk<8, GATHER>(c, a, count, s);
+        default:
+            launch_pdl(k_ip_stream<GATHER>, dim3(count, unsigned((c.n / 2 + 255) / 256), a.M),
+                       dim3(256), 0, s, a, c.d_mods, uint32_t(c.log_n));
+            return ok();
+    }
+}
+
 int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
-    const size_t n = c.n;
     // bulk copies: every buffer is a workspace, a key or a ciphertext, refused
     // at the entry points unless 16-byte aligned
     bool aligned = a.status != nullptr && aligned16(a.ext) && aligned16(a.key) && aligned16(a.y) &&
@@ -321,26 +355,7 @@ int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s)
                    ((a.ext_item | a.own_item | a.add_item | a.y_item) & 1) == 0;
     for (uint32_t k = 0; a.gathered && k < count; k++) aligned = aligned && aligned16(a.ga[k]);
     if (!aligned) return CATFHE_EINVAL;
-    switch (a.beta) {
-#define IPB(B)                                                                                   \
-    case B: {                                                                                    \
-        constexpr uint32_t tile = IpTile<B>::value;                                              \
-        const size_t smb = size_t(4 * B + 4) * tile * 8;                                         \
-        if (cudaFuncSetAttribute(k_ip_bulk<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                 int(smb)) != cudaSuccess)                                       \
-            return CATFHE_ECUDA;                                                                 \
-        const unsigned groups = ip_groups(k_ip_bulk<B>, tile / 2, smb, n / tile * a.M, count);   \
-        launch_pdl(k_ip_bulk<B>, dim3(unsigned(n / tile), a.M, groups), dim3(tile / 2), smb, s,  \
-                   a, c.d_mods, c.log_n, count);                                                 \
-        break;                                                                                   \
-    }
-        IPB(1) IPB(2) IPB(3) IPB(4) IPB(5) IPB(6) IPB(7) IPB(8)
-#undef IPB
-        default:
-            launch_pdl(k_ip_stream, dim3(count, unsigned((n / 2 + 255) / 256), a.M), dim3(256), 0, s,
-                       a, c.d_mods, c.log_n);
-    }
-    return ok();
+    return a.gathered ? ip_run<true>(c, a, count, s) : ip_run<false>(c, a, count, s);
 }
 
 // ------------------------------------------------------------------ ModDown combine

@@ -280,7 +280,8 @@ __device__ __forceinline__ void fwd_rows_body(uint64_t (&x)[1 << LOGE], uint64_t
 // CTA's y tile (its CC chunks of R words are contiguous) brought into shared
 // memory by one bulk copy issued before the butterflies, so that no registers
 // are held for it (y 16-byte aligned, checked on the host; the dynamic shared
-// memory holds NT E words); 3, the plain
+// memory holds NT E words); 4, the same with sigma_g applied as it stores; 3,
+// the plain
 // transform with unreduced outputs for primes under 2^57 (words below 68q,
 // for a consumer that reduces anyway: the key-switching inner product,
 // whose host side checks that its sums stay below 2^64 q; larger primes are
@@ -320,7 +321,7 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
     // the copy overlaps them.  The barrier is initialised and the copy issued
     // by the same thread; the others reach the barrier after the exchange's
     // __syncthreads.
-    if (EPI == 2 && threadIdx.x == 0) {
+    if ((EPI == 2 || EPI == 4) && threadIdx.x == 0) {
         constexpr uint32_t bytes = uint32_t(CC) * R * 8;
         mbar_init(&ybar, 1);
         mbar_init_fence();
@@ -331,7 +332,7 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
                   bytes, &ybar);
     }
     // q < 2^57: no conditional subtractions in either pass, words stay below
-    // 4q + 4 log2(N) q <= 68q < 2^64, then one reduction (none for EPI 1-3);
+    // 4q + 4 log2(N) q <= 68q < 2^64, then one reduction (none for EPI 2-4);
     // else below 8q, then three conditional subtractions.  (Each branch with
     // its own reduction, and 3 CTAs per SM: fewer register spills, measured
     // forward transform 297 -> 284 us.)
@@ -351,7 +352,7 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
         for (int v = 0; v < E; v++) base[tau + T * v] = s[PAD(tau + T * v)];
     } else {
         // a bounded wait that the CTA decides together (__syncthreads_and)
-        if (EPI == 2 && !__syncthreads_and(mbar_wait(&ybar, 0))) {
+        if (!__syncthreads_and(mbar_wait(&ybar, 0))) {
             if (threadIdx.x == 0) {
                 atomicOr(epi.status, kStatusNttWait);
                 mbar_wait(&ybar, 0);  // a bounded time for the copy to land
@@ -364,7 +365,7 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
         const uint64_t dv = epi.dinv[r], dvs = epi.dinv_s[r];
         const uint64_t cq = wide ? kWideWordsQ * q : q;  // above every lift word
         const uint64_t *yt = ytile + chl * R;
-        if (epi.galois == 0) {
+        if (EPI == 2) {
             op += size_t(h) * R;
 #pragma unroll
             for (int v = 0; v < E; v++) {
@@ -587,11 +588,12 @@ static int run_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const L
         // entry points unless 16-byte aligned
         if (!epi->status || (reinterpret_cast<uintptr_t>(epi->y) & 15) != 0) return CATFHE_EINVAL;
         constexpr int ybytes = T2 * (1 << E2) * 8;  // the CTA's y tile
-        if (cudaFuncSetAttribute(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, ybytes) != cudaSuccess)
+        const auto kernel = epi->galois ? k_ntt_fwd_rows<LN, R2, E2, T2, B2, 4>
+                                        : k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ybytes) !=
+            cudaSuccess)
             return CATFHE_ECUDA;
-        launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>, g2, dim3(T2), ybytes, s, dst, map,
-                   c.d_mods, c.d_twf, *epi);
+        launch_pdl(kernel, g2, dim3(T2), ybytes, s, dst, map, c.d_mods, c.d_twf, *epi);
     } else if (lazy) {
         launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 3>, g2, dim3(T2), 0, s, dst, map, c.d_mods,
                    c.d_twf, NttEpilogue{});
