@@ -131,7 +131,9 @@ int ctx_init(Context &c, const catfhe_params &p) {
         }
     }
     h_cdt(c.cdt);
-    if (cudaGetDevice(&c.device) != cudaSuccess) return CATFHE_ECUDA;
+    if (cudaGetDevice(&c.device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess)
+        return CATFHE_ECUDA;
     if (cudaMalloc(&c.d_status, sizeof(int)) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMemset(c.d_status, 0, sizeof(int)) != cudaSuccess) return CATFHE_ECUDA;
     if (cudaMalloc(&c.d_mods, sizeof(DevMod) * np) != cudaSuccess) return CATFHE_ENOMEM;
@@ -151,6 +153,7 @@ void ctx_free(Context &c) {
     cudaFree(c.d_twf);
     cudaFree(c.d_twi);
     for (auto &kv : c.plans) cudaFree(kv.second);
+    for (auto &kv : c.mma_plans) cudaFree(const_cast<uint64_t *>(kv.second.p));
     cudaFree(c.scratch.ptr);
     c.plans.clear();
 }
@@ -353,6 +356,25 @@ PlanRef get_plan_extra(Context &c, const std::string &key0, const PlanSpec &spec
         return ref;
     }
     return upload_plan(c, key, build_plan(spec), extra);
+}
+
+MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec) {
+    auto it = c.mma_plans.find(key);
+    if (it != c.mma_plans.end()) return it->second;
+    MmaRef ref;
+    const std::vector<uint64_t> img = build_mma_plan(spec, c.n);
+    if (!img.empty()) {
+        uint64_t *dev = nullptr;
+        if (cudaMalloc(&dev, img.size() * 8) != cudaSuccess) return ref;
+        if (cudaMemcpy(dev, img.data(), img.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaFree(dev);
+            return ref;
+        }
+        ref.p = dev;
+        ref.head = img[0];
+        ref.counts = img[1];
+    }
+    return c.mma_plans[key] = ref;
 }
 
 PlanRef get_plan(Context &c, const std::string &key, const PlanSpec &spec) {

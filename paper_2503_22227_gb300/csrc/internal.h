@@ -108,8 +108,50 @@ struct PlanRef {
 };
 struct Context;
 PlanRef get_plan(Context &c, const std::string &key, const PlanSpec &spec);
+// Device copy of a plan's tensor-core image and its header words.
+struct MmaRef {
+    const uint64_t *p = nullptr;  // device image, null when the plan has none
+    uint64_t head = 0, counts = 0;
+};
+MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec);
 PlanRef get_plan_extra(Context &c, const std::string &key, const PlanSpec &spec,
                        const std::vector<uint64_t> &extra);
+
+// Image of a plan for the tensor-core conversion (mmaplan.cpp, conv_mma.cu),
+// in 64-bit words: word 0 is the header
+//   K | column blocks << 8 | K cores << 16 | lazy << 24 | (6-digit blocks) << 32
+// word 1 the targets of each block (4 bits each), then per source {m, w, w's
+// Shoup quotient, c | shift << 32, src_off N, 0}, per block three target slots
+// {C, -p, 4 floats (top, middle, low weight, bias), dst_off N, 0}, and the
+// fp16 matrix as 16-byte rows of 8 elements, [core][column]: one core per
+// source (its bytes), one for v and the constant row, padded to an even number.
+constexpr uint32_t kMmaMaxK = 15;
+constexpr uint32_t kMmaMaxBlocks = 16;
+constexpr uint32_t kMmaSrcWords = 6, kMmaTgtWords = 6;
+// Column blocks of 16: three targets of 5 digits or two of 6.
+constexpr uint32_t kMmaBlock = 16, kMmaSlots = 3;
+struct MmaLayout {
+    uint32_t cores, src, tgt, b, words;
+};
+__host__ __device__ inline MmaLayout mma_layout(uint32_t K, uint32_t nblk) {
+    MmaLayout l;
+    l.cores = (K + 2) & ~1u;
+    l.src = 2;
+    l.tgt = l.src + K * kMmaSrcWords;
+    l.b = (l.tgt + nblk * kMmaSlots * kMmaTgtWords + 15) & ~15u;
+    l.words = l.b + l.cores * kMmaBlock * nblk * 2;
+    return l;
+}
+// Targets of an image, from its word 1.
+inline uint32_t mma_targets(uint64_t counts) {
+    uint32_t t = 0;
+    for (; counts; counts >>= 4) t += uint32_t(counts & 15);
+    return t;
+}
+// Empty when the conversion does not fit (K > 15, a source modulus outside
+// (2^32, 2^60), a target outside (2^40, 2^60), or a column's sums not provably
+// below 2^22).
+std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n);
 
 // Up to this many plans run in one launch (grid.z).
 struct PlanList {
@@ -120,6 +162,21 @@ struct PlanList {
     uint32_t words;  // largest packed size among them
     uint32_t mont;   // all plans use the Montgomery layout
     uint32_t split;  // ... with split weights
+};
+
+// The same launch in the tensor-core form: each plan's image, its two header
+// words (as launch constants, so that what depends on them is uniform), and
+// the plan in the Montgomery layout for the rare exact comparison.
+constexpr uint32_t kMmaPlans = 16;
+struct MmaList {
+    const uint64_t *img[kMmaPlans], *p[kMmaPlans];
+    uint64_t head[kMmaPlans], counts[kMmaPlans];
+    uint32_t n;
+};
+struct ConvPlans {
+    PlanList l;
+    MmaList m;
+    bool mma = false;  // m is complete: the launch takes it
 };
 
 // Host-side prime record.
@@ -145,8 +202,10 @@ struct Context {
     uint64_t cdt[19] = {};
     std::map<std::string, uint64_t *> plans;     // device copies of packed plans
     std::map<std::string, uint32_t> plan_sizes;  // words
+    std::map<std::string, MmaRef> mma_plans;     // tensor-core images (device)
     Scratch scratch;
     int device = 0;
+    int sms = 0;  // the device's SM count
     // NTT schedule index for this ring degree (see ntt.cu), per launch size
     // class (ntt_class)
     int ntt_sched[3] = {0, 0, 0};
@@ -229,9 +288,13 @@ int tune_ntt(Context &c, uint32_t limbs, cudaStream_t s, int *chosen, float *us_
 // grid.z runs plan z over items item = 0..items-1 (grid.y): sources at
 // src + item * src_item + src_off * N, targets at dst + item * dst_item + ...;
 // plan z may add z * src_plan / dst_plan to the item bases.
-int launch_conv(const Context &c, const PlanList &plans, const uint64_t *src, size_t src_item,
+int launch_conv(const Context &c, const ConvPlans &plans, const uint64_t *src, size_t src_item,
                 size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan, uint32_t items,
                 cudaStream_t s);
+// The tensor-core form of launch_conv for plans that have an image.
+int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src, size_t src_item,
+                    size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan,
+                    uint32_t items, cudaStream_t s);
 // BFV: given the tensor x over Q u B (coefficient form, Q limbs first) of
 // each item, writes round(t x / Q) mod q_i: y = t x; z = (y - [y]_Q) Q^-1 over
 // B (plan q_to_b lifts [y]_Q with pre = t and post = 1); then the centred

@@ -146,14 +146,15 @@ int op_rescale_noalloc_impl(Context &c, const uint64_t *a, uint64_t *out, uint32
         m.prime[p] = uint8_t(lvl - 1);
     }
     if ((rc = launch_ntt_inv(c, a, last, m, 2 * count, s))) return rc;
-    PlanList pl{};
+    ConvPlans cp{};
+    PlanList &pl = cp.l;
     pl.n = 1;
     pl.kmax = 1;
     pl.kmin = 1;
     pl.words = uint32_t(words);
     pl.mont = 1;
     pl.p[0] = plan;
-    if ((rc = launch_conv(c, pl, last, n, 0, lift, size_t(lo) * n, 0, 2 * count, s))) return rc;
+    if ((rc = launch_conv(c, cp, last, n, 0, lift, size_t(lo) * n, 0, 2 * count, s))) return rc;
     LimbMap ml{};
     ml.period = uint32_t(lo);
     ml.src_stride = ml.dst_stride = uint32_t(lo);

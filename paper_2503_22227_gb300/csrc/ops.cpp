@@ -57,18 +57,32 @@ static int get_ws(Context &c, void *ws, size_t ws_bytes, size_t need, char **out
     return CATFHE_OK;
 }
 
-// One launch's plans, all in one layout: Montgomery when every plan fits it
-// (with split weights when every plan fits those too), else exact.
+// One launch's plans, all in one form: Montgomery when every plan fits it
+// (with split weights when every plan fits those too), else exact; and the
+// tensor-core form beside it when every plan has one and some plan has more
+// than one source.  launch_conv chooses between the two.
 static int make_list(Context &c, const std::vector<std::pair<std::string, PlanSpec>> &specs,
-                     PlanList &pl) {
+                     ConvPlans &cp) {
     bool all = true, all_split = true;
     for (const auto &s : specs) {
         all = all && plan_fits_mont(s.second);
         all_split = all_split && plan_fits_split(s.second);
     }
-    pl = PlanList{};
-    pl.n = uint32_t(specs.size());
+    PlanList &pl = cp.l;
+    MmaList &ml = cp.m;
+    pl.n = ml.n = uint32_t(specs.size());
     pl.mont = all ? 1 : 0;
+    for (const auto &s : specs) cp.mma = cp.mma || s.second.src_mod.size() > 1;
+    cp.mma = cp.mma && specs.size() <= kMmaPlans;
+    for (size_t i = 0; i < specs.size() && cp.mma; i++) {
+        const MmaRef r = get_mma_plan(c, specs[i].first, specs[i].second);
+        ml.img[i] = r.p;
+        ml.head[i] = r.head;
+        ml.counts[i] = r.counts;
+        cp.mma = r.p != nullptr;
+        if (cp.mma) ml.p[i] = get_plan(c, specs[i].first, specs[i].second).p;
+        if (cp.mma && !ml.p[i]) return CATFHE_ENOMEM;
+    }
     pl.split = all && all_split ? 1 : 0;
     for (size_t i = 0; i < specs.size(); i++) {
         PlanSpec sp = specs[i].second;
@@ -142,7 +156,7 @@ static int modup(Context &c, const uint64_t *d2c, size_t d2_item, uint64_t *ext,
                                (own_too ? "/own" : ""),
                            sp);
     }
-    PlanList pl;
+    ConvPlans pl{};
     TRY(make_list(c, specs, pl));
     const size_t n = c.n;
     return launch_conv(c, pl, d2c, d2_item, 0, ext, size_t(beta) * M * n, size_t(M) * n, count, s);
@@ -270,7 +284,7 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint3
         for (int d = 0; d < Kd; d++) sp.pre.push_back(h_invmod(c.t % sp.src_mod[d], sp.src_mod[d]));
         for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
     }
-    PlanList pl;
+    ConvPlans pl{};
     TRY(make_list(c, {{"moddown/" + std::to_string(level) + (fused ? "/f" : ""), sp}}, pl));
     TRY(launch_conv(c, pl, y, size_t(M) * n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
     // D^-1 mod q_i, D = P (fused: P q_{l-1})
@@ -499,7 +513,7 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
             sp.dst_mod.push_back(c.mod(i < level ? i : c.pb(i - level)));
             sp.dst_off.push_back(uint32_t(i));
         }
-        PlanList pl;
+        ConvPlans pl{};
         TRY(make_list(c, {{"bfv_lift/" + std::to_string(level), sp}}, pl));
         // items: (ct, poly) for a then for b
         TRY(launch_conv(c, pl, a, size_t(level) * n, 0, k.xin, size_t(kb) * n, 0, 2 * count, s));
@@ -838,7 +852,7 @@ int op_rescale(Context &c, const uint64_t *a, uint64_t *out, uint32_t level, uin
         sp.pre.push_back(h_invmod(c.t % c.mod(lvl - 1), c.mod(lvl - 1)));
         for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
     }
-    PlanList pl;
+    ConvPlans pl{};
     TRY(make_list(c, {{"rescale/" + std::to_string(lvl), sp}}, pl));
     TRY(launch_conv(c, pl, last, n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
     // NTT of the lift, its last pass writing (a - lift) q_{l-1}^-1 to out
@@ -1405,7 +1419,7 @@ static int decrypt_device(Context &c, const Keys &k, const uint64_t *ct, uint32_
             sp.post.push_back((c.t - h_invmod(qt, c.t)) % c.t);
         }
     }
-    PlanList pl;
+    ConvPlans pl{};
     TRY(make_list(c, {{key, sp}}, pl));
     return launch_conv(c, pl, x, 0, 0, reinterpret_cast<uint64_t *>(res), 0, 0, 1, s);
 }
