@@ -153,6 +153,7 @@ void ctx_free(Context &c) {
     cudaFree(c.d_twf);
     cudaFree(c.d_twi);
     for (auto &kv : c.plans) cudaFree(kv.second);
+    for (auto &kv : c.lifts) cudaFree(kv.second);
     for (auto &kv : c.mma_plans) cudaFree(const_cast<uint64_t *>(kv.second.p));
     cudaFree(c.scratch.ptr);
     c.plans.clear();
@@ -375,6 +376,38 @@ MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec) {
         ref.counts = img[1];
     }
     return c.mma_plans[key] = ref;
+}
+
+LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post) {
+    LiftEntry e{};
+    e.m = m;
+    e.half = (m - 1) / 2;
+    e.pre = pre % m;
+    e.pre_s = h_shoup(e.pre, m);
+    e.post = post % p;
+    e.post_s = h_shoup(e.post, p);
+    if (e.pre != 1) e.flags |= kLiftPre;
+    if (e.post != 1)
+        e.flags |= kLiftPost;
+    else if ((m - 1) / 4 >= p)  // m > 4p
+        e.flags |= kLiftReduce;
+    if (e.flags & (kLiftPost | kLiftReduce))
+        e.cst = (p - h_mulmod(m % p, e.post, p)) % p;
+    else
+        e.cst = (m + p - 1) / p * p - m;
+    return e;
+}
+
+const LiftEntry *upload_lifts(Context &c, const std::string &key,
+                              const std::vector<LiftEntry> &table) {
+    LiftEntry *dev = nullptr;
+    const size_t bytes = table.size() * sizeof(LiftEntry);
+    if (cudaMalloc(&dev, bytes) != cudaSuccess) return nullptr;
+    if (cudaMemcpy(dev, table.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaFree(dev);
+        return nullptr;
+    }
+    return c.lifts[key] = dev;
 }
 
 PlanRef get_plan(Context &c, const std::string &key, const PlanSpec &spec) {

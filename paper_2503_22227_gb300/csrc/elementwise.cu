@@ -360,7 +360,8 @@ int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s)
 
 // ------------------------------------------------------------------ ModDown combine
 
-// out_p[i] = (y_p[i] - lift_p[i]) * D^-1 (+ add_p[i]), coefficient form; with
+// out_p[i] = (y_p[i] - lift_p[i]) * D^-1 (+ add_p[i]), coefficient form (the
+// lift in [0, 4q), or formed here from the one special limb); with
 // a Galois element g the coefficient at x goes to x g mod 2N, negated past N
 // (one scattered store per word instead of permuted copies of the inputs).
 __global__ void __launch_bounds__(256)
@@ -369,10 +370,12 @@ k_combine(const CombineArgs A, const DevMod *__restrict__ mods, uint32_t log_n) 
     const size_t x = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const uint32_t i = blockIdx.y % A.lo, p = blockIdx.y / A.lo, item = blockIdx.z;
     if (x >= n) return;
-    const uint64_t q = mods[A.prime[i]].q;
-    const uint64_t y = A.y[item * A.y_item + p * A.y_poly + size_t(i) * n + x];
-    const uint64_t l = A.lift[item * A.lift_item + p * A.lift_poly + size_t(i) * n + x];
-    uint64_t r = shoup(y + q - l, A.dinv[i], A.dinv_s[i], q);
+    const DevMod m = mods[A.prime[i]];
+    const uint64_t q = m.q;
+    const uint64_t *yp = A.y + item * A.y_item + p * A.y_poly + x;
+    const uint64_t l = A.lift ? A.lift[item * A.lift_item + p * A.lift_poly + size_t(i) * n + x]
+                              : lift_word(yp[A.y_last], A.lifts[i], m);
+    uint64_t r = shoup(yp[size_t(i) * n] + 4 * q - l, A.dinv[i], A.dinv_s[i], q);
     if (A.add && p < A.add_polys)
         r = add_mod(r, A.add[item * A.add_item + p * A.add_poly + size_t(i) * n + x], q);
     size_t to = x;

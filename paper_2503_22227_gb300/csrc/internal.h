@@ -153,6 +153,23 @@ inline uint32_t mma_targets(uint64_t counts) {
 // below 2^22).
 std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n);
 
+// A centred lift from one source modulus m to a target p, for the kernels that
+// lift as they load (one entry per position of a launch's map): y = a pre mod
+// m, x = y post (+ cst when y > half) mod p, unreduced (below 4p).
+struct LiftEntry {
+    uint64_t m, half;       // source modulus, (m - 1) / 2
+    uint64_t pre, pre_s;    // kLiftPre: factor mod m (Shoup pair)
+    uint64_t post, post_s;  // kLiftPost: factor mod p (Shoup pair)
+    uint64_t cst;           // -m post mod p (without kLiftPost and kLiftReduce: 4p - m or less)
+    uint64_t flags;
+};
+constexpr uint64_t kLiftPre = 1, kLiftPost = 2, kLiftReduce = 4;
+// The entry for source m, target p and factors pre, post (1: none).
+LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post);
+// Device copy of a lift table (null: no memory), kept under key.
+const LiftEntry *upload_lifts(Context &c, const std::string &key,
+                              const std::vector<LiftEntry> &table);
+
 // Up to this many plans run in one launch (grid.z).
 struct PlanList {
     const uint64_t *p[64];
@@ -203,6 +220,7 @@ struct Context {
     std::map<std::string, uint64_t *> plans;     // device copies of packed plans
     std::map<std::string, uint32_t> plan_sizes;  // words
     std::map<std::string, MmaRef> mma_plans;     // tensor-core images (device)
+    std::map<std::string, LiftEntry *> lifts;    // lift tables (device)
     Scratch scratch;
     int device = 0;
     int sms = 0;  // the device's SM count
@@ -275,6 +293,13 @@ int launch_ntt_fwd_lazy(const Context &c, const uint64_t *src, uint64_t *dst, co
                         uint32_t n_limbs, cudaStream_t s);
 int launch_ntt_fwd_combine(const Context &c, uint64_t *lift, const LimbMap &map, uint32_t n_limbs,
                            const NttEpilogue &epi, cudaStream_t s);
+// The last two with their input lifted from another modulus as it is loaded:
+// map entry r's source words (any limb, at src) go through lifts[r].
+int launch_ntt_lift(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
+                         uint32_t n_limbs, const LiftEntry *lifts, bool lazy, cudaStream_t s);
+int launch_ntt_lift_combine(const Context &c, const uint64_t *src, uint64_t *lift,
+                            const LimbMap &map, uint32_t n_limbs, const LiftEntry *lifts,
+                            const NttEpilogue &epi, cudaStream_t s);
 
 // Launch size classes of the NTT schedule choice: up to 64 limbs in one
 // launch (about one ciphertext), up to 256, more.
@@ -353,7 +378,10 @@ int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s);
 
 struct CombineArgs {
     const uint64_t *y;         // [count][2][.][N] at y_off positions
-    const uint64_t *lift;      // [count][2][lo][N]
+    const uint64_t *lift;      // [count][2][lo][N], or null: lifted here from the one limb at
+                               // y_last of each polynomial of y by lifts[i]
+    const LiftEntry *lifts;
+    size_t y_last;
     const uint64_t *add;       // [count][add_polys][lo][N] (strides below) or null
     uint32_t add_polys;        // polynomials that have an addend (1 or 2)
     uint32_t galois;           // X -> X^galois on the result (coefficient form); 0: none

@@ -27,7 +27,7 @@ namespace catfhe {
 #define NTT_DECL(LN)                                                                          \
     int ntt_fwd_n##LN(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map, \
                       uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy,      \
-                      int sched);                                                              \
+                      int sched, const LiftEntry *lifts);                                      \
     int ntt_inv_n##LN(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map, \
                       uint32_t n_limbs, cudaStream_t s, int sched);
 NTT_DECL(12) NTT_DECL(13) NTT_DECL(14) NTT_DECL(15) NTT_DECL(16)
@@ -51,15 +51,16 @@ void ntt_schedule_shape(int log_n, int sched, int shape[4]) {
 }
 
 static int fwd_dispatch(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
-                        uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy) {
+                        uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy,
+                        const LiftEntry *lifts = nullptr) {
     if (n_limbs == 0) return CATFHE_OK;
     const int sched = c.ntt_sched[ntt_class(n_limbs)];
     switch (c.log_n) {
-        case 12: return ntt_fwd_n12(c, src, dst, map, n_limbs, s, epi, lazy, sched);
-        case 13: return ntt_fwd_n13(c, src, dst, map, n_limbs, s, epi, lazy, sched);
-        case 14: return ntt_fwd_n14(c, src, dst, map, n_limbs, s, epi, lazy, sched);
-        case 15: return ntt_fwd_n15(c, src, dst, map, n_limbs, s, epi, lazy, sched);
-        case 16: return ntt_fwd_n16(c, src, dst, map, n_limbs, s, epi, lazy, sched);
+        case 12: return ntt_fwd_n12(c, src, dst, map, n_limbs, s, epi, lazy, sched, lifts);
+        case 13: return ntt_fwd_n13(c, src, dst, map, n_limbs, s, epi, lazy, sched, lifts);
+        case 14: return ntt_fwd_n14(c, src, dst, map, n_limbs, s, epi, lazy, sched, lifts);
+        case 15: return ntt_fwd_n15(c, src, dst, map, n_limbs, s, epi, lazy, sched, lifts);
+        case 16: return ntt_fwd_n16(c, src, dst, map, n_limbs, s, epi, lazy, sched, lifts);
         default: return CATFHE_EINVAL;
     }
 }
@@ -77,6 +78,17 @@ int launch_ntt_fwd_lazy(const Context &c, const uint64_t *src, uint64_t *dst, co
 int launch_ntt_fwd_combine(const Context &c, uint64_t *lift, const LimbMap &map, uint32_t n_limbs,
                            const NttEpilogue &epi, cudaStream_t s) {
     return fwd_dispatch(c, lift, lift, map, n_limbs, s, &epi, false);
+}
+
+int launch_ntt_lift(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
+                    uint32_t n_limbs, const LiftEntry *lifts, bool lazy, cudaStream_t s) {
+    return fwd_dispatch(c, src, dst, map, n_limbs, s, nullptr, lazy, lifts);
+}
+
+int launch_ntt_lift_combine(const Context &c, const uint64_t *src, uint64_t *lift,
+                            const LimbMap &map, uint32_t n_limbs, const LiftEntry *lifts,
+                            const NttEpilogue &epi, cudaStream_t s) {
+    return fwd_dispatch(c, src, lift, map, n_limbs, s, &epi, false, lifts);
 }
 
 int launch_ntt_inv(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,

@@ -43,17 +43,9 @@ __device__ __forceinline__ uint64_t reduce_any(uint64_t x, const DevMod &m) {
     return csub(shoup_lazy(x, 1, m.one_s, m.q), m.q);
 }
 
-// Any word below 2^64 -> [0, q) for q > 2^33, m64 = floor(2^64 / q) < 2^31:
-// est = floor(hi32(x) m64 / 2^32) is at most floor(x/q) and at most 2 below
-// it (x - hi32(x) 2^32 < 2^32 < q, m64 is short of 2^64/q by less than 1,
-// which hi32(x) / 2^32 < 1 turns into less than 1, and the floor drops less
-// than 1), so x - est q lies in [0, 3q).  Three 32-bit multiplies (one
-// high, one wide, one low) instead of the 64-bit high product of the Shoup
-// form: measured on the 384-limb forward row pass, 174 -> 166 us.
+// Any word below 2^64 -> [0, q) for q > 2^33.
 __device__ __forceinline__ uint64_t reduce_fast(uint64_t x, uint64_t q, uint32_t m64) {
-    const uint32_t est = __umulhi(uint32_t(x >> 32), m64);
-    const uint64_t r = x - uint64_t(est) * q;
-    return csub(csub(r, 2 * q), q);
+    return csub(csub(reduce_lazy3(x, q, m64), 2 * q), q);
 }
 
 // The row pass's final reduction of a word of the forward transform: below
@@ -171,10 +163,17 @@ __device__ __forceinline__ void fwd_cols_body(uint64_t (&x)[1 << LOGE], uint64_t
 // is the one these kernels saturate.  NT threads per CTA: 256, or 128 for
 // E = 32 words per thread (whose exchange buffer would not fit 48 KB of
 // static shared memory at 256 threads).
-template <int LOGN, int LOGR, int LOGE, int NT, int MINB>
+// LIFT: the words loaded are residues of another modulus, lifted here (lifts,
+// one entry per position of the map): a digit of one prime, a rescale or a
+// ModDown by one prime then need no conversion pass, which would write every
+// target limb for this pass to read back (rescale of 3 ciphertexts at
+// N = 2^15, l = 13: 42.8 -> 35.8 us; BGV batch of 16 at N = 2^14 with eight
+// one-prime digits: 349 -> 310 us).
+template <int LOGN, int LOGR, int LOGE, int NT, int MINB, bool LIFT>
 __global__ void __launch_bounds__(NT, MINB)
 k_ntt_fwd_cols(const uint64_t *src, uint64_t *dst, const LimbMap map,
-               const DevMod *__restrict__ mods, const ulonglong2 *__restrict__ tw) {
+               const DevMod *__restrict__ mods, const ulonglong2 *__restrict__ tw,
+               const LiftEntry *__restrict__ lifts) {
     grid_dep_wait();
     constexpr int R = 1 << LOGR, E = 1 << LOGE, T = R / E, CW = NT / T;
     __shared__ uint64_t sm[R * CW];
@@ -201,6 +200,17 @@ k_ntt_fwd_cols(const uint64_t *src, uint64_t *dst, const LimbMap map,
     // 278 us, inverse 298 -> 294 us for 384 limbs)
     __shared__ ulonglong2 stw[R];
     for (int i = threadIdx.x; i < R; i += NT) stw[i] = wg[i];
+    if (LIFT) {
+        const LiftEntry e = lifts[r];
+        const DevMod m = mods[p];
+        if (e.flags == 0) {
+#pragma unroll
+            for (int v = 0; v < E; v++) x[v] += x[v] > e.half ? e.cst : 0;
+        } else {
+#pragma unroll
+            for (int v = 0; v < E; v++) x[v] = lift_word(x[v], e, m);
+        }
+    }
     __syncthreads();
     const ulonglong2 *w = stw;
     // q < 2^57: no conditional subtractions; words leave below 4q + 4 LOGR q
@@ -577,11 +587,13 @@ k_ntt_inv_cols(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
 // or the ModDown combine epilogue when epi is given.
 template <int LN, int R1, int E1, int T1, int B1, int R2, int E2, int T2, int B2>
 static int run_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
-                   uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy) {
+                   uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy,
+                   const LiftEntry *lifts) {
     constexpr size_t N = size_t(1) << LN;
     const dim3 g1(unsigned((N >> R1) / (T1 / ((1 << R1) >> E1))), n_limbs);
-    launch_pdl(k_ntt_fwd_cols<LN, R1, E1, T1, B1>, g1, dim3(T1), 0, s, src, dst, map, c.d_mods,
-               c.d_twf);
+    launch_pdl(lifts ? k_ntt_fwd_cols<LN, R1, E1, T1, B1, true>
+                     : k_ntt_fwd_cols<LN, R1, E1, T1, B1, false>,
+               g1, dim3(T1), 0, s, src, dst, map, c.d_mods, c.d_twf, lifts);
     const dim3 g2(unsigned((N >> R2) / (T2 / ((1 << R2) >> E2))), n_limbs);
     if (epi) {
         // every caller's y is a workspace or ciphertext buffer, refused at the

@@ -9,12 +9,13 @@ namespace catfhe {
 
 int NTT_CAT(ntt_fwd_n, NTT_LOGN)(const Context &c, const uint64_t *src, uint64_t *dst,
                                  const LimbMap &map, uint32_t n_limbs, cudaStream_t s,
-                                 const NttEpilogue *epi, bool lazy, int sched) {
+                                 const NttEpilogue *epi, bool lazy, int sched,
+                                 const LiftEntry *lifts) {
 #define FWD(LN, S, A, B, TA, BA, C, D, TC, BC)                                              \
     if constexpr (LN == NTT_LOGN) {                                                        \
         if (sched == S)                                                                    \
             return run_fwd<LN, A, B, TA, BA, C, D, TC, BC>(c, src, dst, map, n_limbs, s, epi, \
-                                                           lazy);                          \
+                                                           lazy, lifts);                          \
     }
     NTT_SCHEDULES(FWD)
 #undef FWD

@@ -100,6 +100,25 @@ static int make_list(Context &c, const std::vector<std::pair<std::string, PlanSp
     return CATFHE_OK;
 }
 
+// The lift table kept under key, built by make() on first use.
+template <class F>
+static const LiftEntry *get_lifts(Context &c, const std::string &key, F make) {
+    const auto it = c.lifts.find(key);
+    return it != c.lifts.end() ? it->second : upload_lifts(c, key, make());
+}
+
+// The entries of a ModDown or rescale by the one prime at index `from`, for
+// both polynomials' targets q_0 .. q_{lo-1}.
+static std::vector<LiftEntry> division_lifts(const Context &c, int from, int lo) {
+    const uint64_t m = c.mod(from);
+    const bool bgv = c.scheme == CATFHE_BGV;
+    std::vector<LiftEntry> t;
+    for (int p = 0; p < 2; p++)
+        for (int i = 0; i < lo; i++)
+            t.push_back(lift_entry(m, c.mod(i), bgv ? h_invmod(c.t % m, m) : 1, bgv ? c.t : 1));
+    return t;
+}
+
 static LimbMap map_identity(uint32_t limbs, uint32_t first_prime = 0) {
     LimbMap m{};
     m.period = limbs;
@@ -180,10 +199,13 @@ static bool ext_lazy(const Context &c, int level) {
     return true;
 }
 
-// NTT of the lifted limbs of ext (all positions if own_too).
-static int ntt_ext(Context &c, uint64_t *ext, uint32_t count, int level, bool own_too,
-                   cudaStream_t s) {
+// ModUp and the NTT of the lifted limbs (all positions if own_too).  Digits of
+// one prime are lifted by the transform's first pass as it loads; wider ones
+// are converted first.
+static int modup_ntt(Context &c, const uint64_t *d2c, size_t d2_item, uint64_t *ext, uint32_t count,
+                     int level, bool own_too, cudaStream_t s) {
     const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
+    const bool one = c.alpha == 1 && d2_item % c.n == 0;
     LimbMap m{};
     uint32_t e = 0;
     for (int j = 0; j < beta; j++) {
@@ -191,15 +213,30 @@ static int ntt_ext(Context &c, uint64_t *ext, uint32_t count, int level, bool ow
         for (int i = 0; i < M; i++) {
             if (!own_too && i >= lo && i < hi) continue;
             if (e >= uint32_t(kMapMax)) return CATFHE_EINVAL;
-            m.src_off[e] = m.dst_off[e] = uint16_t(j * M + i);
+            m.dst_off[e] = uint16_t(j * M + i);
+            m.src_off[e] = one ? uint16_t(j) : m.dst_off[e];
             m.prime[e] = uint8_t(ext_prime(c, level, i));
             e++;
         }
     }
     m.period = e;
-    m.src_stride = m.dst_stride = uint32_t(beta * M);
-    return ext_lazy(c, level) ? launch_ntt_fwd_lazy(c, ext, ext, m, e * count, s)
-                              : launch_ntt_fwd(c, ext, ext, m, e * count, s);
+    m.dst_stride = uint32_t(beta * M);
+    m.src_stride = one ? uint32_t(d2_item / c.n) : m.dst_stride;
+    const bool lazy = ext_lazy(c, level);
+    if (one) {
+        const LiftEntry *lifts =
+            get_lifts(c, "modup/" + std::to_string(level) + (own_too ? "/own" : ""), [&] {
+                std::vector<LiftEntry> t;
+                for (uint32_t r = 0; r < e; r++)
+                    t.push_back(lift_entry(c.mod(m.src_off[r]), c.mod(m.prime[r]), 1, 1));
+                return t;
+            });
+        if (!lifts) return CATFHE_ENOMEM;
+        return launch_ntt_lift(c, d2c, ext, m, e * count, lifts, lazy, s);
+    }
+    TRY(modup(c, d2c, d2_item, ext, count, level, own_too, s));
+    return lazy ? launch_ntt_fwd_lazy(c, ext, ext, m, e * count, s)
+                : launch_ntt_fwd(c, ext, ext, m, e * count, s);
 }
 
 // own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
@@ -270,23 +307,31 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint3
             }
         TRY(launch_ntt_inv(c, y, y, m, m.period * count, s));
     }
-    PlanSpec sp;
-    sp.lazy = ntt_form;  // NTT schemes transform the lift before the combine
-    for (int d = 0; d < Kd; d++) {
-        sp.src_mod.push_back(c.mod(ext_prime(c, level, dpos[d])));
-        sp.src_off.push_back(uint32_t(dpos[d]));
+    const std::string key = "moddown/" + std::to_string(level) + (fused ? "/f" : "");
+    const LiftEntry *lifts = nullptr;
+    if (Kd == 1) {  // lifted by the next kernel as it loads
+        lifts = get_lifts(c, key, [&] { return division_lifts(c, ext_prime(c, level, dpos[0]), lo); });
+        if (!lifts) return CATFHE_ENOMEM;
+    } else {
+        PlanSpec sp;
+        sp.lazy = ntt_form;  // NTT schemes transform the lift before the combine
+        for (int d = 0; d < Kd; d++) {
+            sp.src_mod.push_back(c.mod(ext_prime(c, level, dpos[d])));
+            sp.src_off.push_back(uint32_t(dpos[d]));
+        }
+        for (int i = 0; i < lo; i++) {
+            sp.dst_mod.push_back(c.mod(i));
+            sp.dst_off.push_back(uint32_t(i));
+        }
+        if (c.scheme == CATFHE_BGV) {
+            for (int d = 0; d < Kd; d++)
+                sp.pre.push_back(h_invmod(c.t % sp.src_mod[d], sp.src_mod[d]));
+            for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
+        }
+        ConvPlans pl{};
+        TRY(make_list(c, {{key, sp}}, pl));
+        TRY(launch_conv(c, pl, y, size_t(M) * n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
     }
-    for (int i = 0; i < lo; i++) {
-        sp.dst_mod.push_back(c.mod(i));
-        sp.dst_off.push_back(uint32_t(i));
-    }
-    if (c.scheme == CATFHE_BGV) {
-        for (int d = 0; d < Kd; d++) sp.pre.push_back(h_invmod(c.t % sp.src_mod[d], sp.src_mod[d]));
-        for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
-    }
-    ConvPlans pl{};
-    TRY(make_list(c, {{"moddown/" + std::to_string(level) + (fused ? "/f" : ""), sp}}, pl));
-    TRY(launch_conv(c, pl, y, size_t(M) * n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
     // D^-1 mod q_i, D = P (fused: P q_{l-1})
     std::vector<uint64_t> dinv(lo), dinv_s(lo);
     for (int i = 0; i < lo; i++) {
@@ -306,7 +351,8 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint3
             for (uint32_t i = 0; i < gth->n; i++) e.gout[i] = gth->out[i];
         }
         m.period = uint32_t(2 * lo);
-        m.src_stride = m.dst_stride = uint32_t(2 * lo);
+        m.dst_stride = uint32_t(2 * lo);
+        m.src_stride = lifts ? uint32_t(2 * M) : uint32_t(2 * lo);
         e.y = y;
         e.out = out;
         e.status = c.d_status;
@@ -317,18 +363,22 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint3
         for (int p = 0; p < 2; p++)
             for (int i = 0; i < lo; i++) {
                 const int r = p * lo + i;
-                m.src_off[r] = m.dst_off[r] = uint16_t(r);
+                m.dst_off[r] = uint16_t(r);
+                m.src_off[r] = lifts ? uint16_t(p * M + dpos[0]) : uint16_t(r);
                 m.prime[r] = uint8_t(i);
                 e.y_off[r] = uint16_t(p * M + i);
                 e.out_off[r] = uint16_t(r);
                 e.dinv[r] = dinv[i];
                 e.dinv_s[r] = dinv_s[i];
             }
-        return launch_ntt_fwd_combine(c, lift, m, uint32_t(2 * lo) * count, e, s);
+        return lifts ? launch_ntt_lift_combine(c, y, lift, m, uint32_t(2 * lo) * count, lifts, e, s)
+                     : launch_ntt_fwd_combine(c, lift, m, uint32_t(2 * lo) * count, e, s);
     }
     CombineArgs a{};
     a.y = y;
-    a.lift = lift;
+    a.lift = lifts ? nullptr : lift;
+    a.lifts = lifts;
+    a.y_last = size_t(dpos[0]) * n;
     a.add = add;
     a.add_polys = add_polys;
     a.galois = uint32_t(g);
@@ -487,8 +537,7 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(launch_tensor(c, t, count, s));
     LimbMap m = map_identity(uint32_t(level));
     TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(level) * count, s));
-    TRY(modup(c, k.d2c, size_t(level) * n, k.ext, count, level, false, s));
-    TRY(ntt_ext(c, k.ext, count, level, false, s));
+    TRY(modup_ntt(c, k.d2c, size_t(level) * n, k.ext, count, level, false, s));
     TRY(inner_product(c, k.ext, k.d2, rlk, k.d0, k.d1, size_t(level) * n, k.y, count, level, s));
     return moddown(c, k.y, k.lift, out, count, level, fused, s, 0, gth);
 }
@@ -578,8 +627,7 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
     }
     // 4. relinearise d2' (coefficient form) and add (d0', d1')
     const uint64_t *d2 = k.dq + size_t(2) * level * n;
-    TRY(modup(c, d2, size_t(3) * level * n, k.ext, count, level, true, s));
-    TRY(ntt_ext(c, k.ext, count, level, true, s));
+    TRY(modup_ntt(c, d2, size_t(3) * level * n, k.ext, count, level, true, s));
     TRY(inner_product(c, k.ext, nullptr, rlk, nullptr, nullptr, 0, k.y, count, level, s));
     {
         const int M = level + c.K;
@@ -702,8 +750,7 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
             for (uint32_t i = 0; i < gth->n; i++) m.gsrc[i] = gth->a[i];
         }
         TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(lvl) * count, s));
-        TRY(modup(c, k.d2c, half, k.ext, count, lvl, false, s));
-        TRY(ntt_ext(c, k.ext, count, lvl, false, s));
+        TRY(modup_ntt(c, k.d2c, half, k.ext, count, lvl, false, s));
         TRY(inner_product(c, k.ext, a + half, gk, a, nullptr, item, k.y, count, lvl, s, gth));
         return moddown(c, k.y, k.lift, out, count, lvl, false, s, g, gth);
     }
@@ -717,8 +764,7 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
                               uint32_t(2 * lvl) * count, s));
         add = k.add;
     }
-    TRY(modup(c, a + half, item, k.ext, count, lvl, true, s));
-    TRY(ntt_ext(c, k.ext, count, lvl, true, s));
+    TRY(modup_ntt(c, a + half, item, k.ext, count, lvl, true, s));
     TRY(inner_product(c, k.ext, nullptr, gk, nullptr, nullptr, 0, k.y, count, lvl, s));
     {
         const int M = lvl + c.K;
@@ -789,8 +835,7 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     // a1 (NTT form) -> coefficient form -> lifted digits in NTT form, once
     const size_t item = size_t(2) * lvl * n, half = size_t(lvl) * n;
     TRY(launch_ntt_inv(c, a, k.d2c, map_second(lvl), uint32_t(lvl) * count, s));
-    TRY(modup(c, k.d2c, half, ext0, count, lvl, false, s));
-    TRY(ntt_ext(c, ext0, count, lvl, false, s));
+    TRY(modup_ntt(c, k.d2c, half, ext0, count, lvl, false, s));
     auto one = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
         TRY(inner_product(c, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, lvl, st));
         return moddown(c, kb.y, kb.lift, out + size_t(r) * count * item, count, lvl, false, st,
@@ -840,26 +885,16 @@ int op_rescale(Context &c, const uint64_t *a, uint64_t *out, uint32_t level, uin
         m.prime[p] = uint8_t(lvl - 1);
     }
     TRY(launch_ntt_inv(c, a, last, m, 2 * count, s));
-    PlanSpec sp;
-    sp.lazy = true;  // NTT'd before the combine
-    sp.src_mod.push_back(c.mod(lvl - 1));
-    sp.src_off.push_back(0);
-    for (int i = 0; i < lo; i++) {
-        sp.dst_mod.push_back(c.mod(i));
-        sp.dst_off.push_back(uint32_t(i));
-    }
-    if (c.scheme == CATFHE_BGV) {
-        sp.pre.push_back(h_invmod(c.t % c.mod(lvl - 1), c.mod(lvl - 1)));
-        for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
-    }
-    ConvPlans pl{};
-    TRY(make_list(c, {{"rescale/" + std::to_string(lvl), sp}}, pl));
-    TRY(launch_conv(c, pl, last, n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
-    // NTT of the lift, its last pass writing (a - lift) q_{l-1}^-1 to out
+    const LiftEntry *lifts = get_lifts(c, "rescale/" + std::to_string(lvl),
+                                       [&] { return division_lifts(c, lvl - 1, lo); });
+    if (!lifts) return CATFHE_ENOMEM;
+    // NTT of the lift (lifted as it loads), its last pass writing
+    // (a - lift) q_{l-1}^-1 to out
     LimbMap m2{};
     NttEpilogue e{};
     m2.period = uint32_t(2 * lo);
-    m2.src_stride = m2.dst_stride = uint32_t(2 * lo);
+    m2.src_stride = 2;
+    m2.dst_stride = uint32_t(2 * lo);
     e.y = a;
     e.out = out;
     e.status = c.d_status;
@@ -868,14 +903,15 @@ int op_rescale(Context &c, const uint64_t *a, uint64_t *out, uint32_t level, uin
     for (int p = 0; p < 2; p++)
         for (int i = 0; i < lo; i++) {
             const int r = p * lo + i;
-            m2.src_off[r] = m2.dst_off[r] = uint16_t(r);
+            m2.src_off[r] = uint16_t(p);
+            m2.dst_off[r] = uint16_t(r);
             m2.prime[r] = uint8_t(i);
             e.y_off[r] = uint16_t(p * lvl + i);
             e.out_off[r] = uint16_t(r);
             e.dinv[r] = h_invmod(c.mod(lvl - 1) % c.mod(i), c.mod(i));
             e.dinv_s[r] = h_shoup(e.dinv[r], c.mod(i));
         }
-    return launch_ntt_fwd_combine(c, lift, m2, uint32_t(2 * lo) * count, e, s);
+    return launch_ntt_lift_combine(c, last, lift, m2, uint32_t(2 * lo) * count, lifts, e, s);
 }
 
 int op_add(Context &c, const uint64_t *a, const uint64_t *b, uint64_t *out, uint32_t level,
