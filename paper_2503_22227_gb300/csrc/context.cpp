@@ -359,11 +359,12 @@ PlanRef get_plan_extra(Context &c, const std::string &key0, const PlanSpec &spec
     return upload_plan(c, key, build_plan(spec), extra);
 }
 
-MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec) {
+MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec,
+                    uint64_t target_unit) {
     auto it = c.mma_plans.find(key);
     if (it != c.mma_plans.end()) return it->second;
     MmaRef ref;
-    const std::vector<uint64_t> img = build_mma_plan(spec, c.n);
+    const std::vector<uint64_t> img = build_mma_plan(spec, c.n, target_unit);
     if (!img.empty()) {
         uint64_t *dev = nullptr;
         if (cudaMalloc(&dev, img.size() * 8) != cudaSuccess) return ref;

@@ -113,7 +113,9 @@ struct MmaRef {
     const uint64_t *p = nullptr;  // device image, null when the plan has none
     uint64_t head = 0, counts = 0;
 };
-MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec);
+// target_unit: what a target's offset counts (N: limbs; 1: an index).
+MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec,
+                    uint64_t target_unit);
 PlanRef get_plan_extra(Context &c, const std::string &key, const PlanSpec &spec,
                        const std::vector<uint64_t> &extra);
 
@@ -151,7 +153,7 @@ inline uint32_t mma_targets(uint64_t counts) {
 // Empty when the conversion does not fit (K > 15, a source modulus outside
 // (2^32, 2^60), a target outside (2^40, 2^60), or a column's sums not provably
 // below 2^22).
-std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n);
+std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t target_unit);
 
 // A centred lift from one source modulus m to a target p, for the kernels that
 // lift as they load (one entry per position of a launch's map): y = a pre mod
@@ -328,6 +330,16 @@ int launch_bfv_scale_round(const Context &c, const uint64_t *q_to_b, uint32_t q_
                            const uint64_t *b_to_q, uint32_t b_to_q_words, const uint64_t *src,
                            size_t src_item, uint64_t *dst, size_t dst_item, uint32_t items,
                            cudaStream_t s);
+
+// The same on the tensor cores.  a lifts [t x]_Q (pre t) to Q^-1 (B/b_j)^-1
+// times it mod b_j, its target slots' word 4 the index j; b has the sources b_j
+// at their limbs of x with pre t Q^-1, and the targets q_i.  a_exact, b_exact:
+// Montgomery plans of the same sources, b's with pre B/b_j.
+bool bfv_round_mma_fits(const MmaRef &a, const MmaRef &b);
+int launch_bfv_round_mma(const Context &c, const MmaRef &a, const uint64_t *a_exact,
+                         const MmaRef &b, const uint64_t *b_exact, const uint64_t *src,
+                         size_t src_item, uint64_t *dst, size_t dst_item, uint32_t items,
+                         cudaStream_t s);
 
 // Element-wise kernels (elementwise.cu)
 // Per-ciphertext base pointers of an operation whose ciphertexts are not

@@ -53,7 +53,7 @@ static bool balanced_digits(uint64_t w, uint64_t p, int D, int out[6]) {
     return true;
 }
 
-std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n) {
+std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t target_unit) {
     const uint32_t K = uint32_t(s.src_mod.size()), T = uint32_t(s.dst_mod.size());
     if (K < 1 || K > kMmaMaxK || T < 1 || !plan_fits_mont(s)) return {};
     for (uint64_t m : s.src_mod)
@@ -152,7 +152,7 @@ std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n) {
             const float f[4] = {float(ct), float(cm), float(cl),
                                 float(double(c0) / pd - big * (double(float(cm)) + double(float(cl))))};
             memcpy(o + 2, f, 16);
-            o[4] = s.dst_off[t] * n;
+            o[4] = s.dst_off[t] * target_unit;
         }
     }
     return img;

@@ -75,7 +75,7 @@ static int make_list(Context &c, const std::vector<std::pair<std::string, PlanSp
     for (const auto &s : specs) cp.mma = cp.mma || s.second.src_mod.size() > 1;
     cp.mma = cp.mma && specs.size() <= kMmaPlans;
     for (size_t i = 0; i < specs.size() && cp.mma; i++) {
-        const MmaRef r = get_mma_plan(c, specs[i].first, specs[i].second);
+        const MmaRef r = get_mma_plan(c, specs[i].first, specs[i].second, c.n);
         ml.img[i] = r.p;
         ml.head[i] = r.head;
         ml.counts[i] = r.counts;
@@ -550,7 +550,20 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(key_for(keys, 0, &rlk));
     const size_t n = c.n;
     const int kb = level + c.nb;
-    // 1. centred lift of the 4 input polys from Q_l to Q_l u B
+    // 1. the 4 input polys over Q_l u B in NTT form: the q limbs transformed
+    // straight from the inputs, the b limbs from their centred lift
+    uint64_t *xb = k.xin + size_t(count) * 2 * kb * n;  // b's half of xin
+    LimbMap mb{}, mq{};  // the b limbs of xin; all of them
+    mb.period = uint32_t(c.nb);
+    mq.period = uint32_t(kb);
+    mb.src_stride = mb.dst_stride = mq.src_stride = mq.dst_stride = uint32_t(kb);
+    for (int i = 0; i < kb; i++) {
+        mq.src_off[i] = mq.dst_off[i] = uint16_t(i);
+        mq.prime[i] = uint8_t(i < level ? i : c.pb(i - level));
+        if (i < level) continue;
+        mb.src_off[i - level] = mb.dst_off[i - level] = uint16_t(i);
+        mb.prime[i - level] = mq.prime[i];
+    }
     {
         PlanSpec sp;
         sp.lazy = true;  // NTT'd before the tensor
@@ -558,30 +571,28 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
             sp.src_mod.push_back(c.mod(i));
             sp.src_off.push_back(uint32_t(i));
         }
-        for (int i = 0; i < kb; i++) {
-            sp.dst_mod.push_back(c.mod(i < level ? i : c.pb(i - level)));
-            sp.dst_off.push_back(uint32_t(i));
+        for (int j = 0; j < c.nb; j++) {
+            sp.dst_mod.push_back(c.mod(c.pb(j)));
+            sp.dst_off.push_back(uint32_t(level + j));
         }
         ConvPlans pl{};
         TRY(make_list(c, {{"bfv_lift/" + std::to_string(level), sp}}, pl));
-        // items: (ct, poly) for a then for b
-        TRY(launch_conv(c, pl, a, size_t(level) * n, 0, k.xin, size_t(kb) * n, 0, 2 * count, s));
-        TRY(launch_conv(c, pl, b, size_t(level) * n, 0, k.xin + size_t(count) * 2 * kb * n,
-                        size_t(kb) * n, 0, 2 * count, s));
+        LimbMap in = map_identity(uint32_t(level));
+        in.dst_stride = uint32_t(kb);
+        // items: (ct, poly) of a, then of b
+        for (int h = 0; h < 2; h++) {
+            const uint64_t *src = h ? b : a;
+            uint64_t *dst = h ? xb : k.xin;
+            TRY(launch_conv(c, pl, src, size_t(level) * n, 0, dst, size_t(kb) * n, 0, 2 * count, s));
+            TRY(launch_ntt_fwd(c, src, dst, in, uint32_t(level) * 2 * count, s));
+        }
     }
-    LimbMap mq{};
-    mq.period = uint32_t(kb);
-    mq.src_stride = mq.dst_stride = uint32_t(kb);
-    for (int i = 0; i < kb; i++) {
-        mq.src_off[i] = mq.dst_off[i] = uint16_t(i);
-        mq.prime[i] = uint8_t(i < level ? i : c.pb(i - level));
-    }
-    TRY(launch_ntt_fwd(c, k.xin, k.xin, mq, uint32_t(kb) * 4 * count, s));
+    TRY(launch_ntt_fwd(c, k.xin, k.xin, mb, uint32_t(c.nb) * 4 * count, s));
     // 2. tensor over Q u B
     {
         TensorArgs t{};
         t.a = k.xin;
-        t.b = k.xin + size_t(count) * 2 * kb * n;
+        t.b = xb;
         t.in_item = size_t(2) * kb * n;
         t.d0 = k.tens;
         t.d1 = k.tens + size_t(kb) * n;
@@ -622,7 +633,30 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
         const PlanRef pa = get_plan_extra(c, "bfv_sr_a/" + std::to_string(level), A, tq);
         const PlanRef pb = get_plan(c, "bfv_sr_b/" + std::to_string(level), B);
         if (!pa.p || !pb.p) return CATFHE_ENOMEM;
-        TRY(launch_bfv_scale_round(c, pa.p, pa.words, pb.p, pb.words, k.tens, size_t(kb) * n, k.dq,
+        // the tensor-core form: A's results times (B/b_j)^-1 meet the digits of
+        // b's conversion, whose sources are x_b times t Q^-1
+        const std::string key = "bfv_sr/" + std::to_string(level);
+        PlanSpec Am = A, Bm = B, Be = B;
+        for (int j = 0; j < c.nb && !c.mma_plans.count(key + "/a"); j++) {
+            const uint64_t bj = c.mod(c.pb(j));
+            uint64_t rest = 1;  // B / b_j mod b_j
+            for (int l = 0; l < c.nb; l++)
+                if (l != j) rest = h_mulmod(rest, c.mod(c.pb(l)) % bj, bj);
+            Am.dst_off[size_t(j)] = uint32_t(j);
+            Am.post[size_t(j)] = h_mulmod(A.post[size_t(j)], h_invmod(rest, bj), bj);
+            Bm.src_off[size_t(j)] = uint32_t(level + j);
+            Bm.pre.push_back(tq[2 * size_t(j)]);
+            Be.src_off[size_t(j)] = uint32_t(j);
+            Be.pre.push_back(rest);
+        }
+        const MmaRef ma = get_mma_plan(c, key + "/a", Am, 1), mb2 = get_mma_plan(c, key + "/b", Bm, n);
+        if (bfv_round_mma_fits(ma, mb2)) {
+            const PlanRef pe = get_plan(c, key + "/b/exact", Be);
+            if (!pe.p) return CATFHE_ENOMEM;
+            TRY(launch_bfv_round_mma(c, ma, pa.p, mb2, pe.p, k.tens, size_t(kb) * n, k.dq,
+                                     size_t(level) * n, 3 * count, s));
+        } else
+            TRY(launch_bfv_scale_round(c, pa.p, pa.words, pb.p, pb.words, k.tens, size_t(kb) * n, k.dq,
                                    size_t(level) * n, 3 * count, s));
     }
     // 4. relinearise d2' (coefficient form) and add (d0', d1')

@@ -27,6 +27,9 @@ PRESETS = [
     W.Preset("six_digit_targets", W.CKKS, 12, (45, 51, 60) * 3, (59,) * 5, 2, log_n_max=12),
     W.Preset("bgv", W.BGV, 12, (55,) * 9, (60,) * 4, 2, t=65537, log_n_max=12),
     W.Preset("bfv", W.BFV, 12, (50,) * 6, (60,) * 3, 2, t=65537, log_n_max=12),
+    W.Preset("bfv_12_primes", W.BFV, 12, (50,) * 12, (60,) * 4, 3, t=65537, log_n_max=12),
+    # 61-bit primes: the integer scale-and-round
+    W.Preset("bfv_61", W.BFV, 12, (61,) * 3, (61,), 3, t=65537, log_n_max=12, b_bits=61),
 ]
 
 
