@@ -411,6 +411,16 @@ const LiftEntry *upload_lifts(Context &c, const std::string &key,
     return c.lifts[key] = dev;
 }
 
+const uint64_t *upload_words(Context &c, const std::string &key, const std::vector<uint64_t> &w) {
+    uint64_t *dev = nullptr;
+    if (cudaMalloc(&dev, w.size() * 8) != cudaSuccess) return nullptr;
+    if (cudaMemcpy(dev, w.data(), w.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaFree(dev);
+        return nullptr;
+    }
+    return c.plans[key] = dev;
+}
+
 PlanRef get_plan(Context &c, const std::string &key, const PlanSpec &spec) {
     return get_plan_extra(c, key, spec, {});
 }

@@ -35,6 +35,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include "conv_mma.cuh"
 #include "launch.cuh"
 #include "modarith.cuh"
 
@@ -618,6 +619,65 @@ k_bfv_scale_round(const uint64_t *__restrict__ p_qb, const uint64_t *__restrict_
         const bool gz = mixed_radix_mont<KB>(z, B);
         for (uint32_t t = 0; t < B.T; t++) d[B.dst_off[t] * n + x] = eval_mont<KB>(z, gz, B, t);
     }
+}
+
+// The lift to 64-bit integers (launch_lift_wrap).  With y_i = x_i (M/m_i)^-1
+// mod m_i and v = round(sum y_i / m_i), the value is sum y_i M/m_i - v M mod
+// 2^64: one Shoup product and two 64-bit ones per prime, where mixed radix
+// takes k (k + 1) / 2 (24 primes, N = 2^16: 71 us, here about 6).  v comes from 57-bit
+// fixed-point terms, each short by less than 2; sums too close to a boundary
+// (never a decrypted message, which is far below M/2) compare exact digits.
+__global__ void __launch_bounds__(128)
+k_lift_wrap(const uint64_t *__restrict__ consts, const uint64_t *__restrict__ exact, uint32_t level,
+            const uint64_t *__restrict__ x, uint64_t *__restrict__ out, uint32_t log_n) {
+    grid_dep_wait();
+    const size_t n = size_t(1) << log_n;
+    const size_t j = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    constexpr uint32_t F = 57;
+    uint64_t fr = uint64_t(1) << (F - 1), r = 0;
+#pragma unroll 8
+    for (uint32_t i = 0; i < level; i++) {
+        const uint64_t *k = consts + size_t(i) * 6;
+        const uint64_t m = k[0];
+        const uint64_t y = csub(shoup_lazy(x[i * n + j], k[1], k[2], m), m);
+        fr += mulhi(y << k[4], k[3]);
+        r += y * k[5];
+    }
+    uint64_t v = fr >> F;
+    if ((fr & ((uint64_t(1) << F) - 1)) >= (uint64_t(1) << F) - 2 * level)
+        v = ((fr - (uint64_t(1) << (F - 1))) >> F) + (above_half(exact, x + j, n) ? 1 : 0);
+    out[j] = r - v * consts[size_t(level) * 6];
+}
+
+std::vector<uint64_t> wrap_consts(const std::vector<uint64_t> &mods) {
+    typedef unsigned __int128 u128;
+    std::vector<uint64_t> out;
+    uint64_t M = 1;
+    for (uint64_t m : mods) M *= m;
+    for (size_t i = 0; i < mods.size(); i++) {
+        const uint64_t m = mods[i];
+        uint64_t rest = 1 % m, rest64 = 1;
+        for (size_t l = 0; l < mods.size(); l++) {
+            if (l == i) continue;
+            rest = h_mulmod(rest, mods[l] % m, m);
+            rest64 *= mods[l];
+        }
+        const uint64_t w = h_invmod(rest, m);
+        const int bits = 64 - __builtin_clzll(m);
+        out.insert(out.end(), {m, w, h_shoup(w, m), uint64_t(((u128)1 << (60 + bits)) / m),
+                               uint64_t(61 - bits), rest64});
+    }
+    out.push_back(M);
+    return out;
+}
+
+int launch_lift_wrap(const Context &c, const uint64_t *consts, const uint64_t *exact,
+                     uint32_t level, const uint64_t *x, uint64_t *out, cudaStream_t s) {
+    launch_pdl(k_lift_wrap, dim3(unsigned(c.n / 128)), dim3(128), 0, s, consts, exact, level, x, out,
+               uint32_t(c.log_n));
+    note_launches(1);
+    return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 
 static int pick_kmax(uint32_t k) { return k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32; }

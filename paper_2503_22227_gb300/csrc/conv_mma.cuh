@@ -22,7 +22,7 @@ constexpr uint32_t kFrac = 27;          // fraction bits of sum y_i / m_i
 static __device__ __noinline__ bool above_half(const uint64_t *plan, const uint64_t *s, size_t n) {
     const uint32_t k = uint32_t(plan[0] & 0xffff), T = uint32_t((plan[0] >> 16) & 0xffff);
     const uint64_t *off = plan + 1, *smod = off + k + T, *C = smod + 2 * k + 2 * T, *h = C + k * k;
-    uint64_t a[kMmaMaxK];
+    uint64_t a[kConvMaxK];
     bool gt = false;
     for (uint32_t j = 0; j < k; j++) {
         const uint64_t mj = smod[2 * j];

@@ -8,10 +8,17 @@
 //           j' = (2N - 5^k - 1)/2), then m_i = round(Re(zeta^-i IDFT(E)_i));
 //   decode: z_k = DFT(m_i zeta^i)[j(k)] / scale.
 // This is the only floating-point stage of the library (float64); the
-// result is rounded to integers before any modular arithmetic.  The DFT is
-// an iterative radix-2 transform (bit-reversal copy, then log2 N butterfly
-// passes of N/2 threads): the vectors are small (N complex doubles) and the
-// transform runs once per encoded or decoded message.
+// result is rounded to integers before any modular arithmetic.
+//
+// The DFT is an iterative radix-2 transform of log2 N stages in two launches,
+// 512 points per CTA in shared memory: the first reads its points in
+// bit-reversed order straight from the slots (or coefficients) and runs the 8
+// stages inside runs of 256, the second the rest over columns 256 apart, and
+// writes the rounded coefficients (or slots).  One launch per stage was bound
+// by launches: 17 of them, 85 us at N = 2^16 (one encode and one decode with
+// their copies and transforms, 24 primes: 386 us so, 197 us with two launches
+// and k_lift_wrap).  The stages are the same operations on the same twiddles,
+// so the results are the same bit for bit.
 #include <math.h>
 
 #include <vector>
@@ -26,76 +33,93 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-__global__ void k_scatter_slots(const double2 *__restrict__ z, double scale,
-                                const uint32_t *__restrict__ idx, double2 *E, uint32_t half) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= half) return;
-    const double2 v = make_double2(scale * z[k].x, scale * z[k].y);
-    E[idx[k]] = v;
-    E[idx[half + k]] = make_double2(v.x, -v.y);
+constexpr uint32_t kFftLow = 8;     // stages of the first launch
+constexpr uint32_t kFftPts = 512;   // points per CTA, two per thread
+
+// One butterfly with twiddle w.
+__device__ __forceinline__ void fft_bfly(double2 &x0, double2 &x1, double2 w) {
+    const double2 a = x0, b = cmul(w, x1);
+    x0 = make_double2(a.x + b.x, a.y + b.y);
+    x1 = make_double2(a.x - b.x, a.y - b.y);
 }
 
-__global__ void k_bitrev(const double2 *__restrict__ in, double2 *__restrict__ out,
-                         uint32_t log_n) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >> log_n) return;
-    out[__brev(i) >> (32 - log_n)] = in[i];
+// Stages 0 .. 7 of bit-reversed points.  ENC: point j of the input is the slot
+// named by slot[j] (its conjugate where the top bit is set) times scale; else
+// coefficient j times twist[j].
+template <bool ENC>
+__global__ void __launch_bounds__(kFftPts / 2)
+k_fft_low(const double2 *__restrict__ z, double scale, const uint32_t *__restrict__ slot,
+          const int64_t *__restrict__ m, const double2 *__restrict__ twist,
+          const double2 *__restrict__ tw, double2 *__restrict__ out, uint32_t log_n) {
+    __shared__ double2 x[kFftPts];
+    const uint32_t t = threadIdx.x, i0 = blockIdx.x * kFftPts;
+#pragma unroll
+    for (uint32_t u = 0; u < 2; u++) {
+        const uint32_t i = t + u * (kFftPts / 2), j = __brev(i0 + i) >> (32 - log_n);
+        if (ENC) {
+            const uint32_t k = slot[j];
+            const double2 s = z[k & 0x7fffffffu];
+            const double2 v = make_double2(scale * s.x, scale * s.y);
+            x[i] = make_double2(v.x, k >> 31 ? -v.y : v.y);
+        } else {
+            const double v = double(m[j]);
+            x[i] = make_double2(v * twist[j].x, v * twist[j].y);
+        }
+    }
+#pragma unroll
+    for (uint32_t h = 0; h < kFftLow; h++) {
+        __syncthreads();
+        const uint32_t half = 1u << h, pos = t & (half - 1), a = ((t >> h) << (h + 1)) + pos;
+        fft_bfly(x[a], x[a + half], tw[pos << (log_n - 1 - h)]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < 2; u++) out[i0 + t + u * (kFftPts / 2)] = x[t + u * (kFftPts / 2)];
 }
 
-// One radix-2 pass: butterflies of span `half` with twiddles tw[pos * N / (2 half)].
-__global__ void k_fft_pass(double2 *x, const double2 *__restrict__ tw, uint32_t lg_half,
-                           uint32_t log_n) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >> (log_n - 1)) return;
-    const uint32_t half = 1u << lg_half;
-    const uint32_t pos = t & (half - 1), grp = t >> lg_half;
-    const uint32_t i0 = (grp << (lg_half + 1)) + pos, i1 = i0 + half;
-    const double2 w = tw[pos << (log_n - 1 - lg_half)];
-    const double2 a = x[i0], b = cmul(w, x[i1]);
-    x[i0] = make_double2(a.x + b.x, a.y + b.y);
-    x[i1] = make_double2(a.x - b.x, a.y - b.y);
-}
-
-__global__ void k_untwist_round(const double2 *__restrict__ x, const double2 *__restrict__ twist,
-                                double inv_n, int64_t *m, uint32_t n) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    // Re(x_i conj(zeta^i)) / N, rounded half away from zero
-    const double v = (x[i].x * twist[i].x + x[i].y * twist[i].y) * inv_n;
-    m[i] = (int64_t)round(v);
-}
-
-__global__ void k_twist(const int64_t *__restrict__ m, const double2 *__restrict__ twist, double2 *x,
-                        uint32_t n) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double v = double(m[i]);
-    x[i] = make_double2(v * twist[i].x, v * twist[i].y);
-}
-
-__global__ void k_gather_slots(const double2 *__restrict__ X, const uint32_t *__restrict__ idx,
-                               double inv_scale, double2 *z, uint32_t half) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= half) return;
-    const double2 v = X[idx[k]];
-    z[k] = make_double2(v.x * inv_scale, v.y * inv_scale);
-}
-
-inline unsigned blocks(size_t n) { return unsigned((n + 255) / 256); }
-
-// x (N complex) <- DFT with twiddles tw (omega^(+-k), k < N/2), via tmp.
-int dft(const Context &c, const double2 *in, double2 *out, const double2 *tw, cudaStream_t s) {
-    const uint32_t lg = uint32_t(c.log_n);
-    k_bitrev<<<blocks(c.n), 256, 0, s>>>(in, out, lg);
-    for (uint32_t h = 0; h < lg; h++) k_fft_pass<<<blocks(c.n / 2), 256, 0, s>>>(out, tw, h, lg);
-    note_launches(1 + lg);
-    return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
+// Stages 8 .. log_n - 1: a CTA holds 512 >> (log_n - 8) adjacent columns.
+// ENC: m_i = Re(x_i conj(zeta^i)) / N, rounded half away from zero; else point
+// j goes to its slot, times scale (the conjugates are dropped).
+template <bool ENC>
+__global__ void __launch_bounds__(kFftPts / 2)
+k_fft_high(const double2 *__restrict__ in, const double2 *__restrict__ tw,
+           const double2 *__restrict__ twist, double scale, int64_t *__restrict__ m,
+           const uint32_t *__restrict__ slot, double2 *__restrict__ z, uint32_t log_n) {
+    __shared__ double2 x[kFftPts];
+    const uint32_t t = threadIdx.x, lb = log_n - kFftLow, lc = 9 - lb;  // log rows, log columns
+    const uint32_t c0 = blockIdx.x << lc, cm = (1u << lc) - 1;
+    // x[r << lc | c] is point (r << 8) + c0 + c
+#pragma unroll
+    for (uint32_t u = 0; u < 2; u++) {
+        const uint32_t i = t + u * (kFftPts / 2);
+        x[i] = in[((i >> lc) << kFftLow) + c0 + (i & cm)];
+    }
+    for (uint32_t h = 0; h < lb; h++) {
+        __syncthreads();
+        const uint32_t c = t & cm, r = t >> lc;  // column, butterfly of the column
+        const uint32_t half = 1u << h, pr = r & (half - 1);
+        const uint32_t a = ((((r >> h) << (h + 1)) + pr) << lc) | c;
+        fft_bfly(x[a], x[a + (half << lc)],
+                 tw[((pr << kFftLow) + c0 + c) << (lb - 1 - h)]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < 2; u++) {
+        const uint32_t i = t + u * (kFftPts / 2), j = ((i >> lc) << kFftLow) + c0 + (i & cm);
+        if (ENC) {
+            const double v = (x[i].x * twist[j].x + x[i].y * twist[j].y) * scale;
+            m[j] = (int64_t)round(v);
+        } else {
+            const uint32_t k = slot[j];
+            if (!(k >> 31)) z[k] = make_double2(x[i].x * scale, x[i].y * scale);
+        }
+    }
 }
 
 }  // namespace
 
 // Tables: d_enc = [twist zeta^i (N)][omega^k (N/2)][omega^-k (N/2)],
-// d_slot = [j(k) (N/2)][j'(k) (N/2)].
+// d_slot[j] = the slot k whose point j(k) is, or k | 2^31 where j is j'(k).
 int enc_tables(Context &c) {
     if (c.d_enc) return CATFHE_OK;
     const size_t n = c.n, half = n / 2;
@@ -110,8 +134,8 @@ int enc_tables(Context &c) {
     std::vector<uint32_t> idx(n);
     uint64_t e = 1;
     for (size_t k = 0; k < half; k++) {
-        idx[k] = uint32_t((e - 1) / 2);
-        idx[half + k] = uint32_t((2 * n - e - 1) / 2);
+        idx[(e - 1) / 2] = uint32_t(k);
+        idx[(2 * n - e - 1) / 2] = uint32_t(k) | 0x80000000u;
         e = e * 5 % (2 * n);
     }
     double2 *d = nullptr;
@@ -132,29 +156,28 @@ int enc_tables(Context &c) {
     return CATFHE_OK;
 }
 
-int launch_encode_ckks(const Context &c, const double2 *slots, double scale, double2 *buf0,
-                       double2 *buf1, int64_t *m, cudaStream_t s) {
-    const size_t n = c.n, half = n / 2;
-    const double2 *twist = c.d_enc, *tw_inv = c.d_enc + n + half;
-    k_scatter_slots<<<blocks(half), 256, 0, s>>>(slots, scale, c.d_slot, buf0, uint32_t(half));
-    note_launches(1);
-    const int rc = dft(c, buf0, buf1, tw_inv, s);
-    if (rc) return rc;
-    k_untwist_round<<<blocks(n), 256, 0, s>>>(buf1, twist, 1.0 / double(n), m, uint32_t(n));
-    note_launches(1);
+int launch_encode_ckks(const Context &c, const double2 *slots, double scale, double2 *buf,
+                       int64_t *m, cudaStream_t s) {
+    const size_t n = c.n;
+    const uint32_t lg = uint32_t(c.log_n), ctas = uint32_t(n / kFftPts);
+    const double2 *twist = c.d_enc, *tw = c.d_enc + n + n / 2;
+    k_fft_low<true><<<ctas, kFftPts / 2, 0, s>>>(slots, scale, c.d_slot, nullptr, nullptr, tw, buf,
+                                                 lg);
+    k_fft_high<true><<<ctas, kFftPts / 2, 0, s>>>(buf, tw, twist, 1.0 / double(n), m, nullptr,
+                                                  nullptr, lg);
+    note_launches(2);
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 
-int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, double2 *buf0,
-                       double2 *buf1, double2 *slots, cudaStream_t s) {
-    const size_t n = c.n, half = n / 2;
-    const double2 *twist = c.d_enc, *tw_fwd = c.d_enc + n;
-    k_twist<<<blocks(n), 256, 0, s>>>(m, twist, buf0, uint32_t(n));
-    note_launches(1);
-    const int rc = dft(c, buf0, buf1, tw_fwd, s);
-    if (rc) return rc;
-    k_gather_slots<<<blocks(half), 256, 0, s>>>(buf1, c.d_slot, inv_scale, slots, uint32_t(half));
-    note_launches(1);
+int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, double2 *buf,
+                       double2 *slots, cudaStream_t s) {
+    const size_t n = c.n;
+    const uint32_t lg = uint32_t(c.log_n), ctas = uint32_t(n / kFftPts);
+    const double2 *twist = c.d_enc, *tw = c.d_enc + n;
+    k_fft_low<false><<<ctas, kFftPts / 2, 0, s>>>(nullptr, 0.0, nullptr, m, twist, tw, buf, lg);
+    k_fft_high<false><<<ctas, kFftPts / 2, 0, s>>>(buf, tw, nullptr, inv_scale, nullptr, c.d_slot,
+                                                   slots, lg);
+    note_launches(2);
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 

@@ -108,6 +108,8 @@ struct PlanRef {
 };
 struct Context;
 PlanRef get_plan(Context &c, const std::string &key, const PlanSpec &spec);
+// Device copy of plain words, kept in c.plans[key]; null: no memory.
+const uint64_t *upload_words(Context &c, const std::string &key, const std::vector<uint64_t> &w);
 // Device copy of a plan's tensor-core image and its header words.
 struct MmaRef {
     const uint64_t *p = nullptr;  // device image, null when the plan has none
@@ -166,6 +168,8 @@ struct LiftEntry {
     uint64_t flags;
 };
 constexpr uint64_t kLiftPre = 1, kLiftPost = 2, kLiftReduce = 4;
+// The words are signed integers instead, reduced mod p (nothing else is read).
+constexpr uint64_t kLiftSigned = 8;
 // The entry for source m, target p and factors pre, post (1: none).
 LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post);
 // Device copy of a lift table (null: no memory), kept under key.
@@ -322,6 +326,13 @@ int launch_conv(const Context &c, const ConvPlans &plans, const uint64_t *src, s
 int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src, size_t src_item,
                     size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan,
                     uint32_t items, cudaStream_t s);
+// The centred lift of x from q_0 .. q_{level-1} to 64-bit two's complement (the
+// CKKS decryption's last step): out[j] from limbs j + i N of x.  consts: device
+// {m, w, w's Shoup quotient, c | shift, M/m, .} per prime and then M mod 2^64
+// (wrap_consts); exact: the Montgomery plan of the same primes.
+std::vector<uint64_t> wrap_consts(const std::vector<uint64_t> &mods);
+int launch_lift_wrap(const Context &c, const uint64_t *consts, const uint64_t *exact,
+                     uint32_t level, const uint64_t *x, uint64_t *out, cudaStream_t s);
 // BFV: given the tensor x over Q u B (coefficient form, Q limbs first) of
 // each item, writes round(t x / Q) mod q_i: y = t x; z = (y - [y]_Q) Q^-1 over
 // B (plan q_to_b lifts [y]_Q with pre = t and post = 1); then the centred
@@ -413,12 +424,12 @@ int launch_mul_plain(const Context &c, const uint64_t *a, const uint64_t *pt, ui
 
 // CKKS canonical embedding on the device (encode.cu).  enc_tables builds
 // the context's tables once; encode: N/2 device slots -> int64 m[N];
-// decode: int64 m[N] -> N/2 device slots.  buf0, buf1: N complex each.
+// decode: int64 m[N] -> N/2 device slots.  buf: N complex.
 int enc_tables(Context &c);
-int launch_encode_ckks(const Context &c, const double2 *slots, double scale, double2 *buf0,
-                       double2 *buf1, int64_t *m, cudaStream_t s);
-int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, double2 *buf0,
-                       double2 *buf1, double2 *slots, cudaStream_t s);
+int launch_encode_ckks(const Context &c, const double2 *slots, double scale, double2 *buf,
+                       int64_t *m, cudaStream_t s);
+int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, double2 *buf,
+                       double2 *slots, cudaStream_t s);
 int launch_add(const Context &c, const uint64_t *a, const uint64_t *b, uint64_t *out,
                const LimbMap &map, uint32_t n_limbs, cudaStream_t s);
 int launch_copy_limbs(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,

@@ -1480,6 +1480,15 @@ static int decrypt_device(Context &c, const Keys &k, const uint64_t *ct, uint32_
     std::string key = "decrypt/" + std::to_string(level);
     if (c.scheme == CATFHE_CKKS) {
         sp.dst_mod.push_back(0);
+        if (plan_fits_mont(sp)) {
+            const PlanRef exact = get_plan(c, key, sp);
+            if (!exact.p) return CATFHE_ENOMEM;
+            const std::string wkey = key + "/wrap";
+            if (!c.plans.count(wkey) && !upload_words(c, wkey, wrap_consts(sp.src_mod)))
+                return CATFHE_ENOMEM;
+            return launch_lift_wrap(c, c.plans[wkey], exact.p, level, x,
+                                    reinterpret_cast<uint64_t *>(res), s);
+        }
     } else {
         sp.dst_mod.push_back(c.t);
         if (c.scheme == CATFHE_BFV) {
@@ -1525,14 +1534,21 @@ int op_encode_ckks(Context &c, const double *slots, double scale, uint32_t level
     Bump b{base};
     const size_t n = c.n;
     double2 *dz = b.take<double2>(n / 2);
-    double2 *b0 = b.take<double2>(n), *b1 = b.take<double2>(n);
+    double2 *buf = b.take<double2>(n);
     int64_t *m = b.take<int64_t>(n);
     if (cudaMemcpyAsync(dz, slots, n / 2 * sizeof(double2), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return CATFHE_ECUDA;
-    TRY(launch_encode_ckks(c, dz, scale, b0, b1, m, s));
+    TRY(launch_encode_ckks(c, dz, scale, buf, m, s));
+    // every limb's transform reduces the signed coefficients as it loads them
     LimbMap mp = map_identity(level);
-    TRY(launch_small_to_rns(c, m, pt, mp, level, nullptr, nullptr, 0, s));
-    TRY(launch_ntt_fwd(c, pt, pt, mp, level, s));
+    for (uint32_t i = 0; i < level; i++) mp.src_off[i] = 0;
+    const LiftEntry *lifts = get_lifts(c, "signed", [&] {
+        LiftEntry e{};
+        e.flags = kLiftSigned;
+        return std::vector<LiftEntry>(size_t(c.L), e);
+    });
+    if (!lifts) return CATFHE_ENOMEM;
+    TRY(launch_ntt_lift(c, reinterpret_cast<const uint64_t *>(m), pt, mp, level, lifts, false, s));
     return cudaStreamSynchronize(s) == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 
@@ -1549,10 +1565,10 @@ int op_decode_ckks(Context &c, const Keys &k, const uint64_t *ct, uint32_t level
     const size_t n = c.n;
     char *dec = reinterpret_cast<char *>(b.take<uint64_t>(size_t(2) * level * n));
     int64_t *m = b.take<int64_t>(n);
-    double2 *b0 = b.take<double2>(n), *b1 = b.take<double2>(n);
+    double2 *buf = b.take<double2>(n);
     double2 *dz = b.take<double2>(n / 2);
     TRY(decrypt_device(c, k, ct, level, m, dec, s));
-    TRY(launch_decode_ckks(c, m, 1.0 / scale, b0, b1, dz, s));
+    TRY(launch_decode_ckks(c, m, 1.0 / scale, buf, dz, s));
     if (cudaMemcpyAsync(slots, dz, n / 2 * sizeof(double2), cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return CATFHE_ECUDA;
     return cudaStreamSynchronize(s) == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
