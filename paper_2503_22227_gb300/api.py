@@ -83,6 +83,8 @@ u8p = ctypes.POINTER(ctypes.c_uint8)
 def load(path: str = LIB_PATH):
     """Loads libcatfhe.so (raises if it is missing: there is no fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -230,12 +232,11 @@ class Context:
         return torch.empty((count, 2, level, self.n), dtype=torch.int64, device="cuda")
 
     def workspace(self, op: int, level: int, count: int):
-        torch = _torch()
-        need = load().catfhe_workspace_bytes(self._h, op, level, count)
         key = (op, level, count)
         ws = self._ws.get(key)
-        if ws is None or ws.numel() < need:
-            ws = torch.empty(max(need, 1), dtype=torch.uint8, device="cuda")
+        if ws is None:
+            need = load().catfhe_workspace_bytes(self._h, op, level, count)
+            ws = _torch().empty(max(need, 1), dtype=_torch().uint8, device="cuda")
             self._ws[key] = ws
         return ws
 

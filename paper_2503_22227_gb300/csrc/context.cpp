@@ -153,7 +153,7 @@ void ctx_free(Context &c) {
     cudaFree(c.d_twf);
     cudaFree(c.d_twi);
     for (auto &kv : c.plans) cudaFree(kv.second);
-    for (auto &kv : c.lifts) cudaFree(kv.second);
+    for (LiftEntry *t : c.lifts) cudaFree(t);
     for (auto &kv : c.mma_plans) cudaFree(const_cast<uint64_t *>(kv.second.p));
     cudaFree(c.scratch.ptr);
     c.plans.clear();
@@ -399,8 +399,7 @@ LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post) {
     return e;
 }
 
-const LiftEntry *upload_lifts(Context &c, const std::string &key,
-                              const std::vector<LiftEntry> &table) {
+const LiftEntry *upload_lifts(Context &c, const std::vector<LiftEntry> &table) {
     LiftEntry *dev = nullptr;
     const size_t bytes = table.size() * sizeof(LiftEntry);
     if (cudaMalloc(&dev, bytes) != cudaSuccess) return nullptr;
@@ -408,7 +407,8 @@ const LiftEntry *upload_lifts(Context &c, const std::string &key,
         cudaFree(dev);
         return nullptr;
     }
-    return c.lifts[key] = dev;
+    c.lifts.push_back(dev);
+    return dev;
 }
 
 const uint64_t *upload_words(Context &c, const std::string &key, const std::vector<uint64_t> &w) {

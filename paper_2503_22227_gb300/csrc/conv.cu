@@ -803,6 +803,21 @@ int resident_slots(const void *kernel, int threads, size_t smem) {
     return cache[key] = sms * occ;
 }
 
+bool allow_smem(const void *kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> allowed;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> g(mu);
+    size_t &have = allowed[{dev, kernel}];
+    if (have >= bytes) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) !=
+        cudaSuccess)
+        return false;
+    have = bytes;
+    return true;
+}
+
 template <typename K>
 static unsigned stride_columns(K kernel, size_t smem, size_t n, uint32_t items) {
     const int slots_i = resident_slots(reinterpret_cast<const void *>(kernel), 256, smem);

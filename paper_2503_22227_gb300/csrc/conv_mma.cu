@@ -291,9 +291,7 @@ int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src,
         lazy = lazy && ((plans.head[i] >> 24) & 1);
     }
     const auto kernel = lazy ? k_conv_mma<true> : k_conv_mma<false>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-        cudaSuccess)
-        return CATFHE_ECUDA;
+    if (!allow_smem(reinterpret_cast<const void *>(kernel), smem)) return CATFHE_ECUDA;
     const uint32_t tiles = uint32_t(items * (c.n / kMmaTile));
     const dim3 grid(mma_grid(c, tiles, smem, plans.n), 1, plans.n);
     launch_pdl(kernel, grid, dim3(kMmaTile), smem, s, plans, src, src_item, src_plan, dst,
@@ -327,9 +325,7 @@ int launch_bfv_round_mma(const Context &c, const MmaRef &a, const uint64_t *a_ex
     l.img[0] = a.p, l.head[0] = a.head, l.counts[0] = a.counts, l.p[0] = a_exact;
     l.img[1] = b.p, l.head[1] = b.head, l.counts[1] = b.counts, l.p[1] = b_exact;
     const uint32_t smem = bfv_round_smem(a, b);
-    if (cudaFuncSetAttribute(k_bfv_round_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(smem)) != cudaSuccess)
-        return CATFHE_ECUDA;
+    if (!allow_smem(reinterpret_cast<const void *>(k_bfv_round_mma), smem)) return CATFHE_ECUDA;
     const uint32_t tiles = uint32_t(items * (c.n / kMmaTile));
     launch_pdl(k_bfv_round_mma, dim3(mma_grid(c, tiles, smem, 1)), dim3(kMmaTile), smem, s, l, src,
                src_item, dst, dst_item, uint32_t(c.log_n), tiles, c.d_status);

@@ -320,9 +320,7 @@ static int ip_run_bulk(const Context &c, const IpArgs &a, uint32_t count, cudaSt
     constexpr uint32_t tile = IpTile<BETA>::value;
     constexpr size_t smem = size_t(4 * BETA + 4) * tile * 8;
     const auto kernel = k_ip_bulk<BETA, GATHER>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-        cudaSuccess)
-        return CATFHE_ECUDA;
+    if (!allow_smem(reinterpret_cast<const void *>(kernel), smem)) return CATFHE_ECUDA;
     const unsigned groups = ip_groups(kernel, tile / 2, smem, c.n / tile * a.M, count);
     launch_pdl(kernel, dim3(unsigned(c.n / tile), a.M, groups), dim3(tile / 2), smem, s, a, c.d_mods,
                uint32_t(c.log_n), count);

@@ -6,6 +6,7 @@
 
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -172,9 +173,8 @@ constexpr uint64_t kLiftPre = 1, kLiftPost = 2, kLiftReduce = 4;
 constexpr uint64_t kLiftSigned = 8;
 // The entry for source m, target p and factors pre, post (1: none).
 LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post);
-// Device copy of a lift table (null: no memory), kept under key.
-const LiftEntry *upload_lifts(Context &c, const std::string &key,
-                              const std::vector<LiftEntry> &table);
+// Device copy of a lift table, freed with the context (null: no memory).
+const LiftEntry *upload_lifts(Context &c, const std::vector<LiftEntry> &table);
 
 // Up to this many plans run in one launch (grid.z).
 struct PlanList {
@@ -226,7 +226,14 @@ struct Context {
     std::map<std::string, uint64_t *> plans;     // device copies of packed plans
     std::map<std::string, uint32_t> plan_sizes;  // words
     std::map<std::string, MmaRef> mma_plans;     // tensor-core images (device)
-    std::map<std::string, LiftEntry *> lifts;    // lift tables (device)
+    std::vector<LiftEntry *> lifts;              // lift tables (device)
+    const LiftEntry *signed_lifts = nullptr;     // signed words to q_0 .. q_{L-1}
+    // launch constants per operation and level (ops.cpp), built on first use
+    // under mu; as many as there are levels
+    std::mutex mu;
+    std::map<int, std::shared_ptr<struct KsConsts>> ks;
+    std::map<int, std::shared_ptr<struct BfvConsts>> bfv;
+    std::map<int, std::shared_ptr<struct RescaleConsts>> rescale;
     Scratch scratch;
     int device = 0;
     int sms = 0;  // the device's SM count
@@ -255,6 +262,9 @@ struct Keys {
     std::map<uint64_t, uint64_t *> ksk;
 };
 
+// Lets `kernel` use `bytes` of dynamic shared memory on the current device; the
+// driver is asked once per kernel, device and larger size.
+bool allow_smem(const void *kernel, size_t bytes);
 // Number of kernels this library has launched (all contexts, all threads).
 void note_launches(uint32_t k);
 // CTAs of `kernel` resident on the whole current device (SMs x CTAs per SM at

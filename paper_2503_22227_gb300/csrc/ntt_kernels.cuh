@@ -602,9 +602,7 @@ static int run_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const L
         constexpr int ybytes = T2 * (1 << E2) * 8;  // the CTA's y tile
         const auto kernel = epi->galois ? k_ntt_fwd_rows<LN, R2, E2, T2, B2, 4>
                                         : k_ntt_fwd_rows<LN, R2, E2, T2, B2, 2>;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ybytes) !=
-            cudaSuccess)
-            return CATFHE_ECUDA;
+        if (!allow_smem(reinterpret_cast<const void *>(kernel), ybytes)) return CATFHE_ECUDA;
         launch_pdl(kernel, g2, dim3(T2), ybytes, s, dst, map, c.d_mods, c.d_twf, *epi);
     } else if (lazy) {
         launch_pdl(k_ntt_fwd_rows<LN, R2, E2, T2, B2, 3>, g2, dim3(T2), 0, s, dst, map, c.d_mods,

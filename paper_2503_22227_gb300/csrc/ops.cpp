@@ -100,13 +100,6 @@ static int make_list(Context &c, const std::vector<std::pair<std::string, PlanSp
     return CATFHE_OK;
 }
 
-// The lift table kept under key, built by make() on first use.
-template <class F>
-static const LiftEntry *get_lifts(Context &c, const std::string &key, F make) {
-    const auto it = c.lifts.find(key);
-    return it != c.lifts.end() ? it->second : upload_lifts(c, key, make());
-}
-
 // The entries of a ModDown or rescale by the one prime at index `from`, for
 // both polynomials' targets q_0 .. q_{lo-1}.
 static std::vector<LiftEntry> division_lifts(const Context &c, int from, int lo) {
@@ -151,36 +144,6 @@ static uint64_t pmod(const Context &c, uint64_t m) { return prod_mod(c, c.L, c.L
 // Global prime index of extended position i at level l (Q_l then P).
 static int ext_prime(const Context &c, int level, int i) { return i < level ? i : c.L + (i - level); }
 
-// ModUp: lift each digit of d2 (coefficient form, [level][N] per ciphertext,
-// d2_item words apart) to the other primes of Q_l u P (own_too: to all of
-// them), written into ext ([count][beta][M][N]).
-static int modup(Context &c, const uint64_t *d2c, size_t d2_item, uint64_t *ext, uint32_t count,
-                 int level, bool own_too, cudaStream_t s) {
-    const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
-    std::vector<std::pair<std::string, PlanSpec>> specs;
-    for (int j = 0; j < beta; j++) {
-        const int lo = j * c.alpha, hi = std::min((j + 1) * c.alpha, level);
-        PlanSpec sp;
-        sp.lazy = true;  // the lifted limbs go straight into an NTT
-        for (int i = lo; i < hi; i++) {
-            sp.src_mod.push_back(c.mod(i));
-            sp.src_off.push_back(uint32_t(i));
-        }
-        for (int i = 0; i < M; i++) {
-            if (!own_too && i >= lo && i < hi) continue;
-            sp.dst_mod.push_back(c.mod(ext_prime(c, level, i)));
-            sp.dst_off.push_back(uint32_t(i));
-        }
-        specs.emplace_back("modup/" + std::to_string(level) + "/" + std::to_string(j) +
-                               (own_too ? "/own" : ""),
-                           sp);
-    }
-    ConvPlans pl{};
-    TRY(make_list(c, specs, pl));
-    const size_t n = c.n;
-    return launch_conv(c, pl, d2c, d2_item, 0, ext, size_t(beta) * M * n, size_t(M) * n, count, s);
-}
-
 // Whether the lifted digits' forward NTT may leave its words unreduced: the
 // inner product is their only reader and reduces its sums once (Montgomery,
 // valid below 2^64 q); with words below 68q from an unreduced transform, its
@@ -199,68 +162,69 @@ static bool ext_lazy(const Context &c, int level) {
     return true;
 }
 
-// ModUp and the NTT of the lifted limbs (all positions if own_too).  Digits of
-// one prime are lifted by the transform's first pass as it loads; wider ones
-// are converted first.
-static int modup_ntt(Context &c, const uint64_t *d2c, size_t d2_item, uint64_t *ext, uint32_t count,
-                     int level, bool own_too, cudaStream_t s) {
+// Everything of a key switching at one level (fused: with the rescale) that does
+// not depend on the call: limb maps, conversion plans, launch arguments with
+// their constants.  Built on first use and kept by the context; a call copies
+// the arguments and fills in its pointers.  (Computing them anew, inverses
+// included, took 10 to 20 us of host time per call, as long as the device
+// needs at the smallest sizes.)
+struct KsConsts {
+    // ModUp and the NTT of the lifted limbs (all positions for BFV)
+    ConvPlans up;
+    const LiftEntry *up_lifts = nullptr;  // digits of one prime: lifted by the transform
+    LimbMap ext{};
+    bool lazy = false;
+    IpArgs ip{};
+    // ModDown by P (fused: P q_{l-1})
+    LimbMap special{};  // the division basis' limbs of y
+    ConvPlans down;
+    const LiftEntry *down_lifts = nullptr;  // division by one prime
+    LimbMap lift{};                         // NTT schemes: the lift's transform
+    NttEpilogue epi{};
+    CombineArgs comb{};                     // BFV
+};
+
+static int build_modup(Context &c, int level, KsConsts &k) {
     const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
-    const bool one = c.alpha == 1 && d2_item % c.n == 0;
-    LimbMap m{};
+    const bool own_too = c.scheme == CATFHE_BFV, one = c.alpha == 1;
+    LimbMap &m = k.ext;
+    std::vector<std::pair<std::string, PlanSpec>> specs;
+    std::vector<LiftEntry> lifts;
     uint32_t e = 0;
     for (int j = 0; j < beta; j++) {
         const int lo = j * c.alpha, hi = std::min((j + 1) * c.alpha, level);
+        PlanSpec sp;
+        sp.lazy = true;  // the lifted limbs go straight into an NTT
+        for (int i = lo; i < hi; i++) {
+            sp.src_mod.push_back(c.mod(i));
+            sp.src_off.push_back(uint32_t(i));
+        }
         for (int i = 0; i < M; i++) {
             if (!own_too && i >= lo && i < hi) continue;
             if (e >= uint32_t(kMapMax)) return CATFHE_EINVAL;
+            const int p = ext_prime(c, level, i);
             m.dst_off[e] = uint16_t(j * M + i);
             m.src_off[e] = one ? uint16_t(j) : m.dst_off[e];
-            m.prime[e] = uint8_t(ext_prime(c, level, i));
+            m.prime[e] = uint8_t(p);
             e++;
+            sp.dst_mod.push_back(c.mod(p));
+            sp.dst_off.push_back(uint32_t(i));
+            if (one) lifts.push_back(lift_entry(c.mod(j), c.mod(p), 1, 1));
         }
+        specs.emplace_back("modup/" + std::to_string(level) + "/" + std::to_string(j), sp);
     }
     m.period = e;
-    m.dst_stride = uint32_t(beta * M);
-    m.src_stride = one ? uint32_t(d2_item / c.n) : m.dst_stride;
-    const bool lazy = ext_lazy(c, level);
-    if (one) {
-        const LiftEntry *lifts =
-            get_lifts(c, "modup/" + std::to_string(level) + (own_too ? "/own" : ""), [&] {
-                std::vector<LiftEntry> t;
-                for (uint32_t r = 0; r < e; r++)
-                    t.push_back(lift_entry(c.mod(m.src_off[r]), c.mod(m.prime[r]), 1, 1));
-                return t;
-            });
-        if (!lifts) return CATFHE_ENOMEM;
-        return launch_ntt_lift(c, d2c, ext, m, e * count, lifts, lazy, s);
-    }
-    TRY(modup(c, d2c, d2_item, ext, count, level, own_too, s));
-    return lazy ? launch_ntt_fwd_lazy(c, ext, ext, m, e * count, s)
-                : launch_ntt_fwd(c, ext, ext, m, e * count, s);
+    m.src_stride = m.dst_stride = uint32_t(beta * M);
+    k.lazy = ext_lazy(c, level);
+    if (!one) return make_list(c, specs, k.up);
+    k.up_lifts = upload_lifts(c, lifts);
+    return k.up_lifts ? CATFHE_OK : CATFHE_ENOMEM;
 }
 
-// own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
-// words apart (null: none).  gth (rotations): ciphertext i's add0 and own are
-// the two polynomials of gth->a[i].
-static int inner_product(Context &c, const uint64_t *ext, const uint64_t *own, const uint64_t *key,
-                         const uint64_t *add0, const uint64_t *add1, size_t in_item, uint64_t *y,
-                         uint32_t count, int level, cudaStream_t s, const Gather *gth = nullptr) {
+static void build_ip(const Context &c, int level, IpArgs &a) {
     const int M = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
-    const size_t n = c.n;
-    IpArgs a{};
-    a.ext = ext;
-    a.own = own;
-    a.key = key;
-    a.add0 = add0;
-    a.add1 = add1;
-    a.y = y;
-    if (gth && gth->n) {
-        a.gathered = 1;
-        for (uint32_t i = 0; i < gth->n; i++) a.ga[i] = gth->a[i];
-    }
-    a.ext_item = size_t(beta) * M * n;
-    a.own_item = a.add_item = in_item;
-    a.y_item = size_t(2) * M * n;
+    a.ext_item = size_t(beta) * M * c.n;
+    a.y_item = size_t(2) * M * c.n;
     a.M = M;
     a.level = level;
     a.beta = beta;
@@ -277,41 +241,28 @@ static int inner_product(Context &c, const uint64_t *ext, const uint64_t *own, c
             a.pfac[i] = h_mulmod(pmod(c, q), r, q);  // P in Montgomery form
         }
     }
-    return launch_ip(c, a, count, s);
 }
 
-// ModDown of y ([count][2][M][N]; NTT form for CKKS/BGV, coefficient form
-// for BFV) by D = P (fused: P q_{l-1}) into out ([count][2][lo][N]).
-// add (BFV): [.][lo][N] added to the first add_polys polynomials, add_item
-// words per ciphertext.  g: sigma_g applied to the result (0: none).
-static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint32_t count,
-                   int level, bool fused, cudaStream_t s, uint64_t g = 0,
-                   const Gather *gth = nullptr, const uint64_t *add = nullptr,
-                   uint32_t add_polys = 0, size_t add_item = 0) {
+static int build_moddown(Context &c, int level, bool fused, KsConsts &k) {
     const int M = level + c.K, lo = fused ? level - 1 : level;
     const size_t n = c.n;
     const bool ntt_form = c.scheme != CATFHE_BFV;
     // division basis positions in y: P, then q_{l-1} when fused
     std::vector<int> dpos;
-    for (int k = 0; k < c.K; k++) dpos.push_back(level + k);
+    for (int i = 0; i < c.K; i++) dpos.push_back(level + i);
     if (fused) dpos.push_back(level - 1);
     const int Kd = int(dpos.size());
-    if (ntt_form) {
-        LimbMap m{};
-        m.period = uint32_t(2 * Kd);
-        m.src_stride = m.dst_stride = uint32_t(2 * M);
-        for (int p = 0; p < 2; p++)
-            for (int d = 0; d < Kd; d++) {
-                m.src_off[p * Kd + d] = m.dst_off[p * Kd + d] = uint16_t(p * M + dpos[d]);
-                m.prime[p * Kd + d] = uint8_t(ext_prime(c, level, dpos[d]));
-            }
-        TRY(launch_ntt_inv(c, y, y, m, m.period * count, s));
-    }
-    const std::string key = "moddown/" + std::to_string(level) + (fused ? "/f" : "");
-    const LiftEntry *lifts = nullptr;
+    LimbMap &m = k.special;
+    m.period = uint32_t(2 * Kd);
+    m.src_stride = m.dst_stride = uint32_t(2 * M);
+    for (int p = 0; p < 2; p++)
+        for (int d = 0; d < Kd; d++) {
+            m.src_off[p * Kd + d] = m.dst_off[p * Kd + d] = uint16_t(p * M + dpos[d]);
+            m.prime[p * Kd + d] = uint8_t(ext_prime(c, level, dpos[d]));
+        }
     if (Kd == 1) {  // lifted by the next kernel as it loads
-        lifts = get_lifts(c, key, [&] { return division_lifts(c, ext_prime(c, level, dpos[0]), lo); });
-        if (!lifts) return CATFHE_ENOMEM;
+        k.down_lifts = upload_lifts(c, division_lifts(c, ext_prime(c, level, dpos[0]), lo));
+        if (!k.down_lifts) return CATFHE_ENOMEM;
     } else {
         PlanSpec sp;
         sp.lazy = ntt_form;  // NTT schemes transform the lift before the combine
@@ -328,75 +279,145 @@ static int moddown(Context &c, uint64_t *y, uint64_t *lift, uint64_t *out, uint3
                 sp.pre.push_back(h_invmod(c.t % sp.src_mod[d], sp.src_mod[d]));
             for (int i = 0; i < lo; i++) sp.post.push_back(c.t % c.mod(i));
         }
-        ConvPlans pl{};
-        TRY(make_list(c, {{key, sp}}, pl));
-        TRY(launch_conv(c, pl, y, size_t(M) * n, 0, lift, size_t(lo) * n, 0, 2 * count, s));
+        TRY(make_list(c, {{"moddown/" + std::to_string(level) + (fused ? "/f" : ""), sp}}, k.down));
     }
     // D^-1 mod q_i, D = P (fused: P q_{l-1})
-    std::vector<uint64_t> dinv(lo), dinv_s(lo);
+    LimbMap &l = k.lift;
+    NttEpilogue &e = k.epi;
+    CombineArgs &a = k.comb;
+    l.period = l.dst_stride = uint32_t(2 * lo);
+    l.src_stride = Kd == 1 ? uint32_t(2 * M) : uint32_t(2 * lo);
+    e.status = c.d_status;
+    e.y_stride = uint32_t(2 * M);
+    e.out_stride = uint32_t(2 * lo);
+    a.lifts = k.down_lifts;
+    a.y_last = size_t(dpos[0]) * n;
+    a.y_item = size_t(2) * M * n;
+    a.y_poly = size_t(M) * n;
+    a.lift_item = a.out_item = size_t(2) * lo * n;
+    a.lift_poly = a.add_poly = a.out_poly = size_t(lo) * n;
+    a.lo = uint32_t(lo);
     for (int i = 0; i < lo; i++) {
         const uint64_t q = c.mod(i);
         uint64_t D = pmod(c, q);
         if (fused) D = h_mulmod(D, c.mod(level - 1) % q, q);
-        dinv[i] = h_invmod(D, q);
-        dinv_s[i] = h_shoup(dinv[i], q);
+        const uint64_t dinv = h_invmod(D, q), dinv_s = h_shoup(dinv, q);
+        a.prime[i] = uint8_t(i);
+        a.dinv[i] = dinv;
+        a.dinv_s[i] = dinv_s;
+        for (int p = 0; p < 2; p++) {
+            const int r = p * lo + i;
+            l.dst_off[r] = uint16_t(r);
+            l.src_off[r] = Kd == 1 ? uint16_t(p * M + dpos[0]) : uint16_t(r);
+            l.prime[r] = uint8_t(i);
+            e.y_off[r] = uint16_t(p * M + i);
+            e.out_off[r] = uint16_t(r);
+            e.dinv[r] = dinv;
+            e.dinv_s[r] = dinv_s;
+        }
     }
+    return CATFHE_OK;
+}
+
+// The entry `key` of a context's map of constants, built by make(entry) on
+// first use; the context's lock covers the look-up and the building.
+template <class T, class F>
+static int kept(Context &c, std::map<int, std::shared_ptr<T>> &map, int key, const T **out, F make) {
+    std::lock_guard<std::mutex> lock(c.mu);
+    auto it = map.find(key);
+    if (it == map.end()) {
+        auto t = std::make_shared<T>();
+        TRY(make(*t));
+        it = map.emplace(key, t).first;
+    }
+    *out = it->second.get();
+    return CATFHE_OK;
+}
+
+static int ks_consts(Context &c, int level, bool fused, const KsConsts **out) {
+    return kept(c, c.ks, 2 * level + (fused ? 1 : 0), out, [&](KsConsts &k) -> int {
+        TRY(build_modup(c, level, k));
+        build_ip(c, level, k.ip);
+        return build_moddown(c, level, fused, k);
+    });
+}
+
+// ModUp of d2 (coefficient form, [level][N] per ciphertext, d2_item words
+// apart) into ext ([count][beta][M][N]) and the NTT of the lifted limbs.
+// Digits of one prime are lifted by the transform's first pass as it loads;
+// wider ones are converted first.
+static int modup_ntt(Context &c, const KsConsts &k, const uint64_t *d2c, size_t d2_item,
+                     uint64_t *ext, uint32_t count, cudaStream_t s) {
+    const size_t n = c.n;
+    if (k.up_lifts) {
+        LimbMap m = k.ext;
+        m.src_stride = uint32_t(d2_item / n);
+        return launch_ntt_lift(c, d2c, ext, m, m.period * count, k.up_lifts, k.lazy, s);
+    }
+    TRY(launch_conv(c, k.up, d2c, d2_item, 0, ext, k.ip.ext_item, size_t(k.ip.M) * n, count, s));
+    return k.lazy ? launch_ntt_fwd_lazy(c, ext, ext, k.ext, k.ext.period * count, s)
+                  : launch_ntt_fwd(c, ext, ext, k.ext, k.ext.period * count, s);
+}
+
+// own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
+// words apart (null: none).  gth (rotations): ciphertext i's add0 and own are
+// the two polynomials of gth->a[i].
+static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, const uint64_t *own,
+                         const uint64_t *key, const uint64_t *add0, const uint64_t *add1,
+                         size_t in_item, uint64_t *y, uint32_t count, cudaStream_t s,
+                         const Gather *gth = nullptr) {
+    IpArgs a = k.ip;
+    a.ext = ext;
+    a.own = own;
+    a.key = key;
+    a.add0 = add0;
+    a.add1 = add1;
+    a.y = y;
+    a.own_item = a.add_item = in_item;
+    if (gth && gth->n) {
+        a.gathered = 1;
+        for (uint32_t i = 0; i < gth->n; i++) a.ga[i] = gth->a[i];
+    }
+    return launch_ip(c, a, count, s);
+}
+
+// ModDown of y ([count][2][M][N]; NTT form for CKKS/BGV, coefficient form
+// for BFV) into out ([count][2][lo][N]).
+// add (BFV): [.][lo][N] added to the first add_polys polynomials, add_item
+// words per ciphertext.  g: sigma_g applied to the result (0: none).
+static int moddown(Context &c, const KsConsts &k, uint64_t *y, uint64_t *lift, uint64_t *out,
+                   uint32_t count, cudaStream_t s, uint64_t g = 0, const Gather *gth = nullptr,
+                   const uint64_t *add = nullptr, uint32_t add_polys = 0, size_t add_item = 0) {
+    const bool ntt_form = c.scheme != CATFHE_BFV;
     if (gth && gth->n && (!ntt_form || add || gth->n != count)) return CATFHE_EINVAL;
+    if (ntt_form) TRY(launch_ntt_inv(c, y, y, k.special, k.special.period * count, s));
+    if (!k.down_lifts)
+        TRY(launch_conv(c, k.down, y, size_t(k.ip.M) * c.n, 0, lift, k.comb.lift_poly, 0, 2 * count,
+                        s));
     if (ntt_form) {
         // NTT of the lift whose last pass writes (y - lift) D^-1 straight to out
-        LimbMap m{};
-        NttEpilogue e{};
+        NttEpilogue e = k.epi;
+        e.y = y;
+        e.out = out;
+        e.galois = uint32_t(g);
+        e.galois_inv = g ? uint32_t(inv_mod_pow2(g, 2 * c.n)) : 0;
         if (gth && gth->n) {
             e.gathered = 1;
             for (uint32_t i = 0; i < gth->n; i++) e.gout[i] = gth->out[i];
         }
-        m.period = uint32_t(2 * lo);
-        m.dst_stride = uint32_t(2 * lo);
-        m.src_stride = lifts ? uint32_t(2 * M) : uint32_t(2 * lo);
-        e.y = y;
-        e.out = out;
-        e.status = c.d_status;
-        e.y_stride = uint32_t(2 * M);
-        e.out_stride = uint32_t(2 * lo);
-        e.galois = uint32_t(g);
-        e.galois_inv = g ? uint32_t(inv_mod_pow2(g, 2 * n)) : 0;
-        for (int p = 0; p < 2; p++)
-            for (int i = 0; i < lo; i++) {
-                const int r = p * lo + i;
-                m.dst_off[r] = uint16_t(r);
-                m.src_off[r] = lifts ? uint16_t(p * M + dpos[0]) : uint16_t(r);
-                m.prime[r] = uint8_t(i);
-                e.y_off[r] = uint16_t(p * M + i);
-                e.out_off[r] = uint16_t(r);
-                e.dinv[r] = dinv[i];
-                e.dinv_s[r] = dinv_s[i];
-            }
-        return lifts ? launch_ntt_lift_combine(c, y, lift, m, uint32_t(2 * lo) * count, lifts, e, s)
-                     : launch_ntt_fwd_combine(c, lift, m, uint32_t(2 * lo) * count, e, s);
+        const uint32_t limbs = k.lift.period * count;
+        return k.down_lifts
+                   ? launch_ntt_lift_combine(c, y, lift, k.lift, limbs, k.down_lifts, e, s)
+                   : launch_ntt_fwd_combine(c, lift, k.lift, limbs, e, s);
     }
-    CombineArgs a{};
+    CombineArgs a = k.comb;
     a.y = y;
-    a.lift = lifts ? nullptr : lift;
-    a.lifts = lifts;
-    a.y_last = size_t(dpos[0]) * n;
+    a.lift = k.down_lifts ? nullptr : lift;
     a.add = add;
     a.add_polys = add_polys;
+    a.add_item = add_item;
     a.galois = uint32_t(g);
     a.out = out;
-    a.y_item = size_t(2) * M * n;
-    a.y_poly = size_t(M) * n;
-    a.lift_item = size_t(2) * lo * n;
-    a.lift_poly = size_t(lo) * n;
-    a.add_item = add_item;
-    a.add_poly = size_t(lo) * n;
-    a.out_item = size_t(2) * lo * n;
-    a.out_poly = size_t(lo) * n;
-    a.lo = uint32_t(lo);
-    for (int i = 0; i < lo; i++) {
-        a.prime[i] = uint8_t(i);
-        a.dinv[i] = dinv[i];
-        a.dinv_s[i] = dinv_s[i];
-    }
     return launch_combine(c, a, count, s);
 }
 
@@ -516,6 +537,8 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
                          cudaStream_t s, const Gather *gth) {
     const uint64_t *rlk;
     TRY(key_for(keys, 0, &rlk));
+    const KsConsts *ks;
+    TRY(ks_consts(c, level, fused, &ks));
     const size_t n = c.n;
     TensorArgs t{};
     t.a = a;
@@ -537,23 +560,24 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(launch_tensor(c, t, count, s));
     LimbMap m = map_identity(uint32_t(level));
     TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(level) * count, s));
-    TRY(modup_ntt(c, k.d2c, size_t(level) * n, k.ext, count, level, false, s));
-    TRY(inner_product(c, k.ext, k.d2, rlk, k.d0, k.d1, size_t(level) * n, k.y, count, level, s));
-    return moddown(c, k.y, k.lift, out, count, level, fused, s, 0, gth);
+    TRY(modup_ntt(c, *ks, k.d2c, size_t(level) * n, k.ext, count, s));
+    TRY(inner_product(c, *ks, k.ext, k.d2, rlk, k.d0, k.d1, size_t(level) * n, k.y, count, s));
+    return moddown(c, *ks, k.y, k.lift, out, count, s, 0, gth);
 }
 
-// BFV: lift to Q u B, NTT, tensor, INTT, exact round(t x / Q) back to Q,
-// then relinearise d2 in coefficient form.
-static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
-                         uint64_t *out, uint32_t count, int level, KsBufs &k, cudaStream_t s) {
-    const uint64_t *rlk;
-    TRY(key_for(keys, 0, &rlk));
-    const size_t n = c.n;
+// A BFV multiplication's constants at one level, kept like KsConsts.
+struct BfvConsts {
+    ConvPlans lift;       // Q_l -> B
+    LimbMap in{};         // an input's q limbs into xin
+    LimbMap mb{}, mq{};   // the b limbs of Q u B; all of them
+    PlanRef pa, pb, pe;   // scale-and-round: both plans, and the exact one of z
+    MmaRef ma, mz;        // its tensor-core form
+    bool mma = false;
+};
+
+static int build_bfv(Context &c, int level, BfvConsts &k) {
     const int kb = level + c.nb;
-    // 1. the 4 input polys over Q_l u B in NTT form: the q limbs transformed
-    // straight from the inputs, the b limbs from their centred lift
-    uint64_t *xb = k.xin + size_t(count) * 2 * kb * n;  // b's half of xin
-    LimbMap mb{}, mq{};  // the b limbs of xin; all of them
+    LimbMap &mb = k.mb, &mq = k.mq;
     mb.period = uint32_t(c.nb);
     mq.period = uint32_t(kb);
     mb.src_stride = mb.dst_stride = mq.src_stride = mq.dst_stride = uint32_t(kb);
@@ -564,30 +588,85 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
         mb.src_off[i - level] = mb.dst_off[i - level] = uint16_t(i);
         mb.prime[i - level] = mq.prime[i];
     }
-    {
-        PlanSpec sp;
-        sp.lazy = true;  // NTT'd before the tensor
-        for (int i = 0; i < level; i++) {
-            sp.src_mod.push_back(c.mod(i));
-            sp.src_off.push_back(uint32_t(i));
-        }
-        for (int j = 0; j < c.nb; j++) {
-            sp.dst_mod.push_back(c.mod(c.pb(j)));
-            sp.dst_off.push_back(uint32_t(level + j));
-        }
-        ConvPlans pl{};
-        TRY(make_list(c, {{"bfv_lift/" + std::to_string(level), sp}}, pl));
-        LimbMap in = map_identity(uint32_t(level));
-        in.dst_stride = uint32_t(kb);
-        // items: (ct, poly) of a, then of b
-        for (int h = 0; h < 2; h++) {
-            const uint64_t *src = h ? b : a;
-            uint64_t *dst = h ? xb : k.xin;
-            TRY(launch_conv(c, pl, src, size_t(level) * n, 0, dst, size_t(kb) * n, 0, 2 * count, s));
-            TRY(launch_ntt_fwd(c, src, dst, in, uint32_t(level) * 2 * count, s));
-        }
+    k.in = map_identity(uint32_t(level));
+    k.in.dst_stride = uint32_t(kb);
+    const std::string l = std::to_string(level);
+    PlanSpec A, B, sp;
+    std::vector<uint64_t> tq;
+    sp.lazy = true;  // NTT'd before the tensor
+    for (int i = 0; i < level; i++) {
+        sp.src_mod.push_back(c.mod(i));
+        sp.src_off.push_back(uint32_t(i));
+        A.src_mod.push_back(c.mod(i));
+        A.src_off.push_back(uint32_t(i));
+        A.pre.push_back(c.t % c.mod(i));
+        B.dst_mod.push_back(c.mod(i));
+        B.dst_off.push_back(uint32_t(i));
     }
-    TRY(launch_ntt_fwd(c, k.xin, k.xin, mb, uint32_t(c.nb) * 4 * count, s));
+    PlanSpec Am = A, Bm = B, Be = B;
+    for (int j = 0; j < c.nb; j++) {
+        const uint64_t bj = c.mod(c.pb(j));
+        const uint64_t qinv = h_invmod(prod_mod(c, 0, level, bj), bj);
+        const uint64_t tqi = h_mulmod(c.t % bj, qinv, bj);
+        sp.dst_mod.push_back(bj);
+        sp.dst_off.push_back(uint32_t(level + j));
+        A.dst_mod.push_back(bj);
+        A.dst_off.push_back(uint32_t(level + j));
+        A.post.push_back(qinv);
+        tq.push_back(tqi);
+        tq.push_back(h_shoup(tqi, bj));
+        B.src_mod.push_back(bj);
+        B.src_off.push_back(0);
+        // the tensor-core form: A's results times (B/b_j)^-1 meet the digits of
+        // B's conversion, whose sources are x_b times t Q^-1
+        uint64_t rest = 1;  // B / b_j mod b_j
+        for (int i = 0; i < c.nb; i++)
+            if (i != j) rest = h_mulmod(rest, c.mod(c.pb(i)) % bj, bj);
+        Am.dst_mod.push_back(bj);
+        Am.dst_off.push_back(uint32_t(j));
+        Am.post.push_back(h_mulmod(qinv, h_invmod(rest, bj), bj));
+        Bm.src_mod.push_back(bj);
+        Bm.src_off.push_back(uint32_t(level + j));
+        Bm.pre.push_back(tqi);
+        Be.src_mod.push_back(bj);
+        Be.src_off.push_back(uint32_t(j));
+        Be.pre.push_back(rest);
+    }
+    TRY(make_list(c, {{"bfv_lift/" + l, sp}}, k.lift));
+    // the fused kernels need both conversions in the Montgomery layout
+    if (!plan_fits_mont(A) || !plan_fits_mont(B)) return CATFHE_EINVAL;
+    k.pa = get_plan_extra(c, "bfv_sr_a/" + l, A, tq);
+    k.pb = get_plan(c, "bfv_sr_b/" + l, B);
+    k.pe = get_plan(c, "bfv_sr_e/" + l, Be);
+    if (!k.pa.p || !k.pb.p || !k.pe.p) return CATFHE_ENOMEM;
+    k.ma = get_mma_plan(c, "bfv_sr_a/" + l, Am, 1);
+    k.mz = get_mma_plan(c, "bfv_sr_b/" + l, Bm, c.n);
+    k.mma = bfv_round_mma_fits(k.ma, k.mz);
+    return CATFHE_OK;
+}
+
+// BFV: lift to Q u B, NTT, tensor, INTT, exact round(t x / Q) back to Q,
+// then relinearise d2 in coefficient form.
+static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
+                         uint64_t *out, uint32_t count, int level, KsBufs &k, cudaStream_t s) {
+    const uint64_t *rlk;
+    TRY(key_for(keys, 0, &rlk));
+    const KsConsts *ks;
+    const BfvConsts *bc;
+    TRY(ks_consts(c, level, false, &ks));
+    TRY(kept(c, c.bfv, level, &bc, [&](BfvConsts &b) { return build_bfv(c, level, b); }));
+    const size_t n = c.n;
+    const int kb = level + c.nb;
+    // 1. the 4 input polys over Q_l u B in NTT form: the q limbs transformed
+    // straight from the inputs, the b limbs from their centred lift
+    uint64_t *xb = k.xin + size_t(count) * 2 * kb * n;  // b's half of xin
+    for (int h = 0; h < 2; h++) {  // items: (ct, poly) of a, then of b
+        const uint64_t *src = h ? b : a;
+        uint64_t *dst = h ? xb : k.xin;
+        TRY(launch_conv(c, bc->lift, src, size_t(level) * n, 0, dst, size_t(kb) * n, 0, 2 * count, s));
+        TRY(launch_ntt_fwd(c, src, dst, bc->in, uint32_t(level) * 2 * count, s));
+    }
+    TRY(launch_ntt_fwd(c, k.xin, k.xin, bc->mb, uint32_t(c.nb) * 4 * count, s));
     // 2. tensor over Q u B
     {
         TensorArgs t{};
@@ -599,70 +678,21 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
         t.d2 = k.tens + size_t(2) * kb * n;
         t.out_item = size_t(3) * kb * n;
         t.limbs = uint32_t(kb);
-        for (int i = 0; i < kb; i++) t.prime[i] = mq.prime[i];
+        for (int i = 0; i < kb; i++) t.prime[i] = bc->mq.prime[i];
         TRY(launch_tensor(c, t, count, s));
     }
-    TRY(launch_ntt_inv(c, k.tens, k.tens, mq, uint32_t(kb) * 3 * count, s));
+    TRY(launch_ntt_inv(c, k.tens, k.tens, bc->mq, uint32_t(kb) * 3 * count, s));
     // 3. exact round(t x / Q) back to Q_l
-    {
-        PlanSpec A, B;
-        std::vector<uint64_t> tq;
-        for (int i = 0; i < level; i++) {
-            A.src_mod.push_back(c.mod(i));
-            A.src_off.push_back(uint32_t(i));
-            A.pre.push_back(c.t % c.mod(i));
-        }
-        for (int j = 0; j < c.nb; j++) {
-            const uint64_t bj = c.mod(c.pb(j));
-            const uint64_t qinv = h_invmod(prod_mod(c, 0, level, bj), bj);
-            A.dst_mod.push_back(bj);
-            A.dst_off.push_back(uint32_t(level + j));
-            A.post.push_back(qinv);
-            const uint64_t tqi = h_mulmod(c.t % bj, qinv, bj);
-            tq.push_back(tqi);
-            tq.push_back(h_shoup(tqi, bj));
-            B.src_mod.push_back(bj);
-            B.src_off.push_back(0);
-        }
-        for (int i = 0; i < level; i++) {
-            B.dst_mod.push_back(c.mod(i));
-            B.dst_off.push_back(uint32_t(i));
-        }
-        // the fused kernel needs both conversions in the Montgomery layout
-        if (!plan_fits_mont(A) || !plan_fits_mont(B)) return CATFHE_EINVAL;
-        const PlanRef pa = get_plan_extra(c, "bfv_sr_a/" + std::to_string(level), A, tq);
-        const PlanRef pb = get_plan(c, "bfv_sr_b/" + std::to_string(level), B);
-        if (!pa.p || !pb.p) return CATFHE_ENOMEM;
-        // the tensor-core form: A's results times (B/b_j)^-1 meet the digits of
-        // b's conversion, whose sources are x_b times t Q^-1
-        const std::string key = "bfv_sr/" + std::to_string(level);
-        PlanSpec Am = A, Bm = B, Be = B;
-        for (int j = 0; j < c.nb && !c.mma_plans.count(key + "/a"); j++) {
-            const uint64_t bj = c.mod(c.pb(j));
-            uint64_t rest = 1;  // B / b_j mod b_j
-            for (int l = 0; l < c.nb; l++)
-                if (l != j) rest = h_mulmod(rest, c.mod(c.pb(l)) % bj, bj);
-            Am.dst_off[size_t(j)] = uint32_t(j);
-            Am.post[size_t(j)] = h_mulmod(A.post[size_t(j)], h_invmod(rest, bj), bj);
-            Bm.src_off[size_t(j)] = uint32_t(level + j);
-            Bm.pre.push_back(tq[2 * size_t(j)]);
-            Be.src_off[size_t(j)] = uint32_t(j);
-            Be.pre.push_back(rest);
-        }
-        const MmaRef ma = get_mma_plan(c, key + "/a", Am, 1), mb2 = get_mma_plan(c, key + "/b", Bm, n);
-        if (bfv_round_mma_fits(ma, mb2)) {
-            const PlanRef pe = get_plan(c, key + "/b/exact", Be);
-            if (!pe.p) return CATFHE_ENOMEM;
-            TRY(launch_bfv_round_mma(c, ma, pa.p, mb2, pe.p, k.tens, size_t(kb) * n, k.dq,
-                                     size_t(level) * n, 3 * count, s));
-        } else
-            TRY(launch_bfv_scale_round(c, pa.p, pa.words, pb.p, pb.words, k.tens, size_t(kb) * n, k.dq,
-                                   size_t(level) * n, 3 * count, s));
-    }
+    if (bc->mma)
+        TRY(launch_bfv_round_mma(c, bc->ma, bc->pa.p, bc->mz, bc->pe.p, k.tens, size_t(kb) * n, k.dq,
+                                 size_t(level) * n, 3 * count, s));
+    else
+        TRY(launch_bfv_scale_round(c, bc->pa.p, bc->pa.words, bc->pb.p, bc->pb.words, k.tens,
+                                   size_t(kb) * n, k.dq, size_t(level) * n, 3 * count, s));
     // 4. relinearise d2' (coefficient form) and add (d0', d1')
     const uint64_t *d2 = k.dq + size_t(2) * level * n;
-    TRY(modup_ntt(c, d2, size_t(3) * level * n, k.ext, count, level, true, s));
-    TRY(inner_product(c, k.ext, nullptr, rlk, nullptr, nullptr, 0, k.y, count, level, s));
+    TRY(modup_ntt(c, *ks, d2, size_t(3) * level * n, k.ext, count, s));
+    TRY(inner_product(c, *ks, k.ext, nullptr, rlk, nullptr, nullptr, 0, k.y, count, s));
     {
         const int M = level + c.K;
         LimbMap my = map_identity(uint32_t(M));
@@ -670,8 +700,7 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
     // (d0', d1') are the first two of each ciphertext's three polynomials
-    return moddown(c, k.y, k.lift, out, count, level, false, s, 0, nullptr, k.dq, 2,
-                   size_t(3) * level * n);
+    return moddown(c, *ks, k.y, k.lift, out, count, s, 0, nullptr, k.dq, 2, size_t(3) * level * n);
 }
 
 // Two streams (and fork / join events) per device for split operations;
@@ -777,6 +806,8 @@ static LimbMap map_second(int lvl) {
 static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_t g, uint64_t *out,
                       int lvl, uint32_t count, KsBufs &k, cudaStream_t s, const Gather *gth) {
     const size_t n = c.n, item = size_t(2) * lvl * n, half = size_t(lvl) * n;
+    const KsConsts *ks;
+    TRY(ks_consts(c, lvl, false, &ks));
     if (c.scheme != CATFHE_BFV) {
         LimbMap m = map_second(lvl);
         if (gth && gth->n) {
@@ -784,9 +815,9 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
             for (uint32_t i = 0; i < gth->n; i++) m.gsrc[i] = gth->a[i];
         }
         TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(lvl) * count, s));
-        TRY(modup_ntt(c, k.d2c, half, k.ext, count, lvl, false, s));
-        TRY(inner_product(c, k.ext, a + half, gk, a, nullptr, item, k.y, count, lvl, s, gth));
-        return moddown(c, k.y, k.lift, out, count, lvl, false, s, g, gth);
+        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+        TRY(inner_product(c, *ks, k.ext, a + half, gk, a, nullptr, item, k.y, count, s, gth));
+        return moddown(c, *ks, k.y, k.lift, out, count, s, g, gth);
     }
     // BFV (coefficient form): a1 is key switched, a0 added by the combine.  It
     // scatters its results, so a0 is copied first when out overlaps a.
@@ -798,15 +829,15 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
                               uint32_t(2 * lvl) * count, s));
         add = k.add;
     }
-    TRY(modup_ntt(c, a + half, item, k.ext, count, lvl, true, s));
-    TRY(inner_product(c, k.ext, nullptr, gk, nullptr, nullptr, 0, k.y, count, lvl, s));
+    TRY(modup_ntt(c, *ks, a + half, item, k.ext, count, s));
+    TRY(inner_product(c, *ks, k.ext, nullptr, gk, nullptr, nullptr, 0, k.y, count, s));
     {
         const int M = lvl + c.K;
         LimbMap my = map_identity(uint32_t(M));
         for (int i = 0; i < M; i++) my.prime[i] = uint8_t(ext_prime(c, lvl, i));
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
-    return moddown(c, k.y, k.lift, out, count, lvl, false, s, g, nullptr, add, 1, item);
+    return moddown(c, *ks, k.y, k.lift, out, count, s, g, nullptr, add, 1, item);
 }
 
 int op_rotate(Context &c, const Keys &keys, const uint64_t *a, uint64_t g, uint64_t *out,
@@ -869,11 +900,12 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     // a1 (NTT form) -> coefficient form -> lifted digits in NTT form, once
     const size_t item = size_t(2) * lvl * n, half = size_t(lvl) * n;
     TRY(launch_ntt_inv(c, a, k.d2c, map_second(lvl), uint32_t(lvl) * count, s));
-    TRY(modup_ntt(c, k.d2c, half, ext0, count, lvl, false, s));
+    const KsConsts *kc;
+    TRY(ks_consts(c, lvl, false, &kc));
+    TRY(modup_ntt(c, *kc, k.d2c, half, ext0, count, s));
     auto one = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
-        TRY(inner_product(c, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, lvl, st));
-        return moddown(c, kb.y, kb.lift, out + size_t(r) * count * item, count, lvl, false, st,
-                       gv[r]);
+        TRY(inner_product(c, *kc, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, st));
+        return moddown(c, *kc, kb.y, kb.lift, out + size_t(r) * count * item, count, st, gv[r]);
     };
     if (n_rot < 2 || c.log_n < 14) {
         for (uint32_t r = 0; r < n_rot; r++) TRY(one(r, k, s));
@@ -895,6 +927,40 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     return CATFHE_OK;
 }
 
+// A rescale's constants at one level, kept like KsConsts.
+struct RescaleConsts {
+    LimbMap last{}, lift{};
+    NttEpilogue epi{};
+    const LiftEntry *lifts = nullptr;
+};
+
+static int build_rescale(Context &c, int lvl, RescaleConsts &k) {
+    const int lo = lvl - 1;
+    LimbMap &m = k.last, &l = k.lift;
+    NttEpilogue &e = k.epi;
+    m.period = m.dst_stride = l.src_stride = 2;
+    m.src_stride = e.y_stride = uint32_t(2 * lvl);
+    l.period = l.dst_stride = e.out_stride = uint32_t(2 * lo);
+    e.status = c.d_status;
+    for (int p = 0; p < 2; p++) {
+        m.src_off[p] = uint16_t(p * lvl + lvl - 1);
+        m.dst_off[p] = uint16_t(p);
+        m.prime[p] = uint8_t(lvl - 1);
+        for (int i = 0; i < lo; i++) {
+            const int r = p * lo + i;
+            l.src_off[r] = uint16_t(p);
+            l.dst_off[r] = uint16_t(r);
+            l.prime[r] = uint8_t(i);
+            e.y_off[r] = uint16_t(p * lvl + i);
+            e.out_off[r] = uint16_t(r);
+            e.dinv[r] = p ? e.dinv[i] : h_invmod(c.mod(lvl - 1) % c.mod(i), c.mod(i));
+            e.dinv_s[r] = h_shoup(e.dinv[r], c.mod(i));
+        }
+    }
+    k.lifts = upload_lifts(c, division_lifts(c, lvl - 1, lo));
+    return k.lifts ? CATFHE_OK : CATFHE_ENOMEM;
+}
+
 // CKKS rescale / BGV modulus switch: divide by q_{l-1}.
 int op_rescale(Context &c, const uint64_t *a, uint64_t *out, uint32_t level, uint32_t count,
                void *ws, size_t ws_bytes_in, cudaStream_t s) {
@@ -908,44 +974,16 @@ int op_rescale(Context &c, const uint64_t *a, uint64_t *out, uint32_t level, uin
     const int lvl = int(level), lo = lvl - 1;
     uint64_t *last = bump.take<uint64_t>(size_t(count) * 2 * n);
     uint64_t *lift = bump.take<uint64_t>(size_t(count) * 2 * lo * n);
+    const RescaleConsts *k;
+    TRY(kept(c, c.rescale, lvl, &k, [&](RescaleConsts &r) { return build_rescale(c, lvl, r); }));
     // INTT of the last limb of both polys: [count][2][level] -> [count][2][1]
-    LimbMap m{};
-    m.period = 2;
-    m.src_stride = uint32_t(2 * lvl);
-    m.dst_stride = 2;
-    for (int p = 0; p < 2; p++) {
-        m.src_off[p] = uint16_t(p * lvl + lvl - 1);
-        m.dst_off[p] = uint16_t(p);
-        m.prime[p] = uint8_t(lvl - 1);
-    }
-    TRY(launch_ntt_inv(c, a, last, m, 2 * count, s));
-    const LiftEntry *lifts = get_lifts(c, "rescale/" + std::to_string(lvl),
-                                       [&] { return division_lifts(c, lvl - 1, lo); });
-    if (!lifts) return CATFHE_ENOMEM;
+    TRY(launch_ntt_inv(c, a, last, k->last, 2 * count, s));
     // NTT of the lift (lifted as it loads), its last pass writing
     // (a - lift) q_{l-1}^-1 to out
-    LimbMap m2{};
-    NttEpilogue e{};
-    m2.period = uint32_t(2 * lo);
-    m2.src_stride = 2;
-    m2.dst_stride = uint32_t(2 * lo);
+    NttEpilogue e = k->epi;
     e.y = a;
     e.out = out;
-    e.status = c.d_status;
-    e.y_stride = uint32_t(2 * lvl);
-    e.out_stride = uint32_t(2 * lo);
-    for (int p = 0; p < 2; p++)
-        for (int i = 0; i < lo; i++) {
-            const int r = p * lo + i;
-            m2.src_off[r] = uint16_t(p);
-            m2.dst_off[r] = uint16_t(r);
-            m2.prime[r] = uint8_t(i);
-            e.y_off[r] = uint16_t(p * lvl + i);
-            e.out_off[r] = uint16_t(r);
-            e.dinv[r] = h_invmod(c.mod(lvl - 1) % c.mod(i), c.mod(i));
-            e.dinv_s[r] = h_shoup(e.dinv[r], c.mod(i));
-        }
-    return launch_ntt_lift_combine(c, last, lift, m2, uint32_t(2 * lo) * count, lifts, e, s);
+    return launch_ntt_lift_combine(c, last, lift, k->lift, uint32_t(2 * lo) * count, k->lifts, e, s);
 }
 
 int op_add(Context &c, const uint64_t *a, const uint64_t *b, uint64_t *out, uint32_t level,
@@ -1481,6 +1519,7 @@ static int decrypt_device(Context &c, const Keys &k, const uint64_t *ct, uint32_
     if (c.scheme == CATFHE_CKKS) {
         sp.dst_mod.push_back(0);
         if (plan_fits_mont(sp)) {
+            std::lock_guard<std::mutex> lock(c.mu);
             const PlanRef exact = get_plan(c, key, sp);
             if (!exact.p) return CATFHE_ENOMEM;
             const std::string wkey = key + "/wrap";
@@ -1499,7 +1538,10 @@ static int decrypt_device(Context &c, const Keys &k, const uint64_t *ct, uint32_
         }
     }
     ConvPlans pl{};
-    TRY(make_list(c, {{key, sp}}, pl));
+    {
+        std::lock_guard<std::mutex> lock(c.mu);
+        TRY(make_list(c, {{key, sp}}, pl));
+    }
     return launch_conv(c, pl, x, 0, 0, reinterpret_cast<uint64_t *>(res), 0, 0, 1, s);
 }
 
@@ -1542,13 +1584,15 @@ int op_encode_ckks(Context &c, const double *slots, double scale, uint32_t level
     // every limb's transform reduces the signed coefficients as it loads them
     LimbMap mp = map_identity(level);
     for (uint32_t i = 0; i < level; i++) mp.src_off[i] = 0;
-    const LiftEntry *lifts = get_lifts(c, "signed", [&] {
+    {
+        std::lock_guard<std::mutex> lock(c.mu);
         LiftEntry e{};
         e.flags = kLiftSigned;
-        return std::vector<LiftEntry>(size_t(c.L), e);
-    });
-    if (!lifts) return CATFHE_ENOMEM;
-    TRY(launch_ntt_lift(c, reinterpret_cast<const uint64_t *>(m), pt, mp, level, lifts, false, s));
+        if (!c.signed_lifts) c.signed_lifts = upload_lifts(c, std::vector<LiftEntry>(size_t(c.L), e));
+        if (!c.signed_lifts) return CATFHE_ENOMEM;
+    }
+    TRY(launch_ntt_lift(c, reinterpret_cast<const uint64_t *>(m), pt, mp, level, c.signed_lifts,
+                        false, s));
     return cudaStreamSynchronize(s) == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 
