@@ -23,6 +23,7 @@
 
 #include <vector>
 
+#include "launch.cuh"
 #include "modarith.cuh"
 
 namespace catfhe {
@@ -51,6 +52,7 @@ __global__ void __launch_bounds__(kFftPts / 2)
 k_fft_low(const double2 *__restrict__ z, double scale, const uint32_t *__restrict__ slot,
           const int64_t *__restrict__ m, const double2 *__restrict__ twist,
           const double2 *__restrict__ tw, double2 *__restrict__ out, uint32_t log_n) {
+    grid_dep_wait();
     __shared__ double2 x[kFftPts];
     const uint32_t t = threadIdx.x, i0 = blockIdx.x * kFftPts;
 #pragma unroll
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(kFftPts / 2)
 k_fft_high(const double2 *__restrict__ in, const double2 *__restrict__ tw,
            const double2 *__restrict__ twist, double scale, int64_t *__restrict__ m,
            const uint32_t *__restrict__ slot, double2 *__restrict__ z, uint32_t log_n) {
+    grid_dep_wait();
     __shared__ double2 x[kFftPts];
     const uint32_t t = threadIdx.x, lb = log_n - kFftLow, lc = 9 - lb;  // log rows, log columns
     const uint32_t c0 = blockIdx.x << lc, cm = (1u << lc) - 1;
@@ -161,10 +164,10 @@ int launch_encode_ckks(const Context &c, const double2 *slots, double scale, dou
     const size_t n = c.n;
     const uint32_t lg = uint32_t(c.log_n), ctas = uint32_t(n / kFftPts);
     const double2 *twist = c.d_enc, *tw = c.d_enc + n + n / 2;
-    k_fft_low<true><<<ctas, kFftPts / 2, 0, s>>>(slots, scale, c.d_slot, nullptr, nullptr, tw, buf,
-                                                 lg);
-    k_fft_high<true><<<ctas, kFftPts / 2, 0, s>>>(buf, tw, twist, 1.0 / double(n), m, nullptr,
-                                                  nullptr, lg);
+    launch_pdl(k_fft_low<true>, dim3(ctas), dim3(kFftPts / 2), 0, s, slots, scale, c.d_slot, m,
+               twist, tw, buf, lg);
+    launch_pdl(k_fft_high<true>, dim3(ctas), dim3(kFftPts / 2), 0, s, buf, tw, twist,
+               1.0 / double(n), m, c.d_slot, buf, lg);
     note_launches(2);
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
@@ -174,9 +177,10 @@ int launch_decode_ckks(const Context &c, const int64_t *m, double inv_scale, dou
     const size_t n = c.n;
     const uint32_t lg = uint32_t(c.log_n), ctas = uint32_t(n / kFftPts);
     const double2 *twist = c.d_enc, *tw = c.d_enc + n;
-    k_fft_low<false><<<ctas, kFftPts / 2, 0, s>>>(nullptr, 0.0, nullptr, m, twist, tw, buf, lg);
-    k_fft_high<false><<<ctas, kFftPts / 2, 0, s>>>(buf, tw, nullptr, inv_scale, nullptr, c.d_slot,
-                                                   slots, lg);
+    launch_pdl(k_fft_low<false>, dim3(ctas), dim3(kFftPts / 2), 0, s, buf, 0.0, c.d_slot, m, twist,
+               tw, buf, lg);
+    launch_pdl(k_fft_high<false>, dim3(ctas), dim3(kFftPts / 2), 0, s, buf, tw, twist, inv_scale,
+               (int64_t *)nullptr, c.d_slot, slots, lg);
     note_launches(2);
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
