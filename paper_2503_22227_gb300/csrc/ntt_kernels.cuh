@@ -650,11 +650,13 @@ static int run_inv(const Context &c, const uint64_t *src, uint64_t *dst, const L
 // threads x 16 CTAs per SM (up to 128 registers) was the fastest for the
 // largest class: forward plus inverse 111.2 against 116.1 us (2^13, 16
 // ciphertexts of 24 primes), 228.2 against 237.1 (2^14), 452.5 against
-// 464.4 (2^15).
+// 464.4 (2^15).  At 2^12 columns of 128 x 6 beat 256 x 3 in every class:
+// forward plus inverse 12.0 against 12.7 us (4 limbs), 17.0 against 18.4 (96),
+// 41.7 against 43.0 (480).
 #define NTT_SCHEDULES(X)                                                                         \
-    X(12, 0, 6, 3, 256, 3, 6, 3, 128, 4) X(12, 1, 6, 3, 256, 3, 6, 3, 256, 3)                    \
+    X(12, 0, 6, 3, 128, 6, 6, 3, 128, 4) X(12, 1, 6, 3, 256, 3, 6, 3, 256, 3)                    \
     X(12, 2, 5, 3, 256, 3, 7, 4, 128, 4) X(12, 3, 7, 4, 256, 3, 5, 3, 128, 4)                    \
-    X(12, 4, 6, 3, 128, 6, 6, 3, 128, 4)                                                         \
+    X(12, 4, 6, 3, 256, 3, 6, 3, 128, 4)                                                         \
     X(13, 0, 7, 4, 128, 6, 6, 3, 32, 16) X(13, 1, 7, 4, 256, 3, 6, 3, 64, 8)                     \
     X(13, 2, 7, 4, 256, 3, 6, 3, 256, 3) X(13, 3, 6, 3, 256, 3, 7, 4, 128, 4)                    \
     X(13, 4, 7, 4, 128, 6, 6, 3, 128, 4) X(13, 5, 7, 4, 256, 3, 6, 3, 128, 4)                    \
