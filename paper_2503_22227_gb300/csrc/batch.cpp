@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "lanes.h"
 
 
 namespace catfhe {
@@ -295,6 +296,7 @@ int run_plan(const catfhe_op *ops, const Plan &p, char *ws, cudaStream_t s) {
     int rc = lane_pool(&pool);
     if (rc) return rc;
     const size_t lanes = p.lane_units.size();
+    LaneScope scope(lanes > 1);
     if (cudaEventRecord(pool->start, s) != cudaSuccess) return CATFHE_ECUDA;
     size_t off = 0;
     for (size_t l = 0; l < lanes; l++) {

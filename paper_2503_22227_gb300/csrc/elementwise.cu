@@ -78,7 +78,7 @@ k_tensor(const TensorArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
 }
 
 int launch_tensor(const Context &c, const TensorArgs &a, uint32_t count, cudaStream_t s) {
-    launch_pdl(k_tensor, coeff_grid(c.n / 2, a.limbs, count), dim3(256), 0, s, a, c.d_mods, c.log_n);
+    launch_pdl_split(kSharedPercent, k_tensor, coeff_grid(c.n / 2, a.limbs, count), dim3(256), 0, s, a, c.d_mods, c.log_n);
     return ok();
 }
 
