@@ -154,23 +154,33 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
 // coefficients (256 threads) up to 4 digits; 256 coefficients (128 threads)
 // for 5 to 8 digits, so that the 2 BETA key tiles and the two buffers
 // (72 KB at BETA = 8) leave room for 3 CTAs per SM.
-template <int BETA>
+template <int BETA, int R>
 struct IpTile {
-    static constexpr uint32_t value = BETA <= 4 ? 512 : 256;
+    static constexpr uint32_t value = BETA * R <= 4 ? 512 : 256;
 };
 
 // blockIdx.z: a group of consecutive ciphertexts of the launch (the host
 // splits them when one group per tile would leave the last wave of CTAs
 // mostly empty); each group's CTA loads its key tiles once.
-template <int BETA, bool GATHER>
-__global__ void __launch_bounds__(IpTile<BETA>::value / 2)
+// R: keys of the launch.  Hoisted rotations multiply the same digits by one
+// key each; with two keys the digits and the first polynomials of 8
+// ciphertexts at N = 2^16, l = 24 (453 MB) are read once for both, 1550 ->
+// 1098 MB a pair.  Tiles of 256
+// coefficients from 3 digits on, so that the key tiles and the two buffers
+// (44 KB at 3 digits) leave room for 3 CTAs per SM in the 164 KB split that
+// these launches ask for (tiles of 512 are slower, 8080 instead of 8023 us).
+// The batch of 16 rotations of 8: 8128 -> 8023 us (the transforms that run
+// beside it bound it); 16 rotations of one: 1349 -> 1267 us; 4 at N = 2^12:
+// 57.0 -> 52.7 us; 2 or 3 rotations at N >= 2^14 stay one to each stream.
+template <int BETA, bool GATHER, int R>
+__global__ void __launch_bounds__(IpTile<BETA, R>::value / 2)
 k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint32_t count) {
     grid_dep_wait();
     const uint32_t per = (count + gridDim.z - 1) / gridDim.z;
     const uint32_t first = blockIdx.z * per;
     if (first >= count) return;  // an empty group (the whole CTA, before any barrier)
     const uint32_t nloc = count - first < per ? count - first : per;
-    constexpr uint32_t kIpTile = IpTile<BETA>::value;
+    constexpr uint32_t kIpTile = IpTile<BETA, R>::value;
     extern __shared__ __align__(128) uint64_t sm[];
     __shared__ __align__(8) uint64_t bars[3];  // buffer 0, buffer 1, keys
     const size_t n = size_t(1) << log_n;
@@ -182,8 +192,8 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
     const bool f0 = fold && A.add0, f1 = fold && A.add1;
     const uint32_t own_digit = (A.own != nullptr && i < A.level) ? i / A.alpha : 0xffffffffu;
     constexpr uint32_t TB = kIpTile * 8;  // bytes per tile
-    uint64_t *skey = sm;                                   // [2 BETA][tile]
-    uint64_t *sbuf[2] = {sm + 2 * BETA * kIpTile, sm + (3 * BETA + 2) * kIpTile};
+    uint64_t *skey = sm;                                   // [R][2 BETA][tile]
+    uint64_t *sbuf[2] = {sm + 2 * R * BETA * kIpTile, sm + ((2 * R + 1) * BETA + 2) * kIpTile};
     const uint32_t item_bytes = (beta + (f0 ? 1 : 0) + (f1 ? 1 : 0)) * TB;
 
     auto issue_item = [&](uint32_t k, uint32_t b) {  // the group's k-th ciphertext
@@ -208,10 +218,15 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
     }
     __syncthreads();
     if (tid == 0) {
-        mbar_expect_tx(&bars[2], 2 * beta * TB);
-        for (uint32_t j = 0; j < beta; j++) {
-            bulk_load(skey + (2 * j) * kIpTile, A.key + ((size_t(j) * 2 + 0) * KL + A.key_limb[i]) * n + x0, TB, &bars[2]);
-            bulk_load(skey + (2 * j + 1) * kIpTile, A.key + ((size_t(j) * 2 + 1) * KL + A.key_limb[i]) * n + x0, TB, &bars[2]);
+        mbar_expect_tx(&bars[2], 2 * R * beta * TB);
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            const uint64_t *key = r ? A.key2 : A.key;
+            uint64_t *dst = skey + r * 2 * BETA * kIpTile;
+            for (uint32_t j = 0; j < beta; j++) {
+                bulk_load(dst + (2 * j) * kIpTile, key + ((size_t(j) * 2 + 0) * KL + A.key_limb[i]) * n + x0, TB, &bars[2]);
+                bulk_load(dst + (2 * j + 1) * kIpTile, key + ((size_t(j) * 2 + 1) * KL + A.key_limb[i]) * n + x0, TB, &bars[2]);
+            }
         }
         issue_item(0, 0);
         if (nloc > 1) issue_item(1, 1);
@@ -225,33 +240,37 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
         ok = __syncthreads_and(mbar_wait(&bars[b], (k >> 1) & 1));
         if (!ok) break;
         const uint64_t *buf = sbuf[b];
-        U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
-        if (f0) {
-            const ulonglong2 d = ld2(buf + BETA * kIpTile + u);
-            mac(a0, d.x, A.pfac[i]);
-            mac(a1, d.y, A.pfac[i]);
-        }
-        if (f1) {
-            const ulonglong2 d = ld2(buf + (BETA + 1) * kIpTile + u);
-            mac(b0, d.x, A.pfac[i]);
-            mac(b1, d.y, A.pfac[i]);
-        }
 #pragma unroll
-        for (int j = 0; j < BETA; j++) {
-            if (uint32_t(j) < beta) {
-                const ulonglong2 c = ld2(buf + j * kIpTile + u);
-                const ulonglong2 kb = ld2(skey + (2 * j) * kIpTile + u);
-                const ulonglong2 ka = ld2(skey + (2 * j + 1) * kIpTile + u);
-                mac(a0, c.x, kb.x);
-                mac(a1, c.y, kb.y);
-                mac(b0, c.x, ka.x);
-                mac(b1, c.y, ka.y);
+        for (int r = 0; r < R; r++) {
+            const uint64_t *key = skey + r * 2 * BETA * kIpTile;
+            U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
+            if (f0) {
+                const ulonglong2 d = ld2(buf + BETA * kIpTile + u);
+                mac(a0, d.x, A.pfac[i]);
+                mac(a1, d.y, A.pfac[i]);
             }
+            if (f1) {
+                const ulonglong2 d = ld2(buf + (BETA + 1) * kIpTile + u);
+                mac(b0, d.x, A.pfac[i]);
+                mac(b1, d.y, A.pfac[i]);
+            }
+#pragma unroll
+            for (int j = 0; j < BETA; j++) {
+                if (uint32_t(j) < beta) {
+                    const ulonglong2 c = ld2(buf + j * kIpTile + u);
+                    const ulonglong2 kb = ld2(key + (2 * j) * kIpTile + u);
+                    const ulonglong2 ka = ld2(key + (2 * j + 1) * kIpTile + u);
+                    mac(a0, c.x, kb.x);
+                    mac(a1, c.y, kb.y);
+                    mac(b0, c.x, ka.x);
+                    mac(b1, c.y, ka.y);
+                }
+            }
+            uint64_t *y = (r ? A.y2 : A.y) + item * A.y_item + x0 + u;
+            st2(y + size_t(i) * n, csub(redc(a0, m.q, m.qinv), m.q), csub(redc(a1, m.q, m.qinv), m.q));
+            st2(y + (size_t(A.M) + i) * n, csub(redc(b0, m.q, m.qinv), m.q),
+                csub(redc(b1, m.q, m.qinv), m.q));
         }
-        uint64_t *y = A.y + item * A.y_item + x0 + u;
-        st2(y + size_t(i) * n, csub(redc(a0, m.q, m.qinv), m.q), csub(redc(a1, m.q, m.qinv), m.q));
-        st2(y + (size_t(A.M) + i) * n, csub(redc(b0, m.q, m.qinv), m.q),
-            csub(redc(b1, m.q, m.qinv), m.q));
         __syncthreads();  // everyone is done with buffer b
         if (tid == 0 && k + 2 < nloc) {
             fence_proxy_async();
@@ -315,40 +334,45 @@ static unsigned ip_groups(K kernel, unsigned threads, size_t smem, size_t ctas, 
     return top >= 1.1 * one ? best : 1;
 }
 
-template <int BETA, bool GATHER>
+template <int BETA, bool GATHER, int R>
 static int ip_run_bulk(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
-    constexpr uint32_t tile = IpTile<BETA>::value;
+    constexpr uint32_t tile = IpTile<BETA, R>::value;
     // two buffers of the ciphertexts' tiles, one when each CTA has a single
     // ciphertext (then more CTAs are resident, 5 instead of 3 per SM at 3 digits:
     // one product at N = 2^16, l = 24 201.8 -> 199.4 us, the 256-operation mix
     // 9.70 -> 9.55 ms)
-    const auto kernel = k_ip_bulk<BETA, GATHER>;
+    const auto kernel = k_ip_bulk<BETA, GATHER, R>;
     const void *const k = reinterpret_cast<const void *>(kernel);
-    constexpr size_t two = size_t(4 * BETA + 4) * tile * 8, one = size_t(3 * BETA + 2) * tile * 8;
+    constexpr size_t one = size_t((2 * R + 1) * BETA + 2) * tile * 8, two = one + size_t(BETA + 2) * tile * 8;
     const unsigned groups =
         count > 1 ? ip_groups(kernel, tile / 2, two, c.n / tile * a.M, count) : 1;
     const size_t smem = groups >= count ? one : two;
     if (!allow_smem(k, two)) return CATFHE_ECUDA;
-    launch_pdl(kernel, dim3(unsigned(c.n / tile), a.M, groups), dim3(tile / 2), smem, s, a, c.d_mods,
-               uint32_t(c.log_n), count);
+    launch_pdl_split(R > 1 ? kSharedPercent : 0, kernel, dim3(unsigned(c.n / tile), a.M, groups),
+                     dim3(tile / 2), smem, s, a, c.d_mods, uint32_t(c.log_n), count);
     return ok();
 }
 
-template <bool GATHER>
+template <bool GATHER, int R>
 static int ip_run(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
     switch (a.beta) {
-        case 1: return ip_run_bulk<1, GATHER>(c, a, count, s);
-        case 2: return ip_run_bulk<2, GATHER>(c, a, count, s);
-        case 3: return ip_run_bulk<3, GATHER>(c, a, count, s);
-        case 4: return ip_run_bulk<4, GATHER>(c, a, count, s);
-        case 5: return ip_run_bulk<5, GATHER>(c, a, count, s);
-        case 6: return ip_run_bulk<6, GATHER>(c, a, count, s);
-        case 7: return ip_run_bulk<7, GATHER>(c, a, count, s);
-        case 8: return ip_run_bulk<8, GATHER>(c, a, count, s);
+        case 1:
+            if constexpr (R > 1) return CATFHE_EINVAL;  // one digit: not paired
+            else return ip_run_bulk<1, GATHER, R>(c, a, count, s);
+        case 2: return ip_run_bulk<2, GATHER, R>(c, a, count, s);
+        case 3: return ip_run_bulk<3, GATHER, R>(c, a, count, s);
+        case 4: return ip_run_bulk<4, GATHER, R>(c, a, count, s);
+        case 5: return ip_run_bulk<5, GATHER, R>(c, a, count, s);
+        case 6: return ip_run_bulk<6, GATHER, R>(c, a, count, s);
+        case 7: return ip_run_bulk<7, GATHER, R>(c, a, count, s);
+        case 8: return ip_run_bulk<8, GATHER, R>(c, a, count, s);
         default:
-            launch_pdl(k_ip_stream<GATHER>, dim3(count, unsigned((c.n / 2 + 255) / 256), a.M),
-                       dim3(256), 0, s, a, c.d_mods, uint32_t(c.log_n));
-            return ok();
+            if constexpr (R > 1) return CATFHE_EINVAL;
+            else {
+                launch_pdl(k_ip_stream<GATHER>, dim3(count, unsigned((c.n / 2 + 255) / 256), a.M),
+                           dim3(256), 0, s, a, c.d_mods, uint32_t(c.log_n));
+                return ok();
+            }
     }
 }
 
@@ -356,11 +380,13 @@ int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s)
     // bulk copies: every buffer is a workspace, a key or a ciphertext, refused
     // at the entry points unless 16-byte aligned
     bool aligned = a.status != nullptr && aligned16(a.ext) && aligned16(a.key) && aligned16(a.y) &&
-                   aligned16(a.own) && aligned16(a.add0) && aligned16(a.add1) &&
+                   aligned16(a.own) && aligned16(a.add0) && aligned16(a.add1) && aligned16(a.key2) &&
+                   aligned16(a.y2) &&
                    ((a.ext_item | a.own_item | a.add_item | a.y_item) & 1) == 0;
     for (uint32_t k = 0; a.gathered && k < count; k++) aligned = aligned && aligned16(a.ga[k]);
     if (!aligned) return CATFHE_EINVAL;
-    return a.gathered ? ip_run<true>(c, a, count, s) : ip_run<false>(c, a, count, s);
+    if (a.key2) return a.gathered ? CATFHE_EINVAL : ip_run<false, 2>(c, a, count, s);
+    return a.gathered ? ip_run<true, 1>(c, a, count, s) : ip_run<false, 1>(c, a, count, s);
 }
 
 // ------------------------------------------------------------------ ModDown combine

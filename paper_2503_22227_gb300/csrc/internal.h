@@ -393,6 +393,8 @@ struct IpArgs {
     const uint64_t *key;       // [beta_L][2][L+K][N], Montgomery form
     const uint64_t *add0, *add1;  // [count][l][N] added times P (Q positions), or null
     uint64_t *y;               // [count][2][M][N]
+    const uint64_t *key2;      // a second key for the same digits, its result to y2 (null: none;
+    uint64_t *y2;              // 2 to kIpPairBeta digits, not gathered)
     size_t ext_item, own_item, add_item, y_item;
     uint32_t M, level, beta, L, K;
     uint32_t alpha;
@@ -406,6 +408,7 @@ struct IpArgs {
     uint32_t gathered;
     const uint64_t *ga[kGatherMax];
 };
+constexpr int kIpPairBeta = 8;
 int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s);
 int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s);
 

@@ -361,11 +361,12 @@ static int modup_ntt(Context &c, const KsConsts &k, const uint64_t *d2c, size_t 
 
 // own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
 // words apart (null: none).  gth (rotations): ciphertext i's add0 and own are
-// the two polynomials of gth->a[i].
+// the two polynomials of gth->a[i].  key2: a second key, its result in y2.
 static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, const uint64_t *own,
                          const uint64_t *key, const uint64_t *add0, const uint64_t *add1,
                          size_t in_item, uint64_t *y, uint32_t count, cudaStream_t s,
-                         const Gather *gth = nullptr) {
+                         const Gather *gth = nullptr, const uint64_t *key2 = nullptr,
+                         uint64_t *y2 = nullptr) {
     IpArgs a = k.ip;
     a.ext = ext;
     a.own = own;
@@ -373,6 +374,8 @@ static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, con
     a.add0 = add0;
     a.add1 = add1;
     a.y = y;
+    a.key2 = key2;
+    a.y2 = y2;
     a.own_item = a.add_item = in_item;
     if (gth && gth->n) {
         a.gathered = 1;
@@ -903,23 +906,42 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     const KsConsts *kc;
     TRY(ks_consts(c, lvl, false, &kc));
     TRY(modup_ntt(c, *kc, k.d2c, half, ext0, count, s));
+    auto down = [&](uint32_t r, KsBufs &kb, uint64_t *y, cudaStream_t st) {
+        return moddown(c, *kc, y, kb.lift, out + size_t(r) * count * item, count, st, gv[r]);
+    };
     auto one = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
         TRY(inner_product(c, *kc, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, st));
-        return moddown(c, *kc, kb.y, kb.lift, out + size_t(r) * count * item, count, st, gv[r]);
+        return down(r, kb, kb.y, st);
     };
+    // two rotations by one inner product, which reads the digits once; the
+    // second result stands in the set's own digit buffer, which holds it from
+    // two digits on and is otherwise unused (the workspace is as before)
+    auto two = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
+        TRY(inner_product(c, *kc, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, st, nullptr,
+                          gk[r + 1], kb.ext));
+        TRY(down(r, kb, kb.y, st));
+        return down(r + 1, kb, kb.ext, st);
+    };
+    const bool pair = beta >= 2 && beta <= kIpPairBeta;
     if (n_rot < 2 || c.log_n < 14) {
-        for (uint32_t r = 0; r < n_rot; r++) TRY(one(r, k, s));
+        uint32_t r = 0;
+        for (; pair && r + 1 < n_rot; r += 2) TRY(two(r, k, s));
+        for (; r < n_rot; r++) TRY(one(r, k, s));
         return CATFHE_OK;
     }
     // rotations alternate over the two split streams, each with its own
-    // buffer set (in order on its stream), after the shared ModUp on s
+    // buffer set (in order on its stream), after the shared ModUp on s; pairs
+    // only while both streams have one, so that the rest still overlaps
     std::lock_guard<std::mutex> lock(g_split_mu);
     SplitPool *sp;
     TRY(split_pool(&sp));
     if (cudaEventRecord(sp->fork, s) != cudaSuccess) return CATFHE_ECUDA;
     for (int h = 0; h < 2; h++)
         if (cudaStreamWaitEvent(sp->st[h], sp->fork, 0) != cudaSuccess) return CATFHE_ECUDA;
-    for (uint32_t r = 0; r < n_rot; r++) TRY(one(r, ks[r & 1], sp->st[r & 1]));
+    uint32_t r = 0;
+    for (; pair && r + 4 <= n_rot; r += 4)
+        for (int h = 0; h < 2; h++) TRY(two(r + 2 * h, ks[h], sp->st[h]));
+    for (; r < n_rot; r++) TRY(one(r, ks[r & 1], sp->st[r & 1]));
     for (int h = 0; h < 2; h++) {
         if (cudaEventRecord(sp->join[h], sp->st[h]) != cudaSuccess) return CATFHE_ECUDA;
         if (cudaStreamWaitEvent(s, sp->join[h], 0) != cudaSuccess) return CATFHE_ECUDA;

@@ -55,3 +55,26 @@ def test_rotation_over_its_input(scheme, count):
         same = a.clone()
         ctx.rotate(keys, same, g, out=same)
         assert torch.equal(same, want), g
+
+
+@pytest.mark.parametrize("log_n,dnum,L", [(12, 1, 3), (12, 2, 4), (12, 3, 5), (13, 8, 8),
+                                          (12, 9, 9), (14, 1, 2), (14, 4, 7), (15, 5, 5)])
+def test_paired_rotations_equal_single_ones(log_n, dnum, L):
+    """1 to 9 digits (pairs from 2 to 8), every remainder of the pairs over one
+    and two streams, one ciphertext (one buffer), two and five, a level with a
+    partly used last digit, and an element given twice."""
+    p = W.Preset("rot-pairs", W.CKKS, log_n, (50,) * L, (60,) * 4, dnum, log_n_max=16)
+    ctx = api.Context(p)
+    keys = ctx.keygen(W.seed_for(f"rot-pairs-{log_n}-{dnum}"))
+    gs = [ctx.galois_elt(r) for r in (1, -3, 5, 2, 7)] + [2 * ctx.n - 1, ctx.galois_elt(1)]
+    for g in gs:
+        keys.gen_galois(g)
+    seed = W.seed_for("rot-pairs-in")
+    for level in {L, max(1, L - 1)}:
+        for count in (1, 2, 5):
+            a = torch.cat([ctx.ct_uniform(seed, i, level) for i in range(count)])
+            want = [ctx.rotate(keys, a, g) for g in gs]
+            for n_rot in range(1, len(gs) + 1):
+                out = ctx.rotate_hoisted(keys, a, gs[:n_rot])
+                for j in range(n_rot):
+                    assert torch.equal(out[j], want[j]), (level, count, n_rot, j)
