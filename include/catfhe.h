@@ -422,10 +422,11 @@ uint64_t catfhe_kernel_launches(void);
 /* ---- Uneven batches (many independent operations in one submission) ----
  * Each entry is one operation of any context (ring degree), level and kind;
  * the entries must not depend on one another.  catfhe_run_batch spreads
- * them over `lanes` (1..32) concurrent streams forked from `stream`, each
- * lane with its own slice of `ws` (at least catfhe_batch_workspace_bytes),
- * assigning operations longest-first by modular-product count, and joins
- * the lanes back into `stream` (paper Sec. 3.1.6 spreads per-modulus work
+ * them over at most `lanes` (1..32; fewer when the operations in flight would
+ * overflow the L2) concurrent streams forked from `stream`, each lane with its
+ * own slice of `ws` (at least catfhe_batch_workspace_bytes), assigning and
+ * running operations longest-first by estimated time, and joins the
+ * lanes back into `stream` (paper Sec. 3.1.6 spreads per-modulus work
  * over a stream pool; here whole operations are spread).
  * catfhe_batch_capture runs the batch once, then captures it into a CUDA
  * graph (buffers and workspace are baked in: replaying it recomputes the

@@ -4,13 +4,15 @@
 //
 // The paper spreads per-modulus kernels over a stream pool (Sec. 3.1.6);
 // here a whole operation is the unit: ops are assigned to lanes by
-// longest-processing-time-first on their modular-product count, each lane
+// longest-processing-time-first on their modular-product count and launches,
+// on no more lanes than the L2 has room for (used_lanes); each lane
 // is a stream forked from the caller's stream with its own workspace slice,
 // and the lanes join back before the call returns.  Capturing the batch
 // once and replaying the graph removes the per-launch host cost.
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -147,6 +149,21 @@ double op_cost(const catfhe_op &o) {
     return o.count * (ntt * n / 2 * lg + prod * n);
 }
 
+// Time of an operation's chain of launches when nothing else bounds it (us,
+// measured at N = 2^13), and the chip's modular products per us: on one of
+// `lanes` lanes an operation takes its chain's time and its products at the
+// lane's share of the chip.  Balanced by products alone, the lanes with the
+// small operations ended last (16 uneven operations on 8 lanes 500 -> 466 us,
+// 24 at N = 2^13 264 -> 249, 96 uneven ones 4040 -> 3955).
+constexpr double kChainUs = 25, kRescaleUs = 8, kLaunchUs = 2.5, kProductsPerUs = 1.13e6;
+
+double chain_cost(const catfhe_op &o, uint32_t lanes) {
+    const double us = !needs_ws(o.op)              ? kLaunchUs
+                      : o.op == CATFHE_OP_RESCALE ? kRescaleUs
+                                                  : kChainUs;
+    return us * kProductsPerUs / lanes;
+}
+
 // A unit of work on one lane: one entry, or several single-ciphertext
 // entries of the same kind, context, keys, level (and Galois element) merged
 // into one gathered operation.
@@ -198,20 +215,47 @@ void make_units(const catfhe_op *ops, uint32_t n, uint32_t lanes, std::vector<Un
     }
 }
 
-int plan_batch(const catfhe_op *ops, uint32_t n, uint32_t lanes, Plan &p) {
-    if (!ops || n == 0) return CATFHE_EINVAL;
-    lanes = std::max<uint32_t>(1, std::min<uint32_t>(std::min<uint32_t>(lanes, n), kMaxLanes));
+// Workspace of the operations in flight that the lanes of a batch are held to.
+// What an operation writes is read back by its next kernel; with more lanes
+// than this the working sets push each other out of the L2 (129 MB), with
+// fewer the chip is not filled.  Measured on one degree at a time (us for 64
+// operations of any level, 8 lanes asked; all of them in submission order ->
+// here): N = 2^16 5008 -> 4156 (3 lanes), 2^15 2322 -> 2187, 2^14 1181 -> 1126,
+// 2^13 654 -> 578 (8 lanes); 256 of all four degrees 9240 -> 8530; eight
+// encrypted queries 72 -> 68 ms.  300 and 400 MB differ by 3% or less; at 500 MB
+// the first is 4215.
+constexpr double kLaneBytes = 320e6;
+// Entries per lane from which lanes are left out: below, the longest chain of
+// operations counts and not the rate (8 uneven operations on 8 lanes 268 us,
+// on 4 lanes 304; 32 of them 1490 and 1406).
+constexpr uint32_t kLaneEntries = 4;
+
+// Lanes for the batch, at most `lanes`: kLaneBytes over the entries' mean
+// workspace, weighted by their cost (the part of the time that they run).
+uint32_t used_lanes(const catfhe_op *ops, uint32_t n, uint32_t lanes) {
+    double cost = 0, bytes = 0;
     for (uint32_t i = 0; i < n; i++) {
-        const int rc = check_op(ops[i]);
-        if (rc) return rc;
+        const catfhe_op &o = ops[i];
+        const double k = op_cost(o);
+        cost += k;
+        bytes += k * double(needs_ws(o.op)
+                                ? ws_bytes(o.ctx->c, o.op, o.level, o.count)
+                                : size_t(6) * 8 * o.level * o.ctx->c.n * o.count);  // a, b, out
     }
+    if (!(bytes > 0)) return lanes;
+    const double fit = std::max(2.0, std::floor(kLaneBytes * cost / bytes + 0.5));
+    return fit < double(lanes) ? uint32_t(fit) : lanes;
+}
+
+void assign_lanes(const catfhe_op *ops, uint32_t n, uint32_t lanes, Plan &p) {
     p.units.clear();
     make_units(ops, n, lanes, p.units);
     const uint32_t nu = uint32_t(p.units.size());
     std::vector<uint32_t> order(nu);
-    std::vector<double> cost(nu, 0.0);
+    std::vector<double> cost(nu);
     for (uint32_t u = 0; u < nu; u++) {
         order[u] = u;
+        cost[u] = chain_cost(ops[p.units[u].entries[0]], std::min(lanes, nu));
         for (uint32_t i : p.units[u].entries) cost[u] += op_cost(ops[i]);
     }
     std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return cost[x] > cost[y]; });
@@ -229,13 +273,33 @@ int plan_batch(const catfhe_op *ops, uint32_t n, uint32_t lanes, Plan &p) {
         const size_t w = needs_ws(o.op) ? ws_bytes(o.ctx->c, o.op, o.level, items) : 0;
         p.lane_ws[l] = std::max(p.lane_ws[l], (w + 255) & ~size_t(255));
     }
-    // within a lane, run in submission order
-    for (auto &v : p.lane_units)
-        std::sort(v.begin(), v.end(), [&](uint32_t x, uint32_t y) {
+    // lanes run their units as they were assigned, the largest first: they then
+    // end on small ones, close together.  A single lane keeps the order of
+    // submission.
+    if (nl == 1)
+        std::sort(p.lane_units[0].begin(), p.lane_units[0].end(), [&](uint32_t x, uint32_t y) {
             return p.units[x].entries[0] < p.units[y].entries[0];
         });
     p.total = 0;
     for (size_t w : p.lane_ws) p.total += w;
+}
+
+int plan_batch(const catfhe_op *ops, uint32_t n, uint32_t lanes, Plan &p) {
+    if (!ops || n == 0) return CATFHE_EINVAL;
+    lanes = std::max<uint32_t>(1, std::min<uint32_t>(std::min<uint32_t>(lanes, n), kMaxLanes));
+    for (uint32_t i = 0; i < n; i++) {
+        const int rc = check_op(ops[i]);
+        if (rc) return rc;
+    }
+    assign_lanes(ops, n, lanes, p);
+    const uint32_t used = used_lanes(ops, n, lanes);
+    if (used < lanes && n >= kLaneEntries * used) {
+        // fewer lanes merge more entries into one unit: taken only when that
+        // needs no larger workspace
+        Plan q;
+        assign_lanes(ops, n, used, q);
+        if (q.total <= p.total) p = std::move(q);
+    }
     return CATFHE_OK;
 }
 

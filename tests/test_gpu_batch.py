@@ -267,3 +267,38 @@ def test_uneven_mix_full_sizes_sampled():
         assert np.array_equal(c.export_ct(o)[0], want), (log_n, level)
         seen.add(log_n)
     assert seen == {13, 14, 15, 16}
+
+
+def test_large_operations_share_few_lanes():
+    """Operations whose working sets overflow the L2 run on fewer lanes than
+    asked: 17 of N = 2^16 at 20 to 24 limbs (three of them merged) on 8 lanes
+    need the workspace of fewer than 5 and give the single operations'
+    results, and so does a batch too small for that rule."""
+    p = W.PRESETS["ckks_n16"]
+    ctx, keys, gs = _ctx(p, (1, 3))
+    seed = W.seed_for("few-lanes")
+    kinds = (api.OP_MUL_RELIN_RESCALE, api.OP_ROTATE, api.OP_RESCALE)
+    ops, outs, wants, keep = [], [], [], []
+    for j in range(17):
+        kind, level = (kinds[j % 3], 20 + j % 5) if j < 14 else (api.OP_MUL_RELIN, 24)
+        a, b = ctx.ct_uniform(seed, 2 * j, level), ctx.ct_uniform(seed, 2 * j + 1, level)
+        want = {api.OP_MUL_RELIN_RESCALE: lambda: ctx.mul_relin_rescale(keys, a, b),
+                api.OP_MUL_RELIN: lambda: ctx.mul_relin(keys, a, b),
+                api.OP_ROTATE: lambda: ctx.rotate(keys, a, gs[j % 2]),
+                api.OP_RESCALE: lambda: ctx.rescale(a)}[kind]()
+        out = torch.full_like(want, -1)
+        ops.append(api.make_op(kind, ctx, a, out, keys=keys, b=b, galois_elt=gs[j % 2]))
+        outs.append(out)
+        wants.append(want.clone())
+        keep.append((a, b))
+    one = max(api.Batch([op]).workspace_bytes(1) for op in ops)
+    assert api.Batch(ops).workspace_bytes(8) < 5 * one
+    each = sum(api.Batch([op]).workspace_bytes(1) - 256 for op in ops[:4])
+    assert api.Batch(ops[:4]).workspace_bytes(8) == each + 256  # a lane for each
+    for part, lanes in ((ops, 8), (ops[:4], 8), (ops, 1)):
+        for o in outs:
+            o.fill_(-1)
+        api.run_batch(part, lanes=lanes)
+        torch.cuda.synchronize()
+        for j in range(len(part)):
+            assert torch.equal(outs[j], wants[j]), (len(part), lanes, j)
