@@ -45,36 +45,11 @@ k_tensor(const TensorArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
     const size_t l0 = size_t(i) * n + x, l1 = (size_t(A.limbs) + i) * n + x;
     const ulonglong2 a0 = ld2(a + l0), a1 = ld2(a + l1), b0 = ld2(b + l0), b1 = ld2(b + l1);
     const size_t o = item * A.out_item + size_t(i) * n + x;
-    // b in Montgomery form (b 2^64 mod q, in [0, 4q), one Shoup product each
-    // on the approximate quotient), then one Montgomery reduction per output:
-    // a b' < 4q^2 and the d1 sum < 8q^2, both below 2^64 q, so REDC returns
-    // a b in [0, 2q) (measured: batched step 1438.5 -> 1435.2 us against two
-    // Shoup products per 128-bit reduction)
-    const uint64_t q = m.q;
-    const ulonglong2 c0 = make_ulonglong2(shoup_lazy4(b0.x, m.r64, m.r64_s, q),
-                                          shoup_lazy4(b0.y, m.r64, m.r64_s, q));
-    const ulonglong2 c1 = make_ulonglong2(shoup_lazy4(b1.x, m.r64, m.r64_s, q),
-                                          shoup_lazy4(b1.y, m.r64, m.r64_s, q));
-    U128 p0{0, 0}, p1{0, 0};
-    mac(p0, a0.x, c0.x);
-    mac(p1, a0.y, c0.y);
-    st2(A.d0 + o, csub(redc(p0, q, m.qinv), q), csub(redc(p1, q, m.qinv), q));
-    U128 r0{0, 0}, r1{0, 0};
-    mac(r0, a1.x, c1.x);
-    mac(r1, a1.y, c1.y);
-    st2(A.d2 + o, csub(redc(r0, q, m.qinv), q), csub(redc(r1, q, m.qinv), q));
-    // d1 by Karatsuba: (a0 + a1)(b0' + b1') - a0 b0' - a1 b1' = a0 b1' + a1 b0',
-    // one 64 x 64 product instead of two.  a0 + a1 < 2q and b0' + b1' < 8q
-    // each fit one word (q < 2^61), their product (< 16 q^2) fits 128 bits,
-    // and the difference is the same d1 sum as above, below 8 q^2
-    U128 s0{0, 0}, s1{0, 0};
-    mac(s0, a0.x + a1.x, c0.x + c1.x);
-    mac(s1, a0.y + a1.y, c0.y + c1.y);
-    sub128(s0, p0);
-    sub128(s0, r0);
-    sub128(s1, p1);
-    sub128(s1, r1);
-    st2(A.d1 + o, csub(redc(s0, q, m.qinv), q), csub(redc(s1, q, m.qinv), q));
+    const Tensor u = tensor_mod(a0.x, a1.x, b0.x, b1.x, m);
+    const Tensor v = tensor_mod(a0.y, a1.y, b0.y, b1.y, m);
+    st2(A.d0 + o, u.d0, v.d0);
+    st2(A.d1 + o, u.d1, v.d1);
+    st2(A.d2 + o, u.d2, v.d2);
 }
 
 int launch_tensor(const Context &c, const TensorArgs &a, uint32_t count, cudaStream_t s) {
@@ -94,6 +69,12 @@ __device__ __forceinline__ const uint64_t *ip_own(const IpArgs &A, uint32_t item
 template <bool GATHER>
 __device__ __forceinline__ const uint64_t *ip_add0(const IpArgs &A, uint32_t item) {
     return GATHER ? A.ga[item] : A.add0 + item * A.add_item;
+}
+
+// The first limb of an item's second factor (products).
+template <bool GATHER>
+__device__ __forceinline__ const uint64_t *ip_b(const IpArgs &A, uint32_t item) {
+    return GATHER ? A.gb[item] : A.b + item * A.add_item;
 }
 
 // Many digits (beta > 8): digit by digit, loads interleaved with products,
@@ -154,6 +135,17 @@ k_ip_stream(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n) {
 // coefficients (256 threads) up to 4 digits; 256 coefficients (128 threads)
 // for 5 to 8 digits, so that the 2 BETA key tiles and the two buffers
 // (72 KB at BETA = 8) leave room for 3 CTAs per SM.
+// FORM, bits: the ciphertexts of the launch are gathered; the addends and the
+// own digits are the tensor product of two ciphertexts, formed here from
+// them (a0 and b0 in the two slots after the digits, a1 in the own digit's);
+// there is a second addend (without it and products a buffer has one tile
+// less: 16 rotations of 8 ciphertexts at N = 2^16 8043 -> 7924 us).
+constexpr int kIpGathered = 1, kIpProduct = 2, kIpTwoAdds = 4;
+template <int BETA, int FORM>
+struct IpSlots {  // tiles of one ciphertext in a buffer
+    static constexpr int value = BETA + (FORM & (kIpProduct | kIpTwoAdds) ? 2 : 1);
+};
+
 template <int BETA, int R>
 struct IpTile {
     static constexpr uint32_t value = BETA * R <= 4 ? 512 : 256;
@@ -172,9 +164,11 @@ struct IpTile {
 // The batch of 16 rotations of 8: 8128 -> 8023 us (the transforms that run
 // beside it bound it); 16 rotations of one: 1349 -> 1267 us; 4 at N = 2^12:
 // 57.0 -> 52.7 us; 2 or 3 rotations at N >= 2^14 stay one to each stream.
-template <int BETA, bool GATHER, int R>
+template <int BETA, int FORM, int R>
 __global__ void __launch_bounds__(IpTile<BETA, R>::value / 2)
 k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint32_t count) {
+    constexpr bool GATHER = (FORM & kIpGathered) != 0, PROD = (FORM & kIpProduct) != 0;
+    constexpr int SLOTS = IpSlots<BETA, FORM>::value;
     grid_dep_wait();
     const uint32_t per = (count + gridDim.z - 1) / gridDim.z;
     const uint32_t first = blockIdx.z * per;
@@ -189,12 +183,13 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
     const uint32_t beta = A.beta, KL = A.L + A.K;
     const DevMod m = mods[A.prime[i]];
     const bool fold = i < A.level && A.pfac[i] != 0;
-    const bool f0 = fold && A.add0, f1 = fold && A.add1;
+    const bool f0 = fold && A.add0, prod = PROD && i < A.level;
+    const bool f1 = (FORM & kIpTwoAdds) != 0 && fold;
     const uint32_t own_digit = (A.own != nullptr && i < A.level) ? i / A.alpha : 0xffffffffu;
     constexpr uint32_t TB = kIpTile * 8;  // bytes per tile
     uint64_t *skey = sm;                                   // [R][2 BETA][tile]
-    uint64_t *sbuf[2] = {sm + 2 * R * BETA * kIpTile, sm + ((2 * R + 1) * BETA + 2) * kIpTile};
-    const uint32_t item_bytes = (beta + (f0 ? 1 : 0) + (f1 ? 1 : 0)) * TB;
+    uint64_t *sbuf[2] = {sm + 2 * R * BETA * kIpTile, sm + (2 * R * BETA + SLOTS) * kIpTile};
+    const uint32_t item_bytes = (beta + (f0 ? 1 : 0) + (prod || f1 ? 1 : 0)) * TB;
 
     auto issue_item = [&](uint32_t k, uint32_t b) {  // the group's k-th ciphertext
         const uint32_t item = first + k;
@@ -208,8 +203,17 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
         }
         if (f0) bulk_load(dst + BETA * kIpTile, ip_add0<GATHER>(A, item) + size_t(i) * n + x0, TB, &bars[b]);
         if (f1) bulk_load(dst + (BETA + 1) * kIpTile, A.add1 + item * A.add_item + size_t(i) * n + x0, TB, &bars[b]);
+        if (prod) bulk_load(dst + (BETA + 1) * kIpTile, ip_b<GATHER>(A, item) + size_t(i) * n + x0, TB, &bars[b]);
     };
 
+    const uint32_t u = 2 * tid;  // this thread's two coefficients in the tile
+    // products: b1's words by plain loads, an item ahead (a third extra tile in
+    // each buffer would take 8 digits from 3 CTAs per SM to 2)
+    auto load_b1 = [&](uint32_t k) {
+        return ld2(ip_b<GATHER>(A, first + k) + (size_t(A.level) + i) * n + x0 + u);
+    };
+    ulonglong2 b1 = make_ulonglong2(0, 0);
+    if (prod) b1 = load_b1(0);
     if (tid == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -234,42 +238,53 @@ k_ip_bulk(const IpArgs A, const DevMod *__restrict__ mods, uint32_t log_n, uint3
     // every wait is bounded, and the CTA decides together whether to go on
     // (__syncthreads_and), so no thread is left waiting at a barrier
     bool ok = __syncthreads_and(mbar_wait(&bars[2], 0));
-    const uint32_t u = 2 * tid;  // this thread's two coefficients in the tile
     for (uint32_t k = 0; k < nloc && ok; k++) {
         const uint32_t item = first + k, b = k & 1;
         ok = __syncthreads_and(mbar_wait(&bars[b], (k >> 1) & 1));
         if (!ok) break;
         const uint64_t *buf = sbuf[b];
+        ulonglong2 d0 = make_ulonglong2(0, 0), d1 = d0, d2 = d0;
+        if (prod) {  // the tensor product of this tile; the own digit's slot holds a1
+            const ulonglong2 p0 = ld2(buf + BETA * kIpTile + u), q0 = ld2(buf + (BETA + 1) * kIpTile + u);
+            const ulonglong2 p1 = ld2(buf + own_digit * kIpTile + u);
+            const Tensor t = tensor_mod(p0.x, p1.x, q0.x, b1.x, m);
+            const Tensor w = tensor_mod(p0.y, p1.y, q0.y, b1.y, m);
+            d0 = make_ulonglong2(t.d0, w.d0);
+            d1 = make_ulonglong2(t.d1, w.d1);
+            d2 = make_ulonglong2(t.d2, w.d2);
+            if (k + 1 < nloc) b1 = load_b1(k + 1);
+        } else {
+            if (f0) d0 = ld2(buf + BETA * kIpTile + u);
+            if (f1) d1 = ld2(buf + (BETA + 1) * kIpTile + u);
+        }
 #pragma unroll
         for (int r = 0; r < R; r++) {
             const uint64_t *key = skey + r * 2 * BETA * kIpTile;
-            U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};
+            U128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1s{0, 0};
             if (f0) {
-                const ulonglong2 d = ld2(buf + BETA * kIpTile + u);
-                mac(a0, d.x, A.pfac[i]);
-                mac(a1, d.y, A.pfac[i]);
+                mac(a0, d0.x, A.pfac[i]);
+                mac(a1, d0.y, A.pfac[i]);
             }
-            if (f1) {
-                const ulonglong2 d = ld2(buf + (BETA + 1) * kIpTile + u);
-                mac(b0, d.x, A.pfac[i]);
-                mac(b1, d.y, A.pfac[i]);
+            if (prod || f1) {
+                mac(b0, d1.x, A.pfac[i]);
+                mac(b1s, d1.y, A.pfac[i]);
             }
 #pragma unroll
             for (int j = 0; j < BETA; j++) {
                 if (uint32_t(j) < beta) {
-                    const ulonglong2 c = ld2(buf + j * kIpTile + u);
+                    const ulonglong2 c = prod && uint32_t(j) == own_digit ? d2 : ld2(buf + j * kIpTile + u);
                     const ulonglong2 kb = ld2(key + (2 * j) * kIpTile + u);
                     const ulonglong2 ka = ld2(key + (2 * j + 1) * kIpTile + u);
                     mac(a0, c.x, kb.x);
                     mac(a1, c.y, kb.y);
                     mac(b0, c.x, ka.x);
-                    mac(b1, c.y, ka.y);
+                    mac(b1s, c.y, ka.y);
                 }
             }
             uint64_t *y = (r ? A.y2 : A.y) + item * A.y_item + x0 + u;
             st2(y + size_t(i) * n, csub(redc(a0, m.q, m.qinv), m.q), csub(redc(a1, m.q, m.qinv), m.q));
             st2(y + (size_t(A.M) + i) * n, csub(redc(b0, m.q, m.qinv), m.q),
-                csub(redc(b1, m.q, m.qinv), m.q));
+                csub(redc(b1s, m.q, m.qinv), m.q));
         }
         __syncthreads();  // everyone is done with buffer b
         if (tid == 0 && k + 2 < nloc) {
@@ -334,16 +349,17 @@ static unsigned ip_groups(K kernel, unsigned threads, size_t smem, size_t ctas, 
     return top >= 1.1 * one ? best : 1;
 }
 
-template <int BETA, bool GATHER, int R>
+template <int BETA, int FORM, int R>
 static int ip_run_bulk(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
     constexpr uint32_t tile = IpTile<BETA, R>::value;
     // two buffers of the ciphertexts' tiles, one when each CTA has a single
     // ciphertext (then more CTAs are resident, 5 instead of 3 per SM at 3 digits:
     // one product at N = 2^16, l = 24 201.8 -> 199.4 us, the 256-operation mix
     // 9.70 -> 9.55 ms)
-    const auto kernel = k_ip_bulk<BETA, GATHER, R>;
+    const auto kernel = k_ip_bulk<BETA, FORM, R>;
     const void *const k = reinterpret_cast<const void *>(kernel);
-    constexpr size_t one = size_t((2 * R + 1) * BETA + 2) * tile * 8, two = one + size_t(BETA + 2) * tile * 8;
+    constexpr int slots = IpSlots<BETA, FORM>::value;
+    constexpr size_t one = size_t(2 * R * BETA + slots) * tile * 8, two = one + size_t(slots) * tile * 8;
     const unsigned groups =
         count > 1 ? ip_groups(kernel, tile / 2, two, c.n / tile * a.M, count) : 1;
     const size_t smem = groups >= count ? one : two;
@@ -353,23 +369,23 @@ static int ip_run_bulk(const Context &c, const IpArgs &a, uint32_t count, cudaSt
     return ok();
 }
 
-template <bool GATHER, int R>
+template <int FORM, int R>
 static int ip_run(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s) {
     switch (a.beta) {
         case 1:
             if constexpr (R > 1) return CATFHE_EINVAL;  // one digit: not paired
-            else return ip_run_bulk<1, GATHER, R>(c, a, count, s);
-        case 2: return ip_run_bulk<2, GATHER, R>(c, a, count, s);
-        case 3: return ip_run_bulk<3, GATHER, R>(c, a, count, s);
-        case 4: return ip_run_bulk<4, GATHER, R>(c, a, count, s);
-        case 5: return ip_run_bulk<5, GATHER, R>(c, a, count, s);
-        case 6: return ip_run_bulk<6, GATHER, R>(c, a, count, s);
-        case 7: return ip_run_bulk<7, GATHER, R>(c, a, count, s);
-        case 8: return ip_run_bulk<8, GATHER, R>(c, a, count, s);
+            else return ip_run_bulk<1, FORM, R>(c, a, count, s);
+        case 2: return ip_run_bulk<2, FORM, R>(c, a, count, s);
+        case 3: return ip_run_bulk<3, FORM, R>(c, a, count, s);
+        case 4: return ip_run_bulk<4, FORM, R>(c, a, count, s);
+        case 5: return ip_run_bulk<5, FORM, R>(c, a, count, s);
+        case 6: return ip_run_bulk<6, FORM, R>(c, a, count, s);
+        case 7: return ip_run_bulk<7, FORM, R>(c, a, count, s);
+        case 8: return ip_run_bulk<8, FORM, R>(c, a, count, s);
         default:
-            if constexpr (R > 1) return CATFHE_EINVAL;
+            if constexpr (R > 1 || (FORM & kIpProduct) != 0) return CATFHE_EINVAL;
             else {
-                launch_pdl(k_ip_stream<GATHER>, dim3(count, unsigned((c.n / 2 + 255) / 256), a.M),
+                launch_pdl(k_ip_stream<FORM == kIpGathered>, dim3(count, unsigned((c.n / 2 + 255) / 256), a.M),
                            dim3(256), 0, s, a, c.d_mods, uint32_t(c.log_n));
                 return ok();
             }
@@ -381,12 +397,21 @@ int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s)
     // at the entry points unless 16-byte aligned
     bool aligned = a.status != nullptr && aligned16(a.ext) && aligned16(a.key) && aligned16(a.y) &&
                    aligned16(a.own) && aligned16(a.add0) && aligned16(a.add1) && aligned16(a.key2) &&
-                   aligned16(a.y2) &&
+                   aligned16(a.y2) && aligned16(a.b) &&
                    ((a.ext_item | a.own_item | a.add_item | a.y_item) & 1) == 0;
-    for (uint32_t k = 0; a.gathered && k < count; k++) aligned = aligned && aligned16(a.ga[k]);
+    for (uint32_t k = 0; a.gathered && k < count; k++)
+        aligned = aligned && aligned16(a.ga[k]) && (!a.product || aligned16(a.gb[k]));
     if (!aligned) return CATFHE_EINVAL;
-    if (a.key2) return a.gathered ? CATFHE_EINVAL : ip_run<false, 2>(c, a, count, s);
-    return a.gathered ? ip_run<true, 1>(c, a, count, s) : ip_run<false, 1>(c, a, count, s);
+    if (a.product) {
+        // two ciphertexts and nothing else, at most kIpBulkBeta digits
+        if (a.add1 || a.key2 || !a.own || !a.add0) return CATFHE_EINVAL;
+        return a.gathered ? ip_run<kIpProduct | kIpGathered, 1>(c, a, count, s)
+                          : ip_run<kIpProduct, 1>(c, a, count, s);
+    }
+    if (a.add1)
+        return a.gathered || a.key2 ? CATFHE_EINVAL : ip_run<kIpTwoAdds, 1>(c, a, count, s);
+    if (a.key2) return a.gathered ? CATFHE_EINVAL : ip_run<0, 2>(c, a, count, s);
+    return a.gathered ? ip_run<kIpGathered, 1>(c, a, count, s) : ip_run<0, 1>(c, a, count, s);
 }
 
 // ------------------------------------------------------------------ ModDown combine

@@ -276,8 +276,14 @@ uint64_t launches_total();
 // NTT (ntt.cu)
 int launch_ntt_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
                    uint32_t n_limbs, cudaStream_t s);
+// The second factor of an inverse transform of products: the limb at the same
+// place of b (or of gb[g], when the map is gathered).
+struct NttFactor {
+    const uint64_t *b;
+    const uint64_t *gb[kGatherMax];
+};
 int launch_ntt_inv(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
-                   uint32_t n_limbs, cudaStream_t s);
+                   uint32_t n_limbs, cudaStream_t s, const NttFactor *factor = nullptr);
 
 // Forward NTT whose last pass also finishes the ModDown: for map entry r of
 // group g it writes out = (y - NTT(lift)) * dinv[r] instead of the
@@ -394,7 +400,7 @@ struct IpArgs {
     const uint64_t *add0, *add1;  // [count][l][N] added times P (Q positions), or null
     uint64_t *y;               // [count][2][M][N]
     const uint64_t *key2;      // a second key for the same digits, its result to y2 (null: none;
-    uint64_t *y2;              // 2 to kIpPairBeta digits, not gathered)
+    uint64_t *y2;              // 2 to kIpBulkBeta digits, not gathered)
     size_t ext_item, own_item, add_item, y_item;
     uint32_t M, level, beta, L, K;
     uint32_t alpha;
@@ -407,8 +413,14 @@ struct IpArgs {
     // there are such limbs)
     uint32_t gathered;
     const uint64_t *ga[kGatherMax];
+    // product: nonzero when the addends and the own digits are the tensor
+    // product of the ciphertexts a = (add0, own) and b (both [count][2][l][N],
+    // or ga and gb), formed by the kernel; at most kIpBulkBeta digits
+    uint32_t product;
+    const uint64_t *b;
+    const uint64_t *gb[kGatherMax];
 };
-constexpr int kIpPairBeta = 8;
+constexpr uint32_t kIpBulkBeta = 8;  // digits of the staged kernel
 int launch_ip(const Context &c, const IpArgs &a, uint32_t count, cudaStream_t s);
 int launch_wait_selftest(const Context &c, uint64_t limit_ns, cudaStream_t s);
 

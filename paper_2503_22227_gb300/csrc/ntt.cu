@@ -29,7 +29,7 @@ namespace catfhe {
                       uint32_t n_limbs, cudaStream_t s, const NttEpilogue *epi, bool lazy,      \
                       int sched, const LiftEntry *lifts);                                      \
     int ntt_inv_n##LN(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map, \
-                      uint32_t n_limbs, cudaStream_t s, int sched);
+                      uint32_t n_limbs, cudaStream_t s, int sched, const NttFactor *factor);
 NTT_DECL(12) NTT_DECL(13) NTT_DECL(14) NTT_DECL(15) NTT_DECL(16)
 #undef NTT_DECL
 
@@ -92,15 +92,15 @@ int launch_ntt_lift_combine(const Context &c, const uint64_t *src, uint64_t *lif
 }
 
 int launch_ntt_inv(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
-                   uint32_t n_limbs, cudaStream_t s) {
+                   uint32_t n_limbs, cudaStream_t s, const NttFactor *factor) {
     if (n_limbs == 0) return CATFHE_OK;
     const int sched = c.ntt_sched[ntt_class(n_limbs)];
     switch (c.log_n) {
-        case 12: return ntt_inv_n12(c, src, dst, map, n_limbs, s, sched);
-        case 13: return ntt_inv_n13(c, src, dst, map, n_limbs, s, sched);
-        case 14: return ntt_inv_n14(c, src, dst, map, n_limbs, s, sched);
-        case 15: return ntt_inv_n15(c, src, dst, map, n_limbs, s, sched);
-        case 16: return ntt_inv_n16(c, src, dst, map, n_limbs, s, sched);
+        case 12: return ntt_inv_n12(c, src, dst, map, n_limbs, s, sched, factor);
+        case 13: return ntt_inv_n13(c, src, dst, map, n_limbs, s, sched, factor);
+        case 14: return ntt_inv_n14(c, src, dst, map, n_limbs, s, sched, factor);
+        case 15: return ntt_inv_n15(c, src, dst, map, n_limbs, s, sched, factor);
+        case 16: return ntt_inv_n16(c, src, dst, map, n_limbs, s, sched, factor);
         default: return CATFHE_EINVAL;
     }
 }

@@ -28,6 +28,8 @@
 // segmentation, Sec. 3.1.4, is replaced by batching).
 #include "bulk.cuh"
 #include "butterfly.cuh"
+#include <type_traits>
+
 #include "launch.cuh"
 #include "modarith.cuh"
 
@@ -416,10 +418,16 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
 
 // ------------------------------------------------------------------ inverse
 
-template <int LOGN, int LOGR, int LOGE, int NT, int MINB>
+// FACTOR: NttFactor to transform the products of two sources, formed as the
+// words are loaded (the multiplication's a1 b1), or NoFactor.
+struct NoFactor {};
+
+template <int LOGN, int LOGR, int LOGE, int NT, int MINB, class FACTOR>
 __global__ void __launch_bounds__(NT, MINB)
 k_ntt_inv_rows(const uint64_t *src, uint64_t *dst, const LimbMap map,
-               const DevMod *__restrict__ mods, const ulonglong2 *__restrict__ tw) {
+               const DevMod *__restrict__ mods, const ulonglong2 *__restrict__ tw,
+               const FACTOR factor) {
+    constexpr bool PROD = std::is_same<FACTOR, NttFactor>::value;
     grid_dep_wait();
     constexpr int R = 1 << LOGR, E = 1 << LOGE, T = R / E, CC = NT / T;
     constexpr int RP = R + R / E;
@@ -460,8 +468,25 @@ k_ntt_inv_rows(const uint64_t *src, uint64_t *dst, const LimbMap map,
         }
     }
     uint64_t x[E];
+    if constexpr (PROD) {
+        const uint64_t *fb = (map.gathered ? factor.gb[g] : factor.b + size_t(g) * map.src_stride * N) +
+                             size_t(map.src_off[r]) * N + size_t(h) * R;
+        const DevMod m = mods[p];
+        constexpr int G = E < 8 ? E : 8;  // words in flight per source
 #pragma unroll
-    for (int v = 0; v < E; v++) s[PAD(tau + T * v)] = ib[tau + T * v];
+        for (int v0 = 0; v0 < E; v0 += G) {
+            uint64_t fa[G], fc[G];
+#pragma unroll
+            for (int v = 0; v < G; v++) fa[v] = ib[tau + T * (v0 + v)];
+#pragma unroll
+            for (int v = 0; v < G; v++) fc[v] = fb[tau + T * (v0 + v)];
+#pragma unroll
+            for (int v = 0; v < G; v++) s[PAD(tau + T * (v0 + v))] = mul_mod_mont(fa[v], fc[v], m);
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < E; v++) s[PAD(tau + T * v)] = ib[tau + T * v];
+    }
     // the last LOGE stages' chunk twiddles, staged with the data (same barrier)
     __shared__ ulonglong2 tw1[CC * (E - 1)];
     stage_chunk_twiddles<LOGN, LOGR, LOGE, NT>(tw1, w);
@@ -617,11 +642,15 @@ static int run_fwd(const Context &c, const uint64_t *src, uint64_t *dst, const L
 
 template <int LN, int R1, int E1, int T1, int B1, int R2, int E2, int T2, int B2>
 static int run_inv(const Context &c, const uint64_t *src, uint64_t *dst, const LimbMap &map,
-                   uint32_t n_limbs, cudaStream_t s) {
+                   uint32_t n_limbs, cudaStream_t s, const NttFactor *factor) {
     constexpr size_t N = size_t(1) << LN;
     const dim3 g2(unsigned((N >> R2) / (T2 / ((1 << R2) >> E2))), n_limbs);
-    launch_pdl(k_ntt_inv_rows<LN, R2, E2, T2, B2>, g2, dim3(T2), 0, s, src, dst, map, c.d_mods,
-               c.d_twi);
+    if (factor)
+        launch_pdl(k_ntt_inv_rows<LN, R2, E2, T2, B2, NttFactor>, g2, dim3(T2), 0, s, src, dst, map,
+                   c.d_mods, c.d_twi, *factor);
+    else
+        launch_pdl(k_ntt_inv_rows<LN, R2, E2, T2, B2, NoFactor>, g2, dim3(T2), 0, s, src, dst, map,
+                   c.d_mods, c.d_twi, NoFactor{});
     const dim3 g1(unsigned((N >> R1) / (T1 / ((1 << R1) >> E1))), n_limbs);
     launch_pdl(k_ntt_inv_cols<LN, R1, E1, T1, B1>, g1, dim3(T1), 0, s, dst, map, c.d_mods,
                c.d_twi);

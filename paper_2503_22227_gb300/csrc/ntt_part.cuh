@@ -23,11 +23,12 @@ int NTT_CAT(ntt_fwd_n, NTT_LOGN)(const Context &c, const uint64_t *src, uint64_t
 }
 
 int NTT_CAT(ntt_inv_n, NTT_LOGN)(const Context &c, const uint64_t *src, uint64_t *dst,
-                                 const LimbMap &map, uint32_t n_limbs, cudaStream_t s, int sched) {
+                                 const LimbMap &map, uint32_t n_limbs, cudaStream_t s, int sched,
+                                 const NttFactor *factor) {
 #define INV(LN, S, A, B, TA, BA, C, D, TC, BC)                                               \
     if constexpr (LN == NTT_LOGN) {                                                         \
         if (sched == S)                                                                     \
-            return run_inv<LN, A, B, TA, BA, C, D, TC, BC>(c, src, dst, map, n_limbs, s);   \
+            return run_inv<LN, A, B, TA, BA, C, D, TC, BC>(c, src, dst, map, n_limbs, s, factor); \
     }
     NTT_SCHEDULES(INV)
 #undef INV

@@ -360,13 +360,10 @@ static int modup_ntt(Context &c, const KsConsts &k, const uint64_t *d2c, size_t 
 }
 
 // own, add0, add1: one limb group of `level` limbs per ciphertext, in_item
-// words apart (null: none).  gth (rotations): ciphertext i's add0 and own are
-// the two polynomials of gth->a[i].  key2: a second key, its result in y2.
-static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, const uint64_t *own,
-                         const uint64_t *key, const uint64_t *add0, const uint64_t *add1,
-                         size_t in_item, uint64_t *y, uint32_t count, cudaStream_t s,
-                         const Gather *gth = nullptr, const uint64_t *key2 = nullptr,
-                         uint64_t *y2 = nullptr) {
+// words apart (null: none).
+static IpArgs ip_args(const KsConsts &k, const uint64_t *ext, const uint64_t *own,
+                      const uint64_t *key, const uint64_t *add0, const uint64_t *add1,
+                      size_t in_item, uint64_t *y) {
     IpArgs a = k.ip;
     a.ext = ext;
     a.own = own;
@@ -374,9 +371,20 @@ static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, con
     a.add0 = add0;
     a.add1 = add1;
     a.y = y;
+    a.own_item = a.add_item = in_item;
+    return a;
+}
+
+// gth (rotations): ciphertext i's add0 and own are the two polynomials of
+// gth->a[i].  key2: a second key, its result in y2.
+static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, const uint64_t *own,
+                         const uint64_t *key, const uint64_t *add0, const uint64_t *add1,
+                         size_t in_item, uint64_t *y, uint32_t count, cudaStream_t s,
+                         const Gather *gth = nullptr, const uint64_t *key2 = nullptr,
+                         uint64_t *y2 = nullptr) {
+    IpArgs a = ip_args(k, ext, own, key, add0, add1, in_item, y);
     a.key2 = key2;
     a.y2 = y2;
-    a.own_item = a.add_item = in_item;
     if (gth && gth->n) {
         a.gathered = 1;
         for (uint32_t i = 0; i < gth->n; i++) a.ga[i] = gth->a[i];
@@ -533,6 +541,31 @@ static int key_for(const Keys &k, uint64_t id, const uint64_t **key) {
     return CATFHE_OK;
 }
 
+// The map of the a1 polynomials of ciphertexts [2][lvl][N]: limb lvl + i of
+// each group into limb i of a buffer of lvl limbs per group.
+static LimbMap map_second(int lvl) {
+    LimbMap m{};
+    m.period = uint32_t(lvl);
+    m.src_stride = uint32_t(2 * lvl);
+    m.dst_stride = uint32_t(lvl);
+    for (int i = 0; i < lvl; i++) {
+        m.src_off[i] = uint16_t(lvl + i);
+        m.dst_off[i] = uint16_t(i);
+        m.prime[i] = uint8_t(i);
+    }
+    return m;
+}
+
+// Up to kProductWords words (N limbs ciphertexts) a multiplication has no
+// tensor kernel, which saves a launch and 5 passes over them but forms a1 b1
+// twice.  Device time with the kernel -> without (us): N = 2^12, 3 limbs 24.6 ->
+// 24.0 (and 5 of 37 us of host time), 2^13, 7 limbs 37.4 -> 36.5, 2^15, 12 limbs
+// 71.8 -> 70.9, 2^16, 7 limbs 78.0 -> 75.8; past it the products weigh more than
+// the launch, the more so beside another half: 2^16, 24 limbs 198.0 both ways, 8 x
+// 2^14, 8 limbs (each half of 16 BGV products) 315 -> 323, 8 x 2^16, 24 limbs
+// 1101 -> 1117.
+constexpr size_t kProductWords = size_t(1) << 19;
+
 // CKKS / BGV: tensor in NTT form, INTT d2, ModUp, NTT, inner product with
 // P*(d0, d1) folded in, ModDown (fused: by P q_{l-1}).
 static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
@@ -542,11 +575,40 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(key_for(keys, 0, &rlk));
     const KsConsts *ks;
     TRY(ks_consts(c, level, fused, &ks));
-    const size_t n = c.n;
+    const size_t n = c.n, half = size_t(level) * n, item = 2 * half;
+    const bool gathered = gth && gth->n;
+    if (ks->ip.beta <= kIpBulkBeta && size_t(count) * half <= kProductWords) {
+        // no tensor kernel: the inverse transform forms a1 b1 as it loads, and
+        // the inner product the three products of its own tile
+        LimbMap m = map_second(level);
+        NttFactor f{};
+        f.b = b;
+        if (gathered) {
+            m.gathered = 1;
+            for (uint32_t i = 0; i < gth->n; i++) {
+                m.gsrc[i] = gth->a[i];
+                f.gb[i] = gth->b[i];
+            }
+        }
+        TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(level) * count, s, &f));
+        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+        IpArgs ip = ip_args(*ks, k.ext, a + half, rlk, a, nullptr, item, k.y);
+        ip.product = 1;
+        ip.b = b;
+        if (gathered) {
+            ip.gathered = 1;
+            for (uint32_t i = 0; i < gth->n; i++) {
+                ip.ga[i] = gth->a[i];
+                ip.gb[i] = gth->b[i];
+            }
+        }
+        TRY(launch_ip(c, ip, count, s));
+        return moddown(c, *ks, k.y, k.lift, out, count, s, 0, gth);
+    }
     TensorArgs t{};
     t.a = a;
     t.b = b;
-    if (gth && gth->n) {
+    if (gathered) {
         t.gathered = 1;
         for (uint32_t i = 0; i < gth->n; i++) {
             t.ga[i] = gth->a[i];
@@ -556,15 +618,15 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     t.d0 = k.d0;
     t.d1 = k.d1;
     t.d2 = k.d2;
-    t.in_item = size_t(2) * level * n;
-    t.out_item = size_t(level) * n;
+    t.in_item = item;
+    t.out_item = half;
     t.limbs = uint32_t(level);
     for (int i = 0; i < level; i++) t.prime[i] = uint8_t(i);
     TRY(launch_tensor(c, t, count, s));
     LimbMap m = map_identity(uint32_t(level));
     TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(level) * count, s));
-    TRY(modup_ntt(c, *ks, k.d2c, size_t(level) * n, k.ext, count, s));
-    TRY(inner_product(c, *ks, k.ext, k.d2, rlk, k.d0, k.d1, size_t(level) * n, k.y, count, s));
+    TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+    TRY(inner_product(c, *ks, k.ext, k.d2, rlk, k.d0, k.d1, half, k.y, count, s));
     return moddown(c, *ks, k.y, k.lift, out, count, s, 0, gth);
 }
 
@@ -785,21 +847,6 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
     return run(0, count, base, s);
 }
 
-// The map of the a1 polynomials of ciphertexts [2][lvl][N]: limb lvl + i of
-// each group into limb i of a buffer of lvl limbs per group.
-static LimbMap map_second(int lvl) {
-    LimbMap m{};
-    m.period = uint32_t(lvl);
-    m.src_stride = uint32_t(2 * lvl);
-    m.dst_stride = uint32_t(lvl);
-    for (int i = 0; i < lvl; i++) {
-        m.src_off[i] = uint16_t(lvl + i);
-        m.dst_off[i] = uint16_t(i);
-        m.prime[i] = uint8_t(i);
-    }
-    return m;
-}
-
 // HRotate of count ciphertexts at lvl with the Galois key gk, workspace k.
 // sigma_g commutes with every step of the key switching: it permutes slots
 // (and signs of coefficients), the centred lifts are odd functions and no
@@ -922,7 +969,7 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
         TRY(down(r, kb, kb.y, st));
         return down(r + 1, kb, kb.ext, st);
     };
-    const bool pair = beta >= 2 && beta <= kIpPairBeta;
+    const bool pair = beta >= 2 && uint32_t(beta) <= kIpBulkBeta;
     if (n_rot < 2 || c.log_n < 14) {
         uint32_t r = 0;
         for (; pair && r + 1 < n_rot; r += 2) TRY(two(r, k, s));
