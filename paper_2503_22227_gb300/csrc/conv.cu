@@ -16,7 +16,8 @@
 //
 // Every sum is accumulated exactly in 128 bits and reduced once, so there is
 // no floating-point estimate and no approximation: the result is the
-// definition, bit for bit.  Two constant layouts exist (see internal.h):
+// definition, bit for bit.  This file has the integer kernels (conv_mma.cu the
+// tensor-core one; launch_conv chooses).  Three constant layouts (internal.h):
 //
 //  - Montgomery (used whenever sum(m_i) + 1 < 2^64): every constant is
 //    stored times 2^64 mod its modulus, the mixed-radix step of a_j is ONE
@@ -25,6 +26,8 @@
 //    by a single Montgomery reduction: u = lo * (-p^-1) mod 2^64,
 //    (acc + u p) / 2^64 = hi + mulhi(u, p) + [lo != 0], in [0, 2p) because
 //    acc < 2^64 p;
+//  - the same with every weight in two 30-bit halves (at most 8 sources, moduli
+//    below 2^60): three 32-bit products a term, no carries;
 //  - exact (fallback): each sum reduced by hi*(2^64 mod p) + lo (Shoup).
 //
 // One thread handles one coefficient of one item; the packed plan (a few
@@ -275,12 +278,10 @@ __device__ __forceinline__ uint64_t ld_plan(const uint64_t *p) {
 // Mixed-radix digits as 30-bit halves, and the centring decision (the
 // lexicographic comparison with the digits of (M-1)/2 runs from the least
 // significant digit up: the last differing digit decides).
-// EXACT: every plan of the launch has k = KMAX sources, so the source count
-// and the constants' row stride are compile-time constants.
-template <int KMAX, bool EXACT>
+template <int KMAX>
 __device__ __forceinline__ bool mixed_radix_split(const uint64_t (&r)[KMAX], uint32_t (&al)[KMAX],
                                                   uint32_t (&ah)[KMAX], const MontView &P) {
-    const uint32_t k = EXACT ? uint32_t(KMAX) : P.k;
+    const uint32_t k = P.k;
     bool gt = false;
 #pragma unroll
     for (int j = 0; j < KMAX; j++) {
@@ -303,11 +304,11 @@ __device__ __forceinline__ bool mixed_radix_split(const uint64_t (&r)[KMAX], uin
 }
 
 // Targets t and t+1 (two independent chains).
-template <int KMAX, bool EXACT>
+template <int KMAX>
 __device__ __forceinline__ void eval_split2(const uint32_t (&al)[KMAX], const uint32_t (&ah)[KMAX],
                                             bool gt, const MontView &P, uint32_t t, uint64_t &r0,
                                             uint64_t &r1) {
-    const uint32_t T = P.T, k = EXACT ? uint32_t(KMAX) : P.k;
+    const uint32_t T = P.T, k = P.k;
     Acc3 a0{0, 0, 0}, a1{0, 0, 0};
 #pragma unroll
     for (int i = 0; i < KMAX; i++) {
@@ -331,11 +332,11 @@ __device__ __forceinline__ void eval_split2(const uint32_t (&al)[KMAX], const ui
     }
 }
 
-template <int KMAX, bool EXACT>
+template <int KMAX>
 __device__ __forceinline__ uint64_t eval_split(const uint32_t (&al)[KMAX],
                                                const uint32_t (&ah)[KMAX], bool gt,
                                                const MontView &P, uint32_t t) {
-    const uint32_t k = EXACT ? uint32_t(KMAX) : P.k;
+    const uint32_t k = P.k;
     Acc3 a{0, 0, 0};
 #pragma unroll
     for (int i = 0; i < KMAX; i++)
@@ -514,7 +515,7 @@ __device__ __forceinline__ void load_sources(uint64_t (&a)[KMAX], uint32_t k,
     for (int i = 0; i < KMAX; i++) a[i] = uint32_t(i) < k ? s[src_off[i] * n + x] : 0;
 }
 
-template <int KMAX, bool MONT, bool SPLIT = false, bool EXACT = false>
+template <int KMAX, bool MONT, bool SPLIT = false>
 __global__ void __launch_bounds__(256, 4)
 k_conv(const PlanList plans, const uint64_t *__restrict__ src, size_t src_item, size_t src_plan,
        uint64_t *__restrict__ dst, size_t dst_item, size_t dst_plan, uint32_t log_n) {
@@ -531,17 +532,17 @@ k_conv(const PlanList plans, const uint64_t *__restrict__ src, size_t src_item, 
         for (size_t x = size_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n;
              x += size_t(gridDim.x) * blockDim.x) {
             uint64_t r[KMAX];
-            load_sources<KMAX>(r, EXACT ? uint32_t(KMAX) : P.k, P.src_off, s, x, n);
+            load_sources<KMAX>(r, P.k, P.src_off, s, x, n);
             uint32_t al[KMAX], ah[KMAX];
-            const bool gt = mixed_radix_split<KMAX, EXACT>(r, al, ah, P);
+            const bool gt = mixed_radix_split<KMAX>(r, al, ah, P);
             uint32_t t = 0;
             for (; t + 1 < P.T; t += 2) {
                 uint64_t r0, r1;
-                eval_split2<KMAX, EXACT>(al, ah, gt, P, t, r0, r1);
+                eval_split2<KMAX>(al, ah, gt, P, t, r0, r1);
                 d[P.dst_off[t] * n + x] = r0;
                 d[P.dst_off[t + 1] * n + x] = r1;
             }
-            if (t < P.T) d[P.dst_off[t] * n + x] = eval_split<KMAX, EXACT>(al, ah, gt, P, t);
+            if (t < P.T) d[P.dst_off[t] * n + x] = eval_split<KMAX>(al, ah, gt, P, t);
         }
     } else if (MONT) {
         const MontView P = mont_view(splan);
@@ -734,7 +735,8 @@ int launch_conv(const Context &c, const ConvPlans &cp, const uint64_t *src, size
             (reinterpret_cast<uintptr_t>(dst) & 15) == 0 && (src_item | src_plan | dst_item |
                                                               dst_plan) % 2 == 0 && n % 256 == 0) {
             // one source count for every plan, 16-byte aligned sources and
-            // results: exact instantiation, two coefficients per thread
+            // results (every buffer's are): exact instantiation, two
+            // coefficients per thread
             const dim3 g2(unsigned(n / 256), items, plans.n);
             switch (plans.kmax) {
 #define PAIRK(K)                                                                               \
@@ -744,19 +746,6 @@ int launch_conv(const Context &c, const ConvPlans &cp, const uint64_t *src, size
         break;
                 PAIRK(1) PAIRK(2) PAIRK(3) PAIRK(4) PAIRK(5) PAIRK(6) PAIRK(7) PAIRK(8)
 #undef PAIRK
-                default:
-                    return CATFHE_EINVAL;
-            }
-        } else if (plans.kmin == plans.kmax) {
-            // one source count for every plan: exact instantiation
-            switch (plans.kmax) {
-#define EXACTK(K)                                                                              \
-    case K:                                                                                    \
-        launch_pdl(k_conv<K, true, true, true>, grid, dim3(256), sm, s, plans, src, src_item, src_plan, dst, \
-                                                          dst_item, dst_plan, c.log_n);        \
-        break;
-                EXACTK(1) EXACTK(2) EXACTK(3) EXACTK(4) EXACTK(5) EXACTK(6) EXACTK(7) EXACTK(8)
-#undef EXACTK
                 default:
                     return CATFHE_EINVAL;
             }
