@@ -45,6 +45,11 @@ static int mw_cmp(const std::vector<uint64_t> &a, const std::vector<uint64_t> &b
     return 0;
 }
 
+cudaError_t copy_in(void *dev, const void *host, size_t bytes) {
+    const cudaError_t e = cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 static int check(cudaError_t e) { return e == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA; }
 
 int ctx_init(Context &c, const catfhe_params &p) {
@@ -139,9 +144,9 @@ int ctx_init(Context &c, const catfhe_params &p) {
     if (cudaMalloc(&c.d_mods, sizeof(DevMod) * np) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMalloc(&c.d_twf, sizeof(ulonglong2) * np * n) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMalloc(&c.d_twi, sizeof(ulonglong2) * np * n) != cudaSuccess) return CATFHE_ENOMEM;
-    int rc = check(cudaMemcpy(c.d_mods, c.hmods.data(), sizeof(DevMod) * np, cudaMemcpyHostToDevice));
-    if (!rc) rc = check(cudaMemcpy(c.d_twf, twf.data(), sizeof(ulonglong2) * np * n, cudaMemcpyHostToDevice));
-    if (!rc) rc = check(cudaMemcpy(c.d_twi, twi.data(), sizeof(ulonglong2) * np * n, cudaMemcpyHostToDevice));
+    int rc = check(copy_in(c.d_mods, c.hmods.data(), sizeof(DevMod) * np));
+    if (!rc) rc = check(copy_in(c.d_twf, twf.data(), sizeof(ulonglong2) * np * n));
+    if (!rc) rc = check(copy_in(c.d_twi, twi.data(), sizeof(ulonglong2) * np * n));
     return rc;
 }
 
@@ -333,7 +338,7 @@ static PlanRef upload_plan(Context &c, const std::string &key, std::vector<uint6
     host.insert(host.end(), extra.begin(), extra.end());
     uint64_t *dev = nullptr;
     if (cudaMalloc(&dev, host.size() * 8) != cudaSuccess) return ref;
-    if (cudaMemcpy(dev, host.data(), host.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (copy_in(dev, host.data(), host.size() * 8) != cudaSuccess) {
         cudaFree(dev);
         return ref;
     }
@@ -368,7 +373,7 @@ MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec,
     if (!img.empty()) {
         uint64_t *dev = nullptr;
         if (cudaMalloc(&dev, img.size() * 8) != cudaSuccess) return ref;
-        if (cudaMemcpy(dev, img.data(), img.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (copy_in(dev, img.data(), img.size() * 8) != cudaSuccess) {
             cudaFree(dev);
             return ref;
         }
@@ -403,7 +408,7 @@ const LiftEntry *upload_lifts(Context &c, const std::vector<LiftEntry> &table) {
     LiftEntry *dev = nullptr;
     const size_t bytes = table.size() * sizeof(LiftEntry);
     if (cudaMalloc(&dev, bytes) != cudaSuccess) return nullptr;
-    if (cudaMemcpy(dev, table.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (copy_in(dev, table.data(), bytes) != cudaSuccess) {
         cudaFree(dev);
         return nullptr;
     }
@@ -414,7 +419,7 @@ const LiftEntry *upload_lifts(Context &c, const std::vector<LiftEntry> &table) {
 const uint64_t *upload_words(Context &c, const std::string &key, const std::vector<uint64_t> &w) {
     uint64_t *dev = nullptr;
     if (cudaMalloc(&dev, w.size() * 8) != cudaSuccess) return nullptr;
-    if (cudaMemcpy(dev, w.data(), w.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (copy_in(dev, w.data(), w.size() * 8) != cudaSuccess) {
         cudaFree(dev);
         return nullptr;
     }

@@ -148,8 +148,8 @@ int enc_tables(Context &c) {
         cudaFree(d);
         return CATFHE_ENOMEM;
     }
-    if (cudaMemcpy(d, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(di, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (copy_in(d, h.data(), h.size() * sizeof(double2)) != cudaSuccess ||
+        copy_in(di, idx.data(), idx.size() * 4) != cudaSuccess) {
         cudaFree(d);
         cudaFree(di);
         return CATFHE_ECUDA;

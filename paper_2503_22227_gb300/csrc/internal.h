@@ -80,6 +80,11 @@ __host__ __device__ inline size_t plan_words(uint64_t header) {
                       ((header >> 34) & 1) != 0);
 }
 
+// Copies constants to the device and waits until they are there: from pageable
+// memory cudaMemcpy returns once the bytes are staged, and the streams that read
+// the constants next need not be ordered after it.
+cudaError_t copy_in(void *dev, const void *host, size_t bytes);
+
 // Source / target description of a conversion plan.  A target modulus of 0
 // means 2^64 (two's complement output).  Empty pre / post mean 1.
 struct PlanSpec {
