@@ -159,7 +159,7 @@ struct IpTile {
 // ciphertexts at N = 2^16, l = 24 (453 MB) are read once for both, 1550 ->
 // 1098 MB a pair.  Tiles of 256
 // coefficients from 3 digits on, so that the key tiles and the two buffers
-// (44 KB at 3 digits) leave room for 3 CTAs per SM in the 164 KB split that
+// (40 KB at 3 digits) leave room for 4 CTAs per SM in the 164 KB split that
 // these launches ask for (tiles of 512 are slower, 8080 instead of 8023 us).
 // The batch of 16 rotations of 8: 8128 -> 8023 us (the transforms that run
 // beside it bound it); 16 rotations of one: 1349 -> 1267 us; 4 at N = 2^12:
