@@ -141,10 +141,21 @@ int ctx_init(Context &c, const catfhe_params &p) {
         return CATFHE_ECUDA;
     if (cudaMalloc(&c.d_status, sizeof(int)) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMemset(c.d_status, 0, sizeof(int)) != cudaSuccess) return CATFHE_ECUDA;
-    if (cudaMalloc(&c.d_mods, sizeof(DevMod) * np) != cudaSuccess) return CATFHE_ENOMEM;
+    std::vector<DevMod> mods = c.hmods;
+    if (c.scheme == CATFHE_BGV)  // once more with t^-1 in the inverse transform's N^-1
+        for (DevMod m : c.hmods) {
+            const uint64_t ti = h_invmod(c.t % m.q, m.q);
+            m.ninv = h_mulmod(m.ninv, ti, m.q);
+            m.ninv_s = h_shoup(m.ninv, m.q);
+            m.ninvw = h_mulmod(m.ninvw, ti, m.q);
+            m.ninvw_s = h_shoup(m.ninvw, m.q);
+            mods.push_back(m);
+        }
+    const size_t mods_bytes = sizeof(DevMod) * mods.size();
+    if (cudaMalloc(&c.d_mods, mods_bytes) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMalloc(&c.d_twf, sizeof(ulonglong2) * np * n) != cudaSuccess) return CATFHE_ENOMEM;
     if (cudaMalloc(&c.d_twi, sizeof(ulonglong2) * np * n) != cudaSuccess) return CATFHE_ENOMEM;
-    int rc = check(copy_in(c.d_mods, c.hmods.data(), sizeof(DevMod) * np));
+    int rc = check(copy_in(c.d_mods, mods.data(), mods_bytes));
     if (!rc) rc = check(copy_in(c.d_twf, twf.data(), sizeof(ulonglong2) * np * n));
     if (!rc) rc = check(copy_in(c.d_twi, twi.data(), sizeof(ulonglong2) * np * n));
     return rc;
@@ -384,15 +395,11 @@ MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec,
     return c.mma_plans[key] = ref;
 }
 
-LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post) {
+LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t post) {
     LiftEntry e{};
-    e.m = m;
     e.half = (m - 1) / 2;
-    e.pre = pre % m;
-    e.pre_s = h_shoup(e.pre, m);
     e.post = post % p;
     e.post_s = h_shoup(e.post, p);
-    if (e.pre != 1) e.flags |= kLiftPre;
     if (e.post != 1)
         e.flags |= kLiftPost;
     else if ((m - 1) / 4 >= p)  // m > 4p

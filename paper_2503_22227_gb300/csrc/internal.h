@@ -48,6 +48,9 @@ struct LimbMap {
     // (gathered ciphertexts) instead of src + g * src_stride limbs
     uint32_t gathered;
     const uint64_t *gsrc[kGatherMax];
+    // inverse transform only: the column pass's constants are those at this
+    // offset of the table (BGV: np, where N^-1 stands for N^-1 t^-1)
+    uint32_t mods_off;
 };
 
 // Constants of one exact, centred base conversion from k source moduli to T
@@ -164,20 +167,19 @@ inline uint32_t mma_targets(uint64_t counts) {
 std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t target_unit);
 
 // A centred lift from one source modulus m to a target p, for the kernels that
-// lift as they load (one entry per position of a launch's map): y = a pre mod
-// m, x = y post (+ cst when y > half) mod p, unreduced (below 4p).
+// lift as they load (one entry per position of a launch's map): x = y post (+ cst
+// when y > half) mod p, unreduced (below 4p).
 struct LiftEntry {
-    uint64_t m, half;       // source modulus, (m - 1) / 2
-    uint64_t pre, pre_s;    // kLiftPre: factor mod m (Shoup pair)
+    uint64_t half;          // (m - 1) / 2
     uint64_t post, post_s;  // kLiftPost: factor mod p (Shoup pair)
     uint64_t cst;           // -m post mod p (without kLiftPost and kLiftReduce: 4p - m or less)
     uint64_t flags;
 };
-constexpr uint64_t kLiftPre = 1, kLiftPost = 2, kLiftReduce = 4;
+constexpr uint64_t kLiftPost = 2, kLiftReduce = 4;
 // The words are signed integers instead, reduced mod p (nothing else is read).
 constexpr uint64_t kLiftSigned = 8;
-// The entry for source m, target p and factors pre, post (1: none).
-LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t pre, uint64_t post);
+// The entry for source m, target p and factor post (1: none).
+LiftEntry lift_entry(uint64_t m, uint64_t p, uint64_t post);
 // Device copy of a lift table, freed with the context (null: no memory).
 const LiftEntry *upload_lifts(Context &c, const std::vector<LiftEntry> &table);
 

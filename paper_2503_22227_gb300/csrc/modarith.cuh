@@ -231,18 +231,16 @@ __device__ __forceinline__ uint64_t reduce_lazy3(uint64_t x, uint64_t q, uint32_
     return x - uint64_t(__umulhi(uint32_t(x >> 32), m64)) * q;
 }
 
-// One word through a lift (LiftEntry): a in [0, m) to below 4q.
-__device__ __forceinline__ uint64_t lift_word(uint64_t a, const LiftEntry &e, const DevMod &t) {
+// One word through a lift (LiftEntry): y in [0, m) to below 4q.
+__device__ __forceinline__ uint64_t lift_word(uint64_t y, const LiftEntry &e, const DevMod &t) {
     const uint64_t q = t.q;
     if (e.flags & kLiftSigned) {
-        const bool neg = int64_t(a) < 0;
-        const uint64_t mag = neg ? 0 - a : a;
+        const bool neg = int64_t(y) < 0;
+        const uint64_t mag = neg ? 0 - y : y;
         const uint64_t r =
             t.m64 ? reduce_lazy3(mag, q, uint32_t(t.m64)) : shoup_lazy(mag, 1, t.one_s, q);
         return neg ? 3 * q - r : r;
     }
-    uint64_t y = a;
-    if (e.flags & kLiftPre) y = csub(csub(shoup_lazy4(a, e.pre, e.pre_s, e.m), 2 * e.m), e.m);
     uint64_t r = y;
     if (e.flags & kLiftPost)
         r = csub(shoup_lazy4(y, e.post, e.post_s, q), 2 * q);

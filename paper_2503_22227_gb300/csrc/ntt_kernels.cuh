@@ -546,7 +546,7 @@ k_ntt_inv_cols(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
     constexpr size_t S = N >> LOGR;
     uint64_t *out = data + (size_t(g) * map.dst_stride + map.dst_off[r]) * N;
     const int p = map.prime[r];
-    const DevMod m = mods[p];
+    const DevMod m = mods[map.mods_off + p];
     const uint64_t q = m.q;
     const ulonglong2 *wg = tw + size_t(p) * N;
     const int cl = threadIdx.x % CW, tau = threadIdx.x / CW;
