@@ -1233,9 +1233,9 @@ struct DevConst {
         for (size_t i = 0; i < vals.size(); i++) sh[i] = h_shoup(vals[i], mods[i]);
         if (cudaMalloc(&v, vals.size() * 8) != cudaSuccess) return CATFHE_ENOMEM;
         if (cudaMalloc(&s, vals.size() * 8) != cudaSuccess) return CATFHE_ENOMEM;
-        if (cudaMemcpy(v, vals.data(), vals.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess)
-            return CATFHE_ECUDA;
-        if (cudaMemcpy(s, sh.data(), vals.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess)
+        // the kernels that read them may run on a stream of the caller's
+        if (copy_in(v, vals.data(), vals.size() * 8) != cudaSuccess ||
+            copy_in(s, sh.data(), vals.size() * 8) != cudaSuccess)
             return CATFHE_ECUDA;
         return CATFHE_OK;
     }
