@@ -123,7 +123,9 @@ k_fft_high(const double2 *__restrict__ in, const double2 *__restrict__ tw,
 
 // Tables: d_enc = [twist zeta^i (N)][omega^k (N/2)][omega^-k (N/2)],
 // d_slot[j] = the slot k whose point j(k) is, or k | 2^31 where j is j'(k).
+// Threads may make their first calls on one context at the same time.
 int enc_tables(Context &c) {
+    std::lock_guard<std::mutex> lock(c.mu);
     if (c.d_enc) return CATFHE_OK;
     const size_t n = c.n, half = n / 2;
     std::vector<double2> h(2 * n);
