@@ -13,6 +13,7 @@
 #include <string>
 
 #include "internal.h"
+#include "lanes.h"
 
 namespace catfhe {
 
@@ -560,28 +561,52 @@ static LimbMap map_second(int lvl) {
     return m;
 }
 
-// Up to kProductWords words (N limbs ciphertexts) a multiplication has no
-// tensor kernel, which saves a launch and 5 passes over them but forms a1 b1
-// twice.  Device time with the kernel -> without (us): N = 2^12, 3 limbs 24.6 ->
-// 24.0 (and 5 of 37 us of host time), 2^13, 7 limbs 37.4 -> 36.5, 2^15, 12 limbs
-// 71.8 -> 70.9, 2^16, 7 limbs 78.0 -> 75.8; past it the products weigh more than
-// the launch, the more so beside another half: 2^16, 24 limbs 198.0 both ways, 8 x
-// 2^14, 8 limbs (each half of 16 BGV products) 315 -> 323, 8 x 2^16, 24 limbs
-// 1101 -> 1117.
-constexpr size_t kProductWords = size_t(1) << 19;
+// Whether a multiplication of `count` ciphertexts has no tensor kernel: the
+// inverse transform and the inner product then form the products, which saves a
+// launch and 5 passes over them but forms a1 b1 twice, and one CTA of the
+// inner product forms those of its ciphertexts one after another.
+// beside: other operations or another half run at the same time.
+//
+// The launch is what counts while the key switching is short, however the words
+// are spread over ciphertexts: up to kProductWork words of lifted digits and
+// sums ((digits + 2) (l + K) N per ciphertext).  us with the tensor kernel ->
+// without: N = 2^12, 3 limbs, 1 digit 36.1 -> 33.0, 8 of them 36.5 -> 34.3, 8
+// limbs x 2 36.9 -> 33.3; halves at 2^14, 3 limbs x 4 61.7 -> 57.6, BGV 2 limbs x
+// 8 55.4 -> 49.9.  At the line both routes are level (2^12, 12 limbs x 4 41.1 ->
+// 41.1; 2^14, 3 limbs x 3 44.6 -> 44.3); past it the products weigh more, 2^12,
+// 2 limbs x 16 41.3 -> 44.0, 2^14, 2 limbs x 16 92.6 -> 96.7, 9 limbs x 5 97.3 ->
+// 105.2, 2^15, 2 limbs x 4 67.7 -> 71.9, 2^16, 2 limbs x 8 167.0 -> 175.1.
+// Up to kProductFew ciphertexts with nothing beside them keep the route to
+// kProductWords words, where the kernels wait for their loads more than for
+// multiplications: 2^14, 16 limbs x 2 75.3 -> 73.7, 24 limbs 74.0 -> 72.5, BGV 8
+// limbs x 3 84.7 -> 83.5, 2^15, 16 limbs 79.4 -> 77.9, 2^16, 8 limbs 81.9 -> 79.2
+// (and 2^14, 9 limbs x 2 55.1 -> 56.0; one ciphertext at 2^16, 24 limbs is level,
+// 198.0).  With fewer limbs than special primes most of the inner product's
+// CTAs have no product to form and wait for those that do: 2^16, 3 limbs 54.9 ->
+// 56.0, 2^15, 2 limbs x 2 48.8 -> 50.2, so these stay with the tensor kernel.
+// A batch on lanes: 8 operations 271.3 with it, 273.8 without, 16 463 and 472.
+constexpr size_t kProductWork = size_t(1) << 20, kProductWords = size_t(1) << 19;
+constexpr uint32_t kProductFew = 3;
+static bool forms_products(const Context &c, const IpArgs &ip, uint32_t level, uint32_t count,
+                           bool beside) {
+    if (ip.beta > kIpBulkBeta) return false;
+    if (size_t(count) * (ip.beta + 2) * ip.M * c.n <= kProductWork) return true;
+    return !beside && count <= kProductFew && int(level) > c.K &&
+           size_t(count) * level * c.n <= kProductWords;
+}
 
 // CKKS / BGV: tensor in NTT form, INTT d2, ModUp, NTT, inner product with
 // P*(d0, d1) folded in, ModDown (fused: by P q_{l-1}).
 static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
                          uint64_t *out, uint32_t count, int level, bool fused, KsBufs &k,
-                         cudaStream_t s, const Gather *gth) {
+                         cudaStream_t s, const Gather *gth, bool beside) {
     const uint64_t *rlk;
     TRY(key_for(keys, 0, &rlk));
     const KsConsts *ks;
     TRY(ks_consts(c, level, fused, &ks));
     const size_t n = c.n, half = size_t(level) * n, item = 2 * half;
     const bool gathered = gth && gth->n;
-    if (ks->ip.beta <= kIpBulkBeta && size_t(count) * half <= kProductWords) {
+    if (forms_products(c, ks->ip, uint32_t(level), count, beside)) {
         // no tensor kernel: the inverse transform forms a1 b1 as it loads, and
         // the inner product the three products of its own tile
         LimbMap m = map_second(level);
@@ -836,6 +861,7 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
     char *base;
     TRY(get_ws(c, ws, ws_bytes_in, need, &base));
     const int lvl = int(level);
+    const bool halves = split && !(gth && gth->n) && split_ok(c, count);
     auto run = [&](uint32_t first, uint32_t cnt, char *wbase, cudaStream_t st) -> int {
         Bump bump{wbase};
         KsBufs k{};
@@ -844,10 +870,10 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
         const uint64_t *ah = a + size_t(first) * 2 * lvl * n, *bh = b + size_t(first) * 2 * lvl * n;
         uint64_t *oh = out + size_t(first) * 2 * lo * n;
         if (c.scheme == CATFHE_BFV) return mul_relin_bfv(c, keys, ah, bh, oh, cnt, lvl, k, st);
-        return mul_relin_ntt(c, keys, ah, bh, oh, cnt, lvl, fused, k, st, gth);
+        return mul_relin_ntt(c, keys, ah, bh, oh, cnt, lvl, fused, k, st, gth,
+                             halves || LaneScope::active());
     };
-    if (split && !(gth && gth->n) && split_ok(c, count))
-        return run_halves(c, count, lvl, fused, base, s, run);
+    if (halves) return run_halves(c, count, lvl, fused, base, s, run);
     return run(0, count, base, s);
 }
 
