@@ -404,7 +404,8 @@ int catfhe_sync(catfhe_ctx *ctx, void *stream);
  * second (any pointer may be NULL); `stream` is synchronised.  These are
  * the integer-pipe ceilings the hot path is measured against.
  * catfhe_kernel_launches returns how many kernels the library has launched
- * since it was loaded. */
+ * since it was loaded, catfhe_tensor_conversions how many of them were base
+ * conversions (and BFV scale-and-rounds) on the tensor cores. */
 int catfhe_measure_int_peak(double *modmul_per_s, double *butterfly_per_s,
                             double *butterfly_wide_per_s, void *stream);
 /* The device's rates, over the whole GPU, of the three 32-bit multiply
@@ -418,6 +419,7 @@ int catfhe_measure_int_peak(double *modmul_per_s, double *butterfly_per_s,
 int catfhe_measure_imad_rates(double *lo_per_s, double *hi_per_s, double *wide_per_s,
                               void *stream);
 uint64_t catfhe_kernel_launches(void);
+uint64_t catfhe_tensor_conversions(void);
 
 /* ---- Uneven batches (many independent operations in one submission) ----
  * Each entry is one operation of any context (ring degree), level and kind;

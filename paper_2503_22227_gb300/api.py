@@ -44,6 +44,7 @@ EXPORTS = [
     "catfhe_encode_ckks", "catfhe_decode_ckks", "catfhe_device_status", "catfhe_wait_selftest",
     "catfhe_packed_words", "catfhe_ct_import_packed", "catfhe_ct_export_packed",
     "catfhe_pack_host", "catfhe_unpack_host", "catfhe_sync", "catfhe_measure_imad_rates",
+    "catfhe_tensor_conversions",
 ]
 
 
@@ -129,6 +130,7 @@ def load(path: str = LIB_PATH):
             "catfhe_measure_int_peak": (ctypes.c_int, [vp, vp, vp, vp]),
             "catfhe_measure_imad_rates": (ctypes.c_int, [vp, vp, vp, vp]),
             "catfhe_kernel_launches": (u64, []),
+            "catfhe_tensor_conversions": (u64, []),
             "catfhe_rescale_noalloc": (ctypes.c_int, [vp, vp, vp, u32, u32, vp]),
             "catfhe_sync": (ctypes.c_int, [vp, vp]),
             "catfhe_batch_workspace_bytes": (sz, [vp, u32, u32]),
@@ -570,6 +572,11 @@ def measure_imad_rates() -> tuple[float, float, float]:
 
 def kernel_launches() -> int:
     return int(load().catfhe_kernel_launches())
+
+
+def tensor_conversions() -> int:
+    """How many of the kernel launches were conversions on the tensor cores."""
+    return int(load().catfhe_tensor_conversions())
 
 
 def make_op(kind: int, ctx: "Context", a, out, keys: "Keys" = None, b=None, galois_elt: int = 0,

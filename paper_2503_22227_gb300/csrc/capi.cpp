@@ -440,6 +440,8 @@ int catfhe_measure_imad_rates(double *lo_per_s, double *hi_per_s, double *wide_p
 
 uint64_t catfhe_kernel_launches(void) { return launches_total(); }
 
+uint64_t catfhe_tensor_conversions(void) { return mma_launches_total(); }
+
 size_t catfhe_workspace_bytes(const catfhe_ctx *ctx, int op, uint32_t level, uint32_t count) {
     if (!ctx) return 0;
     return ws_bytes(ctx->c, op, level, count);

@@ -695,36 +695,14 @@ static void run_conv(int kmax, dim3 grid, size_t sm, cudaStream_t s, const PlanL
     }
 }
 
-// Whether the tensor-core form takes less time than the split-weight one, by
-// a model in cycles per warp of 32 coefficients: the integer kernel's multiply
-// pipe (12 a product, 24 a Montgomery reduction, 70% busy; mixed
-// source counts run one coefficient per thread, about a third slower) against
-// the other's issue slots (half busy) and its start (matrix, TMEM) of about
-// 2000.  A launch below two warps per scheduler takes as long as two.
-// Measured on GB300, us (integer / tensor): 8 sources, 20 targets, 3 x 4 x
-// 2^16 coefficients 103 / 59; 5 sources, 23 targets, 2^19 57 / 37; a whole
-// product at N = 2^12, 24 primes (8 and 5 sources) 43.0 / 38.9; at 3 primes (3
-// and 5 sources) 29.1 / 31.6, and at N = 2^16 57.2 / 59.9.
-static bool mma_is_faster(const ConvPlans &cp, size_t coeffs) {
-    if (!cp.l.split) return true;  // the other layouts are slower than both
-    double gain = 0;
-    for (uint32_t i = 0; i < cp.m.n; i++) {
-        const double K = double(cp.m.head[i] & 0xff), T = double(mma_targets(cp.m.counts[i]));
-        const double pair = (6 * K * (K + 1) + 24 * K + T * (12 * K + 24)) / 0.7;
-        gain += (cp.l.kmin == cp.l.kmax ? 1.0 : 1.3) * pair - (40 * K + 30 * T + 150) / 0.48;
-    }
-    const double warps = std::max(2.0, double(coeffs) * cp.m.n / 32 / (152 * 4));
-    return gain / cp.m.n * warps > 2000;
-}
-
 int launch_conv(const Context &c, const ConvPlans &cp, const uint64_t *src, size_t src_item,
                 size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan, uint32_t items,
-                cudaStream_t s) {
+                cudaStream_t s, bool beside) {
     const PlanList &plans = cp.l;
     if (plans.n == 0 || items == 0) return CATFHE_OK;
     // (its bulk copies need 16-byte aligned sources, as every buffer's are)
     if (cp.mma && ((reinterpret_cast<uintptr_t>(src) & 15) | ((src_item | src_plan) & 1)) == 0 &&
-        mma_is_faster(cp, size_t(items) * c.n))
+        mma_is_faster(cp, size_t(items) * c.n, beside))
         return launch_conv_mma(c, cp.m, src, src_item, src_plan, dst, dst_item, dst_plan, items, s);
     const size_t n = c.n;
     dim3 grid(unsigned((n + 255) / 256), items, plans.n);  // one coefficient per thread (fewer tail waves)

@@ -296,7 +296,7 @@ int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src,
     const dim3 grid(mma_grid(c, tiles, smem, plans.n), 1, plans.n);
     launch_pdl_split(kSharedPercent, kernel, grid, dim3(kMmaTile), smem, s, plans, src, src_item, src_plan, dst,
                dst_item, dst_plan, uint32_t(c.log_n), tiles, c.d_status);
-    note_launches(1);
+    note_mma_launch();
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 
@@ -329,7 +329,7 @@ int launch_bfv_round_mma(const Context &c, const MmaRef &a, const uint64_t *a_ex
     const uint32_t tiles = uint32_t(items * (c.n / kMmaTile));
     launch_pdl_split(kSharedPercent, k_bfv_round_mma, dim3(mma_grid(c, tiles, smem, 1)), dim3(kMmaTile), smem, s, l, src,
                src_item, dst, dst_item, uint32_t(c.log_n), tiles, c.d_status);
-    note_launches(1);
+    note_mma_launch();
     return cudaGetLastError() == cudaSuccess ? CATFHE_OK : CATFHE_ECUDA;
 }
 

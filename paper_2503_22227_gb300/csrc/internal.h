@@ -278,6 +278,9 @@ void note_launches(uint32_t k);
 // `threads` threads and `smem` dynamic shared bytes), 0 if unknown; cached.
 int resident_slots(const void *kernel, int threads, size_t smem);
 uint64_t launches_total();
+// Number of those that were conversions on the tensor cores.
+void note_mma_launch();
+uint64_t mma_launches_total();
 
 // ----------------------------------------------------------------- launchers
 // NTT (ntt.cu)
@@ -342,9 +345,12 @@ int tune_ntt(Context &c, uint32_t limbs, cudaStream_t s, int *chosen, float *us_
 // grid.z runs plan z over items item = 0..items-1 (grid.y): sources at
 // src + item * src_item + src_off * N, targets at dst + item * dst_item + ...;
 // plan z may add z * src_plan / dst_plan to the item bases.
+// beside: the other half of the operation runs at the same time.
 int launch_conv(const Context &c, const ConvPlans &plans, const uint64_t *src, size_t src_item,
                 size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan, uint32_t items,
-                cudaStream_t s);
+                cudaStream_t s, bool beside = false);
+// Which form launch_conv takes for plans that have an image (mmaplan.cpp).
+bool mma_is_faster(const ConvPlans &cp, size_t coeffs, bool beside);
 // The tensor-core form of launch_conv for plans that have an image.
 int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src, size_t src_item,
                     size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan,

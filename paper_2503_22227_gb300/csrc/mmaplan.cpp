@@ -19,6 +19,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace catfhe {
@@ -156,6 +158,41 @@ std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t tar
         }
     }
     return img;
+}
+
+// Whether the tensor-core form takes less time than the split-weight one, by
+// a model in cycles per warp of 32 coefficients: the integer kernel's multiply
+// pipe (12 a product, 24 a Montgomery reduction, 70% busy; mixed
+// source counts run one coefficient per thread, about a third slower) against
+// the other's issue slots (half busy) and its start (matrix, TMEM) of about
+// 2000.  A launch below two warps per scheduler takes as long as two.
+// Measured on GB300, us (integer / tensor): 8 sources, 20 targets, 3 x 4 x
+// 2^16 coefficients 103 / 59; 5 sources, 23 targets, 2^19 57 / 37; a whole
+// product at N = 2^12, 24 primes (8 and 5 sources) 43.0 / 38.9; at 3 primes (3
+// and 5 sources) 29.1 / 31.6, and at N = 2^16 57.2 / 59.9.
+// The layouts without split weights are slower than both: with 9 special
+// primes (9 sources, 10 when fused) a product of one ciphertext at N = 2^12 takes 35.8 /
+// 32.3 us at 8 limbs and 52.3 / 39.2 at 24, at 2^15 64.5 / 58.8 and 149 / 129 (at 2
+// and 5 limbs of 2^12 the host's time decides, 33-34 either way).
+// beside: the other half of the operation runs at the same time.  To up to four
+// targets little of the integer kernel's time is multiplications, and the
+// tensor-core kernel's shared memory and TMEM keep the other half's CTAs out:
+// products at 8 limbs with 4 special primes (8 sources, 4 targets) 229 / 239 us
+// for 11 ciphertexts at N = 2^15, 260 / 270 for 6 at 2^16, a rotation of 4 169 /
+// 177, so they need six times the gain (4 limbs, 8 special primes, 16
+// ciphertexts at 2^16, 679 / 663, have it; alone, 3 ciphertexts of 8 limbs at
+// 2^16 are 168 / 165).
+bool mma_is_faster(const ConvPlans &cp, size_t coeffs, bool beside) {
+    if (!cp.l.split) return true;
+    double gain = 0, most = 0;
+    for (uint32_t i = 0; i < cp.m.n; i++) {
+        const double K = double(cp.m.head[i] & 0xff), T = double(mma_targets(cp.m.counts[i]));
+        const double pair = (6 * K * (K + 1) + 24 * K + T * (12 * K + 24)) / 0.7;
+        gain += (cp.l.kmin == cp.l.kmax ? 1.0 : 1.3) * pair - (40 * K + 30 * T + 150) / 0.48;
+        most = std::max(most, T);
+    }
+    const double warps = std::max(2.0, double(coeffs) * cp.m.n / 32 / (152 * 4));
+    return gain / cp.m.n * warps > (beside && most <= 4 ? 12000 : 2000);
 }
 
 }  // namespace catfhe

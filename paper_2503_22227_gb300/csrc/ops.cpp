@@ -352,14 +352,15 @@ static int ks_consts(Context &c, int level, bool fused, const KsConsts **out) {
 // Digits of one prime are lifted by the transform's first pass as it loads;
 // wider ones are converted first.
 static int modup_ntt(Context &c, const KsConsts &k, const uint64_t *d2c, size_t d2_item,
-                     uint64_t *ext, uint32_t count, cudaStream_t s) {
+                     uint64_t *ext, uint32_t count, cudaStream_t s, bool beside) {
     const size_t n = c.n;
     if (k.up_lifts) {
         LimbMap m = k.ext;
         m.src_stride = uint32_t(d2_item / n);
         return launch_ntt_lift(c, d2c, ext, m, m.period * count, k.up_lifts, k.lazy, s);
     }
-    TRY(launch_conv(c, k.up, d2c, d2_item, 0, ext, k.ip.ext_item, size_t(k.ip.M) * n, count, s));
+    TRY(launch_conv(c, k.up, d2c, d2_item, 0, ext, k.ip.ext_item, size_t(k.ip.M) * n, count, s,
+                    beside));
     return k.lazy ? launch_ntt_fwd_lazy(c, ext, ext, k.ext, k.ext.period * count, s)
                   : launch_ntt_fwd(c, ext, ext, k.ext, k.ext.period * count, s);
 }
@@ -402,14 +403,14 @@ static int inner_product(Context &c, const KsConsts &k, const uint64_t *ext, con
 // add (BFV): [.][lo][N] added to the first add_polys polynomials, add_item
 // words per ciphertext.  g: sigma_g applied to the result (0: none).
 static int moddown(Context &c, const KsConsts &k, uint64_t *y, uint64_t *lift, uint64_t *out,
-                   uint32_t count, cudaStream_t s, uint64_t g = 0, const Gather *gth = nullptr,
+                   uint32_t count, cudaStream_t s, bool beside, uint64_t g = 0, const Gather *gth = nullptr,
                    const uint64_t *add = nullptr, uint32_t add_polys = 0, size_t add_item = 0) {
     const bool ntt_form = c.scheme != CATFHE_BFV;
     if (gth && gth->n && (!ntt_form || add || gth->n != count)) return CATFHE_EINVAL;
     if (ntt_form) TRY(launch_ntt_inv(c, y, y, k.special, k.special.period * count, s));
     if (!k.down_lifts)
         TRY(launch_conv(c, k.down, y, size_t(k.ip.M) * c.n, 0, lift, k.comb.lift_poly, 0, 2 * count,
-                        s));
+                        s, beside));
     if (ntt_form) {
         // NTT of the lift whose last pass writes (y - lift) D^-1 straight to out
         NttEpilogue e = k.epi;
@@ -599,14 +600,14 @@ static bool forms_products(const Context &c, const IpArgs &ip, uint32_t level, u
 // P*(d0, d1) folded in, ModDown (fused: by P q_{l-1}).
 static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
                          uint64_t *out, uint32_t count, int level, bool fused, KsBufs &k,
-                         cudaStream_t s, const Gather *gth, bool beside) {
+                         cudaStream_t s, const Gather *gth, bool other_half) {
     const uint64_t *rlk;
     TRY(key_for(keys, 0, &rlk));
     const KsConsts *ks;
     TRY(ks_consts(c, level, fused, &ks));
     const size_t n = c.n, half = size_t(level) * n, item = 2 * half;
     const bool gathered = gth && gth->n;
-    if (forms_products(c, ks->ip, uint32_t(level), count, beside)) {
+    if (forms_products(c, ks->ip, uint32_t(level), count, other_half || LaneScope::active())) {
         // no tensor kernel: the inverse transform forms a1 b1 as it loads, and
         // the inner product the three products of its own tile
         LimbMap m = map_second(level);
@@ -620,7 +621,7 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
             }
         }
         TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(level) * count, s, &f));
-        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s, other_half));
         IpArgs ip = ip_args(*ks, k.ext, a + half, rlk, a, nullptr, item, k.y);
         ip.product = 1;
         ip.b = b;
@@ -632,7 +633,7 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
             }
         }
         TRY(launch_ip(c, ip, count, s));
-        return moddown(c, *ks, k.y, k.lift, out, count, s, 0, gth);
+        return moddown(c, *ks, k.y, k.lift, out, count, s, other_half, 0, gth);
     }
     TensorArgs t{};
     t.a = a;
@@ -654,9 +655,9 @@ static int mul_relin_ntt(Context &c, const Keys &keys, const uint64_t *a, const 
     TRY(launch_tensor(c, t, count, s));
     LimbMap m = map_identity(uint32_t(level));
     TRY(launch_ntt_inv(c, k.d2, k.d2c, m, uint32_t(level) * count, s));
-    TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+    TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s, other_half));
     TRY(inner_product(c, *ks, k.ext, k.d2, rlk, k.d0, k.d1, half, k.y, count, s));
-    return moddown(c, *ks, k.y, k.lift, out, count, s, 0, gth);
+    return moddown(c, *ks, k.y, k.lift, out, count, s, other_half, 0, gth);
 }
 
 // A BFV multiplication's constants at one level, kept like KsConsts.
@@ -742,7 +743,8 @@ static int build_bfv(Context &c, int level, BfvConsts &k) {
 // BFV: lift to Q u B, NTT, tensor, INTT, exact round(t x / Q) back to Q,
 // then relinearise d2 in coefficient form.
 static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
-                         uint64_t *out, uint32_t count, int level, KsBufs &k, cudaStream_t s) {
+                         uint64_t *out, uint32_t count, int level, KsBufs &k, cudaStream_t s,
+                         bool other_half) {
     const uint64_t *rlk;
     TRY(key_for(keys, 0, &rlk));
     const KsConsts *ks;
@@ -757,7 +759,8 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
     for (int h = 0; h < 2; h++) {  // items: (ct, poly) of a, then of b
         const uint64_t *src = h ? b : a;
         uint64_t *dst = h ? xb : k.xin;
-        TRY(launch_conv(c, bc->lift, src, size_t(level) * n, 0, dst, size_t(kb) * n, 0, 2 * count, s));
+        TRY(launch_conv(c, bc->lift, src, size_t(level) * n, 0, dst, size_t(kb) * n, 0, 2 * count, s,
+                        other_half));
         TRY(launch_ntt_fwd(c, src, dst, bc->in, uint32_t(level) * 2 * count, s));
     }
     TRY(launch_ntt_fwd(c, k.xin, k.xin, bc->mb, uint32_t(c.nb) * 4 * count, s));
@@ -785,7 +788,7 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
                                    size_t(kb) * n, k.dq, size_t(level) * n, 3 * count, s));
     // 4. relinearise d2' (coefficient form) and add (d0', d1')
     const uint64_t *d2 = k.dq + size_t(2) * level * n;
-    TRY(modup_ntt(c, *ks, d2, size_t(3) * level * n, k.ext, count, s));
+    TRY(modup_ntt(c, *ks, d2, size_t(3) * level * n, k.ext, count, s, other_half));
     TRY(inner_product(c, *ks, k.ext, nullptr, rlk, nullptr, nullptr, 0, k.y, count, s));
     {
         const int M = level + c.K;
@@ -794,7 +797,8 @@ static int mul_relin_bfv(Context &c, const Keys &keys, const uint64_t *a, const 
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
     // (d0', d1') are the first two of each ciphertext's three polynomials
-    return moddown(c, *ks, k.y, k.lift, out, count, s, 0, nullptr, k.dq, 2, size_t(3) * level * n);
+    return moddown(c, *ks, k.y, k.lift, out, count, s, other_half, 0, nullptr, k.dq, 2,
+                   size_t(3) * level * n);
 }
 
 // Two streams (and fork / join events) per device for split operations;
@@ -869,9 +873,8 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
         const size_t n = c.n, lo = size_t(fused ? lvl - 1 : lvl);
         const uint64_t *ah = a + size_t(first) * 2 * lvl * n, *bh = b + size_t(first) * 2 * lvl * n;
         uint64_t *oh = out + size_t(first) * 2 * lo * n;
-        if (c.scheme == CATFHE_BFV) return mul_relin_bfv(c, keys, ah, bh, oh, cnt, lvl, k, st);
-        return mul_relin_ntt(c, keys, ah, bh, oh, cnt, lvl, fused, k, st, gth,
-                             halves || LaneScope::active());
+        if (c.scheme == CATFHE_BFV) return mul_relin_bfv(c, keys, ah, bh, oh, cnt, lvl, k, st, halves);
+        return mul_relin_ntt(c, keys, ah, bh, oh, cnt, lvl, fused, k, st, gth, halves);
     };
     if (halves) return run_halves(c, count, lvl, fused, base, s, run);
     return run(0, count, base, s);
@@ -884,7 +887,8 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
 // sigma_g(a0 + KS_gk'(a1)) with gk' = sigma_g^-1(gk), the stored form of the
 // key, bit for bit; only the kernel that writes the result permutes.
 static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_t g, uint64_t *out,
-                      int lvl, uint32_t count, KsBufs &k, cudaStream_t s, const Gather *gth) {
+                      int lvl, uint32_t count, KsBufs &k, cudaStream_t s, const Gather *gth,
+                      bool other_half) {
     const size_t n = c.n, item = size_t(2) * lvl * n, half = size_t(lvl) * n;
     const KsConsts *ks;
     TRY(ks_consts(c, lvl, false, &ks));
@@ -895,9 +899,9 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
             for (uint32_t i = 0; i < gth->n; i++) m.gsrc[i] = gth->a[i];
         }
         TRY(launch_ntt_inv(c, a, k.d2c, m, uint32_t(lvl) * count, s));
-        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s));
+        TRY(modup_ntt(c, *ks, k.d2c, half, k.ext, count, s, other_half));
         TRY(inner_product(c, *ks, k.ext, a + half, gk, a, nullptr, item, k.y, count, s, gth));
-        return moddown(c, *ks, k.y, k.lift, out, count, s, g, gth);
+        return moddown(c, *ks, k.y, k.lift, out, count, s, other_half, g, gth);
     }
     // BFV (coefficient form): a1 is key switched, a0 added by the combine.  It
     // scatters its results, so a0 is copied first when out overlaps a.
@@ -909,7 +913,7 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
                               uint32_t(2 * lvl) * count, s));
         add = k.add;
     }
-    TRY(modup_ntt(c, *ks, a + half, item, k.ext, count, s));
+    TRY(modup_ntt(c, *ks, a + half, item, k.ext, count, s, other_half));
     TRY(inner_product(c, *ks, k.ext, nullptr, gk, nullptr, nullptr, 0, k.y, count, s));
     {
         const int M = lvl + c.K;
@@ -917,7 +921,7 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
         for (int i = 0; i < M; i++) my.prime[i] = uint8_t(ext_prime(c, lvl, i));
         TRY(launch_ntt_inv(c, k.y, k.y, my, uint32_t(2 * M) * count, s));
     }
-    return moddown(c, *ks, k.y, k.lift, out, count, s, g, nullptr, add, 1, item);
+    return moddown(c, *ks, k.y, k.lift, out, count, s, other_half, g, nullptr, add, 1, item);
 }
 
 int op_rotate(Context &c, const Keys &keys, const uint64_t *a, uint64_t g, uint64_t *out,
@@ -935,16 +939,16 @@ int op_rotate(Context &c, const Keys &keys, const uint64_t *a, uint64_t g, uint6
     TRY(get_ws(c, ws, ws_bytes_in, ws_bytes(c, CATFHE_OP_ROTATE, level, count), &base));
     const size_t n = c.n;
     const int lvl = int(level);
+    const bool halves = split && !(gth && gth->n) && split_ok(c, count);
     auto run = [&](uint32_t first, uint32_t cnt, char *wbase, cudaStream_t st) -> int {
         Bump bump{wbase};
         KsBufs k{};
         ks_layout(c, bump, k, cnt, lvl, false);
         const uint64_t *ah = a + size_t(first) * 2 * lvl * n;
         uint64_t *oh = out + size_t(first) * 2 * lvl * n;
-        return rotate_run(c, gk, ah, g, oh, lvl, cnt, k, st, gth);
+        return rotate_run(c, gk, ah, g, oh, lvl, cnt, k, st, gth, halves);
     };
-    if (split && !(gth && gth->n) && split_ok(c, count))
-        return run_halves(c, count, lvl, false, base, s, run);
+    if (halves) return run_halves(c, count, lvl, false, base, s, run);
     return run(0, count, base, s);
 }
 
@@ -982,9 +986,10 @@ int op_rotate_hoisted(Context &c, const Keys &keys, const uint64_t *a, const uin
     TRY(launch_ntt_inv(c, a, k.d2c, map_second(lvl), uint32_t(lvl) * count, s));
     const KsConsts *kc;
     TRY(ks_consts(c, lvl, false, &kc));
-    TRY(modup_ntt(c, *kc, k.d2c, half, ext0, count, s));
+    TRY(modup_ntt(c, *kc, k.d2c, half, ext0, count, s, false));
     auto down = [&](uint32_t r, KsBufs &kb, uint64_t *y, cudaStream_t st) {
-        return moddown(c, *kc, y, kb.lift, out + size_t(r) * count * item, count, st, gv[r]);
+        return moddown(c, *kc, y, kb.lift, out + size_t(r) * count * item, count, st, false,
+                       gv[r]);
     };
     auto one = [&](uint32_t r, KsBufs &kb, cudaStream_t st) -> int {
         TRY(inner_product(c, *kc, ext0, a + half, gk[r], a, nullptr, item, kb.y, count, st));

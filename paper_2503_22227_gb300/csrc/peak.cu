@@ -21,6 +21,12 @@ namespace catfhe {
 static std::atomic<uint64_t> g_launches{0};
 void note_launches(uint32_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 uint64_t launches_total() { return g_launches.load(std::memory_order_relaxed); }
+static std::atomic<uint64_t> g_mma_launches{0};
+void note_mma_launch() {
+    note_launches(1);
+    g_mma_launches.fetch_add(1, std::memory_order_relaxed);
+}
+uint64_t mma_launches_total() { return g_mma_launches.load(std::memory_order_relaxed); }
 
 constexpr int kChains = 8;
 
