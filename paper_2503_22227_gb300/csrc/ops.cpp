@@ -580,19 +580,20 @@ static LimbMap map_second(int lvl) {
 // Up to kProductFew ciphertexts with nothing beside them keep the route to
 // kProductWords words, where the kernels wait for their loads more than for
 // multiplications: 2^14, 16 limbs x 2 75.3 -> 73.7, 24 limbs 74.0 -> 72.5, BGV 8
-// limbs x 3 84.7 -> 83.5, 2^15, 16 limbs 79.4 -> 77.9, 2^16, 8 limbs 81.9 -> 79.2
-// (and 2^14, 9 limbs x 2 55.1 -> 56.0; one ciphertext at 2^16, 24 limbs is level,
-// 198.0).  With fewer limbs than special primes most of the inner product's
-// CTAs have no product to form and wait for those that do: 2^16, 3 limbs 54.9 ->
-// 56.0, 2^15, 2 limbs x 2 48.8 -> 50.2, so these stay with the tensor kernel.
+// limbs x 3 84.7 -> 83.5, 2^15, 16 limbs 79.4 -> 77.9, 2^16, 4 limbs 60.4 -> 58.8,
+// 8 limbs 81.9 -> 79.2, with 8 special primes 7 limbs 91.2 -> 89.2 (and 2^14, 9
+// limbs x 2 55.1 -> 56.0; one ciphertext at 2^16, 24 limbs is level, 198.0).  Below
+// kProductLimbs limbs few of the inner product's CTAs have a product to form and
+// the others wait for them: 2^16, 3 limbs 54.9 -> 56.0, 2^15, 2 limbs x 2 48.8 ->
+// 50.2, so these stay with the tensor kernel.
 // A batch on lanes: 8 operations 271.3 with it, 273.8 without, 16 463 and 472.
 constexpr size_t kProductWork = size_t(1) << 20, kProductWords = size_t(1) << 19;
-constexpr uint32_t kProductFew = 3;
+constexpr uint32_t kProductFew = 3, kProductLimbs = 4;
 static bool forms_products(const Context &c, const IpArgs &ip, uint32_t level, uint32_t count,
                            bool beside) {
     if (ip.beta > kIpBulkBeta) return false;
     if (size_t(count) * (ip.beta + 2) * ip.M * c.n <= kProductWork) return true;
-    return !beside && count <= kProductFew && int(level) > c.K &&
+    return !beside && count <= kProductFew && level >= kProductLimbs &&
            size_t(count) * level * c.n <= kProductWords;
 }
 

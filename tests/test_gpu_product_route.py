@@ -29,13 +29,13 @@ def _uniform(ctx, seed, count, level, first=0):
 
 # (N, limbs, ciphertexts, tensor kernel): 24 primes in digits of 8, 4 special
 # primes; the line is 2^20 words of (digits + 2) (limbs + 4) N per ciphertext,
-# or 3 ciphertexts of more than 4 limbs
+# or up to 2^19 words of at most 3 ciphertexts of at least 4 limbs
 @pytest.mark.parametrize("log_n,level,count,tensor", [
     (12, 2, 8, False), (12, 2, 16, True), (12, 8, 7, False), (12, 8, 16, True), (12, 24, 3, False),
     (12, 24, 5, True), (13, 3, 4, False), (13, 5, 8, True), (13, 9, 5, True), (14, 3, 3, False),
     (14, 3, 4, False), (14, 2, 16, True), (14, 9, 5, True), (14, 16, 2, False), (14, 16, 4, True),
     (15, 2, 1, False), (15, 2, 2, True), (15, 2, 4, True), (15, 16, 1, False), (15, 17, 1, True),
-    (16, 3, 1, True), (16, 8, 1, False), (16, 9, 1, True), (16, 2, 8, True)])
+    (16, 3, 1, True), (16, 4, 1, False), (16, 8, 1, False), (16, 9, 1, True), (16, 2, 8, True)])
 def test_route_and_results(log_n, level, count, tensor):
     p = W.Preset("route", W.CKKS, log_n, (50,) * 24, (60,) * 4, 3, log_n_max=16)
     ctx = api.Context(p)
@@ -57,14 +57,14 @@ def test_route_and_results(log_n, level, count, tensor):
 
 @pytest.mark.parametrize("log_n", [12, 13, 14, 15, 16])
 def test_both_routes_match_the_oracle_under_every_schedule(log_n):
-    p = W.Preset("route-sched", W.CKKS, log_n, (50, 58, 61), (61,), 3, log_n_max=16)
+    p = W.Preset("route-sched", W.CKKS, log_n, (50, 58, 61, 45), (61,), 4, log_n_max=16)
     ctx = api.Context(p)
     octx = oracle.Context(p.scheme, log_n, p.q_bits, p.p_bits, p.dnum, log_n_max=16)
     seed = W.seed_for(f"route-sched-{log_n}")
     keys, okeys = ctx.keygen(seed), octx.keygen(seed)
     parts = 2 if log_n >= 14 else 1
-    many = parts * max(4, (1 << 20) // (5 * 4 << log_n) + 1)  # past the line in each part
-    a, b = _uniform(ctx, seed, many, 3), _uniform(ctx, seed, many, 3, 1000)
+    many = parts * max(4, (1 << 20) // (6 * 5 << log_n) + 1)  # past the line in each part
+    a, b = _uniform(ctx, seed, many, 4), _uniform(ctx, seed, many, 4, 1000)
     want = octx.mul_relin(okeys, ctx.export_ct(a[:1])[0], ctx.export_ct(b[:1])[0])
     scaled = octx.rescale(want)
     _, count, _ = ctx.ntt_schedule()
