@@ -702,7 +702,7 @@ int launch_conv(const Context &c, const ConvPlans &cp, const uint64_t *src, size
     if (plans.n == 0 || items == 0) return CATFHE_OK;
     // (its bulk copies need 16-byte aligned sources, as every buffer's are)
     if (cp.mma && ((reinterpret_cast<uintptr_t>(src) & 15) | ((src_item | src_plan) & 1)) == 0 &&
-        mma_is_faster(cp, size_t(items) * c.n, beside))
+        mma_is_faster(cp, size_t(items) * c.n, c.sms, beside))
         return launch_conv_mma(c, cp.m, src, src_item, src_plan, dst, dst_item, dst_plan, items, s);
     const size_t n = c.n;
     dim3 grid(unsigned((n + 255) / 256), items, plans.n);  // one coefficient per thread (fewer tail waves)

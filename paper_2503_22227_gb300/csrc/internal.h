@@ -350,7 +350,7 @@ int launch_conv(const Context &c, const ConvPlans &plans, const uint64_t *src, s
                 size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan, uint32_t items,
                 cudaStream_t s, bool beside = false);
 // Which form launch_conv takes for plans that have an image (mmaplan.cpp).
-bool mma_is_faster(const ConvPlans &cp, size_t coeffs, bool beside);
+bool mma_is_faster(const ConvPlans &cp, size_t coeffs, int sms, bool beside);
 // The tensor-core form of launch_conv for plans that have an image.
 int launch_conv_mma(const Context &c, const MmaList &plans, const uint64_t *src, size_t src_item,
                     size_t src_plan, uint64_t *dst, size_t dst_item, size_t dst_plan,

@@ -165,7 +165,7 @@ std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t tar
 // pipe (12 a product, 24 a Montgomery reduction, 70% busy; mixed
 // source counts run one coefficient per thread, about a third slower) against
 // the other's issue slots (half busy) and its start (matrix, TMEM) of about
-// 2000.  A launch below two warps per scheduler takes as long as two.
+// 2000.  A launch below two warps per scheduler (four per SM) takes as long as two.
 // Measured on GB300, us (integer / tensor): 8 sources, 20 targets, 3 x 4 x
 // 2^16 coefficients 103 / 59; 5 sources, 23 targets, 2^19 57 / 37; a whole
 // product at N = 2^12, 24 primes (8 and 5 sources) 43.0 / 38.9; at 3 primes (3
@@ -182,7 +182,7 @@ std::vector<uint64_t> build_mma_plan(const PlanSpec &s, uint64_t n, uint64_t tar
 // 177, so they need six times the gain (4 limbs, 8 special primes, 16
 // ciphertexts at 2^16, 679 / 663, have it; alone, 3 ciphertexts of 8 limbs at
 // 2^16 are 168 / 165).
-bool mma_is_faster(const ConvPlans &cp, size_t coeffs, bool beside) {
+bool mma_is_faster(const ConvPlans &cp, size_t coeffs, int sms, bool beside) {
     if (!cp.l.split) return true;
     double gain = 0, most = 0;
     for (uint32_t i = 0; i < cp.m.n; i++) {
@@ -191,7 +191,7 @@ bool mma_is_faster(const ConvPlans &cp, size_t coeffs, bool beside) {
         gain += (cp.l.kmin == cp.l.kmax ? 1.0 : 1.3) * pair - (40 * K + 30 * T + 150) / 0.48;
         most = std::max(most, T);
     }
-    const double warps = std::max(2.0, double(coeffs) * cp.m.n / 32 / (152 * 4));
+    const double warps = std::max(2.0, double(coeffs) * cp.m.n / 32 / (4.0 * sms));
     return gain / cp.m.n * warps > (beside && most <= 4 ? 12000 : 2000);
 }
 

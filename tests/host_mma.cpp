@@ -10,7 +10,7 @@ using namespace catfhe;
 
 // `plans` conversions of K[i] sources and T[i] targets, split weights or not.
 extern "C" int mma_rule(int plans, const int *K, const int *T, int split, uint64_t coeffs,
-                        int beside) {
+                        int sms, int beside) {
     ConvPlans cp{};
     cp.mma = true;
     cp.l.n = cp.m.n = uint32_t(plans);
@@ -24,5 +24,5 @@ extern "C" int mma_rule(int plans, const int *K, const int *T, int split, uint64
         cp.l.kmin = K[i] < int(cp.l.kmin) ? uint32_t(K[i]) : cp.l.kmin;
         cp.l.kmax = K[i] > int(cp.l.kmax) ? uint32_t(K[i]) : cp.l.kmax;
     }
-    return mma_is_faster(cp, coeffs, beside != 0);
+    return mma_is_faster(cp, coeffs, sms, beside != 0);
 }

@@ -25,10 +25,11 @@ def lib(tmp_path_factory):
     return ctypes.CDLL(out)
 
 
-def _rule(lib, shapes, items, log_n, beside, split=1):
+def _rule(lib, shapes, items, log_n, beside, split=1, sms=152):
     n = len(shapes)
     K, T = ((ctypes.c_int * n)(*(s[i] for s in shapes)) for i in (0, 1))
-    return bool(lib.mma_rule(n, K, T, split, ctypes.c_uint64(items << log_n), int(beside)))
+    return bool(lib.mma_rule(n, K, T, split, ctypes.c_uint64(items << log_n), sms,
+                             int(beside)))
 
 
 @pytest.mark.parametrize("shapes,items,log_n,beside,tensor", [
@@ -51,3 +52,13 @@ def test_form_of_a_conversion(lib, shapes, items, log_n, beside, tensor):
 def test_other_layouts_take_the_tensor_cores(lib):
     for beside in (False, True):
         assert _rule(lib, [(9, 2)], 1, 12, beside, split=0)
+
+
+def test_form_follows_the_devices_size(lib):
+    """The same launch spreads its start over fewer coefficients per SM on a
+    larger device."""
+    assert _rule(lib, [(8, 4)], 2, 16, False)
+    assert not _rule(lib, [(8, 4)], 2, 16, False, sms=304)
+    assert _rule(lib, [(8, 4)], 4, 16, False, sms=304)
+    assert _rule(lib, [(8, 4)], 1, 16, False, sms=76)
+    assert not _rule(lib, [(8, 4)], 1, 16, False)
