@@ -1,5 +1,7 @@
 // The host side of the tensor-core base conversion (mmaplan.cpp) for
 // test_host_mma.py: the rule that chooses the form.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace catfhe {
@@ -16,13 +18,13 @@ extern "C" int mma_rule(int plans, const int *K, const int *T, int split, uint64
     cp.l.n = cp.m.n = uint32_t(plans);
     cp.l.mont = 1;
     cp.l.split = uint32_t(split);
-    cp.l.kmin = ~0u;
+    cp.l.kmin = cp.l.kmax = uint32_t(K[0]);
     for (int i = 0; i < plans; i++) {
         cp.m.head[i] = uint64_t(K[i]);
         for (int t = 0; t < T[i]; t += 3)
             cp.m.counts[i] |= uint64_t(T[i] - t < 3 ? T[i] - t : 3) << (4 * (t / 3));
-        cp.l.kmin = K[i] < int(cp.l.kmin) ? uint32_t(K[i]) : cp.l.kmin;
-        cp.l.kmax = K[i] > int(cp.l.kmax) ? uint32_t(K[i]) : cp.l.kmax;
+        cp.l.kmin = std::min(cp.l.kmin, uint32_t(K[i]));
+        cp.l.kmax = std::max(cp.l.kmax, uint32_t(K[i]));
     }
     return mma_is_faster(cp, coeffs, sms, beside != 0);
 }
