@@ -383,7 +383,10 @@ MmaRef get_mma_plan(Context &c, const std::string &key, const PlanSpec &spec,
     const std::vector<uint64_t> img = build_mma_plan(spec, c.n, target_unit);
     if (!img.empty()) {
         uint64_t *dev = nullptr;
-        if (cudaMalloc(&dev, img.size() * 8) != cudaSuccess) return ref;
+        if (cudaMalloc(&dev, img.size() * 8) != cudaSuccess) {
+            cudaGetLastError();  // the integer form's launches read it otherwise
+            return ref;
+        }
         if (copy_in(dev, img.data(), img.size() * 8) != cudaSuccess) {
             cudaFree(dev);
             return ref;

@@ -4,10 +4,14 @@
 //
 // A copy from pageable memory only stages its bytes; they arrive when its
 // stream, the legacy one, is waited for.  Work on another stream in between
-// finds the buffer's old contents.
+// finds the buffer's old contents.  A failed allocation stays the thread's last
+// error until somebody reads it, and every launch reads it.
 //
 //   host_uploads("encrypt", scheme)  the number of constants that kernels of an
 //                                    encryption were given before they arrived
+//   host_uploads("nomem", scheme)    the last error after a conversion's plans
+//                                    were made without memory for its
+//                                    tensor-core image
 #include <stdlib.h>
 #include <string.h>
 
@@ -20,6 +24,8 @@ struct Staged {
 };
 std::vector<Staged> staged;
 int late = 0;
+bool no_memory = false;
+cudaError_t last = cudaSuccess;
 
 void arrive() {
     for (auto &c : staged) memcpy(c.dst, c.bytes.data(), c.bytes.size());
@@ -37,6 +43,7 @@ extern "C" {
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
 cudaError_t cudaMalloc(void **p, size_t n) {
+    if (no_memory) return last = cudaErrorMemoryAllocation;
     *p = calloc(1, n);
     return cudaSuccess;
 }
@@ -62,6 +69,11 @@ cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
     if (s == nullptr || s == cudaStreamLegacy) arrive();
     return cudaSuccess;
+}
+cudaError_t cudaGetLastError() {
+    const cudaError_t e = last;
+    last = cudaSuccess;
+    return e;
 }
 }
 
@@ -123,5 +135,16 @@ extern "C" int host_uploads(const char *what, int scheme) {
         if (op_encrypt(c, k, msg.data(), seed, ct.data(), own)) return -1;
         return late;
     }
-    return -1;
+    PlanSpec s;
+    for (uint32_t i = 0; i < 3; i++) {
+        s.src_mod.push_back(c.mod(int(i)));
+        s.src_off.push_back(i);
+    }
+    s.dst_mod.push_back(c.mod(3));
+    s.dst_off.push_back(0);
+    no_memory = true;
+    const MmaRef image = get_mma_plan(c, "x", s, c.n);
+    no_memory = false;
+    if (image.p || !get_plan(c, "x", s).p) return -1;  // the integer form's plan
+    return int(cudaGetLastError());
 }

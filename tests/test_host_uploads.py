@@ -1,6 +1,7 @@
 """What the library's host code hands to kernels, on a fake CUDA runtime
 (tests/host_uploads.cpp): constants have arrived before a kernel on the
-caller's stream may read them."""
+caller's stream may read them, and an allocation that failed and is made up
+for leaves no error for the next launch to report."""
 import os
 import shutil
 import subprocess
@@ -57,3 +58,7 @@ def _run(program, what, scheme):
 @pytest.mark.parametrize("scheme", [W.CKKS, W.BFV, W.BGV])
 def test_constants_arrive_before_the_kernels_that_read_them(program, scheme):
     assert _run(program, "encrypt", scheme) == 0
+
+
+def test_no_memory_for_an_image_leaves_the_integer_form_usable(program):
+    assert _run(program, "nomem", W.CKKS) == 0
