@@ -1,5 +1,5 @@
 // The host side of the tensor-core base conversion (mmaplan.cpp) for
-// test_host_mma.py: the rule that chooses the form.
+// test_host_mma.py: the rule that chooses the form, and the image of a plan.
 #include <algorithm>
 
 #include "internal.h"
@@ -27,4 +27,25 @@ extern "C" int mma_rule(int plans, const int *K, const int *T, int split, uint64
         cp.l.kmax = std::max(cp.l.kmax, uint32_t(K[i]));
     }
     return mma_is_faster(cp, coeffs, sms, beside != 0);
+}
+
+// The image for sources src (factors pre), targets dst (factors post): its
+// words, -1 if there is none.
+extern "C" int mma_plan(int K, const uint64_t *src, const uint64_t *pre, int T, const uint64_t *dst,
+                        const uint64_t *post, uint64_t *img, int cap) {
+    PlanSpec s;
+    for (int i = 0; i < K; i++) {
+        s.src_mod.push_back(src[i]);
+        s.src_off.push_back(uint32_t(i));
+        s.pre.push_back(pre[i]);
+    }
+    for (int t = 0; t < T; t++) {
+        s.dst_mod.push_back(dst[t]);
+        s.dst_off.push_back(uint32_t(t));
+        s.post.push_back(post[t]);
+    }
+    const std::vector<uint64_t> v = build_mma_plan(s, 1, 1);
+    if (v.empty() || int(v.size()) > cap) return -1;
+    std::copy(v.begin(), v.end(), img);
+    return int(v.size());
 }
