@@ -316,8 +316,8 @@ int catfhe_rotate(catfhe_ctx *ctx, const catfhe_keys *keys, const uint64_t *a,
  * "rotate_vector_random" over many steps; hoisting): the exact lift of each
  * digit of a1 commutes with sigma_g (a signed permutation of coefficients;
  * the centred lift is odd), so ModUp(sigma_g(a1)) = sigma_g(ModUp(a1)) and
- * each rotation only permutes the lifted digits, then runs the inner product
- * and ModDown.  out[r] = catfhe_rotate(a, galois_elts[r]) bit for bit, for
+ * each rotation only runs the inner product with its key (kept permuted by
+ * sigma_g^-1) and ModDown, which permutes the result as it writes it.  out[r] = catfhe_rotate(a, galois_elts[r]) bit for bit, for
  * r < n_rot; out is u64[n_rot][count][2][level][N].  CKKS and BGV (ESCHEME
  * for BFV); every key is checked (ENOKEY) before anything is enqueued.
  * Workspace: catfhe_workspace_bytes(CATFHE_OP_ROTATE_HOISTED, level, count),

@@ -221,8 +221,8 @@ void make_units(const catfhe_op *ops, uint32_t n, uint32_t lanes, std::vector<Un
 // fewer the chip is not filled.  Measured on one degree at a time (us for 64
 // operations of any level, 8 lanes asked; all of them in submission order ->
 // here): N = 2^16 5008 -> 4156 (3 lanes), 2^15 2322 -> 2187, 2^14 1181 -> 1126,
-// 2^13 654 -> 578 (8 lanes); 256 of all four degrees 9240 -> 8530; eight
-// encrypted queries 72 -> 68 ms.  300 and 400 MB differ by 3% or less; at 500 MB
+// 2^13 654 -> 578 (8 lanes); 256 of all four degrees 9240 -> 8530 (the
+// graph alone; 8590 to 8660 a public launch); eight encrypted queries 72 -> 68 ms.  300 and 400 MB differ by 3% or less; at 500 MB
 // the first is 4215.
 constexpr double kLaneBytes = 320e6;
 // Entries per lane from which lanes are left out: below, the longest chain of

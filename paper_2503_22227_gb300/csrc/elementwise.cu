@@ -3,9 +3,10 @@
 // kernel), the key-switching inner product, the ModDown combine, the
 // automorphism X -> X^g, and ChaCha20 sampling for keys and encryption.
 //
-// All are HBM-bound streams over limb-major data: one thread per coefficient,
-// consecutive threads on consecutive words, grids sized by the data (a whole
-// batch of ciphertexts per launch).
+// All are HBM-bound streams over limb-major data: a thread takes one or two
+// 16-byte pairs of coefficients (sampling and the automorphism one coefficient),
+// consecutive threads consecutive words, grids sized by the data (a whole batch
+// of ciphertexts per launch).
 #include <cmath>
 #include "bulk.cuh"
 #include "launch.cuh"

@@ -386,8 +386,9 @@ int launch_bfv_round_mma(const Context &c, const MmaRef &a, const uint64_t *a_ex
 // contiguous: an uneven batch merges compatible single-ciphertext entries
 // into one operation of count = n items; item i reads a[i] (and b[i]) and
 // writes out[i], each u64[2][level][N].  Only the kernels that touch the
-// caller's buffers (the tensor's loads, the automorphism's loads, ModDown's
-// final stores) look at it; everything between runs on contiguous workspace.
+// caller's buffers (the tensor's loads, the inverse transform's, the inner
+// product's, ModDown's final stores) look at it; everything between runs on
+// contiguous workspace.
 struct Gather {
     uint32_t n = 0;
     const uint64_t *a[kGatherMax];

@@ -1,8 +1,10 @@
 // Launches with programmatic dependent launch: the kernel may be scheduled
 // while the previous kernel on the stream finishes its last CTAs, and waits
-// (griddepcontrol.wait, first statement of every kernel launched this way)
-// until that kernel has completed and its memory is visible.  This hides the
-// launch gap between the kernels of an operation.
+// (griddepcontrol.wait) until that kernel has completed and its memory is
+// visible.  Before the wait a kernel touches nothing that a launch writes: the
+// tensor-core conversions allocate TMEM and load their plan, which has been on
+// the device since it was made; in all others the wait is the first statement.
+// This hides the launch gap between the kernels of an operation.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -24,7 +26,8 @@ namespace catfhe {
 //   percent 9440 and 19.0, at 86 percent 9460 and 20.1).
 // - Otherwise the conversions and the tensor product ask for it, which run
 //   beside the other half's transforms: 5 products at N = 2^15 204 -> 196.5
-//   us, 16 BFV products 724 -> 717, 8 at N = 2^16 1105 -> 1101.  The inner
+//   us on the device (200 a public call), 16 BFV products 724 -> 717, 8 at N =
+//   2^16 1105 -> 1101.  The inner
 //   product does not (16 BGV products 315 -> 325 us), nor do the transforms'
 //   row passes (one product at N = 2^16 198 -> 200).
 constexpr unsigned kSharedPercent = 72;

@@ -11,7 +11,8 @@
 // digits, one column each; the kernel multiplies byte - 128 (exact in fp16,
 // as the digits are) and accumulates in fp32.  A column's sums stay below
 // 2^22 in magnitude, checked here against its actual weights, so they are
-// exact integers; a constant row adds 3 * 2^22, which puts the sum's bits in
+// exact integers (relied on: products of fp16 whole numbers are exact and the
+// tensor core adds whole numbers below 2^24 exactly, in any order); a constant row adds 3 * 2^22, which puts the sum's bits in
 // the float's low mantissa.  S_d the sums of a target's columns, the result is
 //     r = sum_d S_d 2^(10 d) + C0 - (e - 1) p,  C0 = 128 sum of all weights,
 // e the rounded quotient, from the top three columns in fp32: r is in

@@ -371,7 +371,7 @@ k_ntt_fwd_rows(uint64_t *__restrict__ data, const LimbMap map, const DevMod *__r
             }
             return;
         }
-        // ModDown combine: out = (y - lift) * D^-1 (+ add), lift now in NTT form
+        // ModDown combine: out = (y - lift) * D^-1, lift now in NTT form
         uint64_t *op = (epi.gathered ? epi.gout[g] : epi.out + size_t(g) * epi.out_stride * N) +
                        size_t(epi.out_off[r]) * N;
         const uint64_t dv = epi.dinv[r], dvs = epi.dinv_s[r];
