@@ -38,6 +38,11 @@ struct Bump {
     }
 };
 
+static bool overlap(const void *a, size_t a_bytes, const void *b, size_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + b_bytes && y < x + a_bytes;
+}
+
 static int get_ws(Context &c, void *ws, size_t ws_bytes, size_t need, char **out) {
     if (ws) {
         // kernels access the workspace in 8- and 16-byte words (and bulk
@@ -866,7 +871,14 @@ int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t
     char *base;
     TRY(get_ws(c, ws, ws_bytes_in, need, &base));
     const int lvl = int(level);
-    const bool halves = split && !(gth && gth->n) && split_ok(c, count);
+    // Fused results are a limb shorter than the inputs: written over an input,
+    // the second half's lie in the first half's inputs, which that one may still
+    // read, so the halves run as one.
+    const size_t in_bytes = size_t(count) * 2 * lvl * c.n * 8;
+    const size_t out_bytes = size_t(count) * 2 * (lvl - 1) * c.n * 8;
+    const bool over = fused && (overlap(a, in_bytes, out, out_bytes) ||
+                                overlap(b, in_bytes, out, out_bytes));
+    const bool halves = split && !over && !(gth && gth->n) && split_ok(c, count);
     auto run = [&](uint32_t first, uint32_t cnt, char *wbase, cudaStream_t st) -> int {
         Bump bump{wbase};
         KsBufs k{};
@@ -907,9 +919,8 @@ static int rotate_run(Context &c, const uint64_t *gk, const uint64_t *a, uint64_
     // BFV (coefficient form): a1 is key switched, a0 added by the combine.  It
     // scatters its results, so a0 is copied first when out overlaps a.
     const uint64_t *add = a;
-    const uintptr_t a0 = reinterpret_cast<uintptr_t>(a), o0 = reinterpret_cast<uintptr_t>(out);
     const size_t bytes = size_t(count) * item * 8;
-    if (a0 < o0 + bytes && o0 < a0 + bytes) {
+    if (overlap(a, bytes, out, bytes)) {
         TRY(launch_copy_limbs(c, a, k.add, map_identity(uint32_t(2 * lvl)),
                               uint32_t(2 * lvl) * count, s));
         add = k.add;

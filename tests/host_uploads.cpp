@@ -12,8 +12,13 @@
 //   host_uploads("nomem", scheme)    the last error after a conversion's plans
 //                                    were made without memory for its
 //                                    tensor-core image
+//   host_uploads("over", scheme)     the number of streams on which a fused
+//                                    product of four is written over its input
+//                                    (1 in its own buffer: 2)
 #include <stdlib.h>
 #include <string.h>
+
+#include <set>
 
 #include "internal.h"
 
@@ -26,6 +31,7 @@ std::vector<Staged> staged;
 int late = 0;
 bool no_memory = false;
 cudaError_t last = cudaSuccess;
+std::set<cudaStream_t> used;
 
 void arrive() {
     for (auto &c : staged) memcpy(c.dst, c.bytes.data(), c.bytes.size());
@@ -70,6 +76,14 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) {
     if (s == nullptr || s == cudaStreamLegacy) arrive();
     return cudaSuccess;
 }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+    static uintptr_t next = 32;
+    *s = reinterpret_cast<cudaStream_t>(next += 16);
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *, unsigned) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaGetLastError() {
     const cudaError_t e = last;
     last = cudaSuccess;
@@ -81,7 +95,39 @@ namespace catfhe {
 int ctx_init(Context &c, const catfhe_params &p);
 int op_encrypt(Context &c, const Keys &k, const int64_t *msg, const uint8_t seed[32], uint64_t *ct,
                cudaStream_t s);
+int op_mul_relin(Context &c, const Keys &keys, const uint64_t *a, const uint64_t *b,
+                 uint64_t *out, uint32_t level, uint32_t count, bool fused, void *ws,
+                 size_t ws_bytes_in, cudaStream_t s, const Gather *gth, bool split);
+size_t ws_bytes(const Context &c, int op, uint32_t level, uint32_t count);
 
+int launch_tensor(const Context &, const TensorArgs &, uint32_t, cudaStream_t s) {
+    used.insert(s);
+    return 0;
+}
+int launch_ip(const Context &, const IpArgs &, uint32_t, cudaStream_t s) {
+    used.insert(s);
+    return 0;
+}
+int launch_conv(const Context &, const ConvPlans &, const uint64_t *, size_t, size_t, uint64_t *,
+                size_t, size_t, uint32_t, cudaStream_t, bool) {
+    return 0;
+}
+int launch_ntt_lift(const Context &, const uint64_t *, uint64_t *, const LimbMap &, uint32_t,
+                    const LiftEntry *, bool, cudaStream_t) {
+    return 0;
+}
+int launch_ntt_fwd_lazy(const Context &, const uint64_t *, uint64_t *, const LimbMap &, uint32_t,
+                        cudaStream_t) {
+    return 0;
+}
+int launch_ntt_fwd_combine(const Context &, uint64_t *, const LimbMap &, uint32_t,
+                           const NttEpilogue &, cudaStream_t) {
+    return 0;
+}
+int launch_ntt_lift_combine(const Context &, const uint64_t *, uint64_t *, const LimbMap &,
+                            uint32_t, const LiftEntry *, const NttEpilogue &, cudaStream_t) {
+    return 0;
+}
 int launch_ntt_fwd(const Context &, const uint64_t *, uint64_t *, const LimbMap &, uint32_t,
                    cudaStream_t) {
     return 0;
@@ -117,7 +163,7 @@ using namespace catfhe;
 extern "C" int host_uploads(const char *what, int scheme) {
     catfhe_params p{};
     p.scheme = scheme;
-    p.log_n = p.log_n_max = 12;
+    p.log_n = p.log_n_max = strcmp(what, "over") ? 12 : 14;
     p.L = 3;
     p.K = 1;
     p.dnum = 1;
@@ -134,6 +180,27 @@ extern "C" int host_uploads(const char *what, int scheme) {
         const cudaStream_t own = reinterpret_cast<cudaStream_t>(16);  // a non-blocking stream
         if (op_encrypt(c, k, msg.data(), seed, ct.data(), own)) return -1;
         return late;
+    }
+    if (!strcmp(what, "over")) {
+        // (the buffers' addresses are all that is looked at)
+        static uint64_t key;
+        Keys k{};
+        k.ksk[0] = &key;
+        uint64_t *at = reinterpret_cast<uint64_t *>(uintptr_t(1) << 40);
+        const size_t words = 4 * 2 * 3 * c.n;
+        const size_t need = ws_bytes(c, CATFHE_OP_MUL_RELIN, 3, 4);  // the larger
+        auto streams = [&](uint64_t *out, bool fused) -> int {
+            used.clear();
+            if (op_mul_relin(c, k, at, at + words, out, 3, 4, fused, at + 4 * words, need, nullptr,
+                             nullptr, true))
+                return -1;
+            return int(used.size());
+        };
+        // in its own buffer, and in place with the shape of the input: halves
+        if (streams(at + 2 * words, true) != 2 || streams(at, false) != 2) return -1;
+        const int a = streams(at, true), b = streams(at + words, true);
+        const int shifted = streams(at + words / 2, true);
+        return a > b ? (a > shifted ? a : shifted) : (b > shifted ? b : shifted);
     }
     PlanSpec s;
     for (uint32_t i = 0; i < 3; i++) {

@@ -101,3 +101,19 @@ def test_gathered_products_of_two_and_three(scheme, dnum):
         torch.cuda.synchronize()
         for j in range(count):
             assert torch.equal(outs[j], want[j]), (count, j)
+
+
+@pytest.mark.parametrize("count,level", [(4, 3), (5, 9), (3, 4)])
+def test_fused_products_over_their_inputs(count, level):
+    """The result, a limb shorter, in the buffer of either input."""
+    p = W.Preset("route-over", W.CKKS, 14, (50,) * 24, (60,) * 4, 3, log_n_max=16)
+    ctx = api.Context(p)
+    seed = W.seed_for(f"route-over-{count}")
+    keys = ctx.keygen(seed)
+    a, b = _uniform(ctx, seed, count, level), _uniform(ctx, seed, count, level, 100)
+    want = ctx.mul_relin_rescale(keys, a, b)
+    for which in (0, 1):
+        ins = [a.clone(), b.clone()]
+        out = ins[which].view(-1)[:want.numel()].view(want.shape)
+        ctx.mul_relin_rescale(keys, ins[0], ins[1], out=out)
+        assert torch.equal(out, want), which

@@ -1,7 +1,8 @@
 """What the library's host code hands to kernels, on a fake CUDA runtime
 (tests/host_uploads.cpp): constants have arrived before a kernel on the
 caller's stream may read them, and an allocation that failed and is made up
-for leaves no error for the next launch to report."""
+for leaves no error for the next launch to report.  And which streams a product
+that is written over its input runs on."""
 import os
 import shutil
 import subprocess
@@ -62,3 +63,9 @@ def test_constants_arrive_before_the_kernels_that_read_them(program, scheme):
 
 def test_no_memory_for_an_image_leaves_the_integer_form_usable(program):
     assert _run(program, "nomem", W.CKKS) == 0
+
+
+def test_fused_products_over_their_inputs_run_on_one_stream(program):
+    """The result's ciphertexts are a limb shorter than the input's, so that the
+    second half's results lie in the first half's inputs."""
+    assert _run(program, "over", W.CKKS) == 1
