@@ -12,9 +12,9 @@
 //   host_uploads("nomem", scheme)    the last error after a conversion's plans
 //                                    were made without memory for its
 //                                    tensor-core image
-//   host_uploads("over", scheme)     the number of streams on which a fused
-//                                    product of four is written over its input
-//                                    (1 in its own buffer: 2)
+//   host_uploads("over", scheme)     the most streams that a fused product of
+//                                    four runs on when it is written over an
+//                                    input (-1 unless it runs on two elsewhere)
 #include <stdlib.h>
 #include <string.h>
 
